@@ -1104,16 +1104,25 @@ __host__ __device__ constexpr size_t solve_smem_curl32(int N, int T) { return (s
 __host__ __device__ constexpr bool solve_stage_fits(int N, int T) { return solve_smem_staged(N, T) <= 100 * 1024; }
 
 // Banded substitution on one real right-hand side held in shared memory at
-// x[i * st], i < N, by a group of 4 consecutive lanes (column-oriented):
-// lane t keeps the partial sum of row c+1+t (and of row c+5+t for the wall
-// rows, whose lower band reaches 8); once row c is final its value is
-// broadcast and each lane subtracts its row's multiple of it.  The factor is
-// stored by columns (13 N values, see to_columns on the host): [N][4]
-// L(c+1+t, c), [N][4] L(c+5+t, c), [N] 1/U_ii, [N][4] U(c-1-t, c) / U_ii,
-// zeros outside the band, so the four lanes of a chain read one 32-byte run
-// per column.  Each lane needs one factor entry per row; it is loaded kAhead
-// rows ahead into a register queue (the loop is unrolled by kAhead so the
-// queue is indexed statically), which keeps the L2 latency off the recursion.
+// x[i * st], i < N, by a group of 4 consecutive lanes: rows are dealt round
+// robin to the lanes, each lane keeps the partial sum of the one row it owns
+// among the four behind the current column, and once row c is final its owner
+// broadcasts it and every lane subtracts its row's multiple of it (the owner
+// from the next row it takes up).  The factor is stored by columns (13 N
+// values, see to_columns on the host): [N][4] L(c+1+t, c), [N][4] L(c+5+t, c),
+// [N] 1/U_ii, [N][4] U(c-1-t, c) / U_ii, zeros outside the band, so the four
+// lanes of a chain read one 32-byte run per column.  The columns are walked in
+// blocks of four counted so that the nine wall columns start a block: owners
+// and queue slots are then compile-time constants, a lane takes up its next
+// row and stores its finished one once per block, and the chain per row is
+// one broadcast and one FMA (a form that shifted the partial sums along the
+// lanes took eight shuffles per row; the same sums in the same order).  What
+// bounds it is that chain, ~110 cycles per row, on grids of a wave, and the
+// FP64 unit (one FMA per row and eight right-hand sides) on larger ones.
+// Per solve launch, shifting against this form: N=48 63 x 24 modes 59.3 ->
+// 47.1 us, N=128 255 x 128 modes 2.30 -> 1.83 ms, N=32 64 x 31 x 16 modes
+// 596 -> 535 us.  Factor entries are loaded kAhead columns ahead into
+// registers, which keeps the L2 latency off the recursion.
 // All 32 lanes of the warp must call this together (8 right-hand sides per
 // warp).
 __device__ __forceinline__ void band_solve4(const double* __restrict__ L, double* x, int st, int N) {
@@ -1123,71 +1132,96 @@ __device__ __forceinline__ void band_solve4(const double* __restrict__ L, double
   const double* Lw = L + 4 * N;  // L(c+5+t, c)
   const double* Dg = L + 8 * N;  // 1/U_ii
   const double* Uc = L + 9 * N;  // U(c-1-t, c) / U_(c-1-t)
-  // forward: y = L^{-1} b.  Row c+1+t's entry in column c, queued kAhead rows
-  // ahead; on the wall rows (c >= N-9) also row c+5+t's entry in column c,
-  // all nine loaded up front.
-  auto la_of = [&](int c) { return c < N ? __ldg(L + c * 4 + t) : 0.0; };
-  double qa[kAhead], qw[9];
+  double q[kAhead], qd[kAhead / 4];
+  // forward: y = L^{-1} b, stored as y_i / U_ii (the U rows are scaled by
+  // 1/U_ii, so the backward sweep has one FMA per row).  Columns v0 < 0 of the
+  // first round do not exist and are skipped.
+  {
+    const int nw = N - 9;                                    // first wall column
+    const int v0 = nw - (nw + kAhead - 1) / kAhead * kAhead;  // <= 0
+    auto l_of = [&](int c, int j) { return c >= 0 && c < N ? __ldg(L + c * 4 + ((t - j - 1) & 3)) : 0.0; };
+    auto d_of = [&](int i) { return i >= 0 && i < N ? __ldg(Dg + i) : 0.0; };
 #pragma unroll
-  for (int j = 0; j < kAhead; ++j) qa[j] = la_of(j);
+    for (int j = 0; j < kAhead; ++j) q[j] = l_of(v0 + j, j & 3);
 #pragma unroll
-  for (int j = 0; j < 9; ++j) {
-    const int c = N - 9 + j;
-    qw[j] = c >= 0 ? __ldg(Lw + c * 4 + t) : 0.0;
-  }
-  double sa = t < N ? x[t * st] : 0.0;
-  double sb = 4 + t < N ? x[(4 + t) * st] : 0.0;
-  for (int c0 = 0; c0 < N; c0 += kAhead) {
+    for (int b = 0; b < kAhead / 4; ++b) qd[b] = d_of(v0 + 4 * b + t);
+    double s = x[((t + v0) & 3) * st];
+    // the last four rows, whose lower band reaches eight: lane t's one of them,
+    // and its entries in the wall columns more than four to the left
+    const int rw = t ? N - 5 + t : N - 1;
+    double w = x[rw * st], qw[4];
 #pragma unroll
-    for (int j = 0; j < kAhead; ++j) {
-      const int c = c0 + j;  // warp-uniform
-      if (c < N) {
-        const double y = __shfl_sync(full, sa, 0, 4);
-        if (t == 0) x[c * st] = y;
-        const double next_b = (t == 3 && c + 8 < N) ? x[(c + 8) * st] : 0.0;
-        double san = __shfl_down_sync(full, sa, 1, 4);
-        const double sb0 = __shfl_sync(full, sb, 0, 4);
-        double sbn = __shfl_down_sync(full, sb, 1, 4);
-        if (t == 3) {
-          san = sb0;
-          sbn = next_b;
+    for (int i = 0; i < 4; ++i) {
+      const int o = rw - (nw + i) - 5;
+      qw[i] = o >= 0 ? __ldg(Lw + (nw + i) * 4 + o) : 0.0;
+    }
+    for (int c0 = v0; c0 < nw; c0 += kAhead) {
+#pragma unroll
+      for (int b = 0; b < kAhead / 4; ++b) {
+        const int cb = c0 + 4 * b;  // warp-uniform
+        if (cb > -4) {
+          const double next = cb + t >= 0 ? x[(cb + 4 + t) * st] : 0.0;
+          double own = 0.0;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (cb + j >= 0) {
+              const double y = __shfl_sync(full, s, j, 4);
+              if (t == j) {
+                own = s;
+                s = next;
+              }
+              s = fma(-q[4 * b + j], y, s);
+            }
+          }
+          if (cb + t >= 0) x[(cb + t) * st] = own * qd[b];
         }
-        sa = san - qa[j] * y;
-        if (c >= N - 9) {
-          double w = qw[0];
 #pragma unroll
-          for (int q = 1; q < 9; ++q)
-            if (c == N - 9 + q) w = qw[q];
-          sbn -= w * y;
-        }
-        sb = sbn;
-        qa[j] = la_of(c + kAhead);
+        for (int j = 0; j < 4; ++j) q[4 * b + j] = l_of(cb + kAhead + j, j);
+        qd[b] = d_of(cb + kAhead + t);
       }
     }
+    const double next = t == 0 ? x[(N - 5) * st] : 0.0;
+    double own = 0.0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const double y = __shfl_sync(full, s, i & 3, 4);
+      if (t == (i & 3)) {
+        own = s;
+        s = i == 0 ? next : w;
+      }
+      s = fma(-q[i], y, s);
+      if (i < 4) w = fma(-qw[i], y, w);
+      if ((i & 3) == 3) x[(nw + (i & ~3) + t) * st] = own * qd[i >> 2];
+    }
+    if (t == 0) x[(N - 1) * st] = own * qd[2];
   }
-  // y_i / U_ii for all rows at once (off the recursion; the U rows are stored
-  // scaled by 1/U_ii, so the backward sweep has a single FMA per row)
   __syncwarp();
-  for (int i = t; i < N; i += 4) x[i * st] *= __ldg(Dg + i);
-  __syncwarp();
-  // backward: x = U~^{-1} (y / diag U).  Row c-1-t's scaled entry in column c.
-  auto ua_of = [&](int c) { return c >= 0 ? __ldg(Uc + c * 4 + t) : 0.0; };
-  double qu[kAhead];
+  // backward: x = U~^{-1} (y / diag U), counted from the wall
+  {
+    auto u_of = [&](int c, int j) { return c >= 0 ? __ldg(Uc + c * 4 + ((t - j - 1) & 3)) : 0.0; };
 #pragma unroll
-  for (int j = 0; j < kAhead; ++j) qu[j] = ua_of(N - 1 - j);
-  sa = N - 1 - t >= 0 ? x[(N - 1 - t) * st] : 0.0;
-  for (int c0 = N - 1; c0 >= 0; c0 -= kAhead) {
+    for (int j = 0; j < kAhead; ++j) q[j] = u_of(N - 1 - j, j & 3);
+    double s = x[(N - 1 - t) * st];
+    for (int c0 = N - 1; c0 >= 0; c0 -= kAhead) {
 #pragma unroll
-    for (int j = 0; j < kAhead; ++j) {
-      const int c = c0 - j;  // warp-uniform
-      if (c >= 0) {
-        const double xc = __shfl_sync(full, sa, 0, 4);
-        if (t == 0) x[c * st] = xc;
-        const double next_y = (t == 3 && c - 4 >= 0) ? x[(c - 4) * st] : 0.0;
-        double san = __shfl_down_sync(full, sa, 1, 4);
-        if (t == 3) san = next_y;
-        sa = san - qu[j] * xc;
-        qu[j] = ua_of(c - kAhead);
+      for (int b = 0; b < kAhead / 4; ++b) {
+        const int cb = c0 - 4 * b;  // warp-uniform
+        if (cb >= 0) {
+          const double next = cb - 4 - t >= 0 ? x[(cb - 4 - t) * st] : 0.0;
+          double own = 0.0;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const double y = __shfl_sync(full, s, j, 4);
+            if (t == j) {
+              own = s;
+              s = next;
+            }
+            s = fma(-q[4 * b + j], y, s);
+          }
+          if (cb - t >= 0) x[(cb - t) * st] = own;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q[4 * b + j] = u_of(cb - kAhead - j, j);
       }
     }
   }
