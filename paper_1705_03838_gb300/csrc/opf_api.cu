@@ -68,6 +68,7 @@ struct Group {
   opf::DevSetup ds;                  // trajectory 0's setup arrays
   char* parena = nullptr;
   char* sarena = nullptr;
+  void* dft_tab = nullptr;  // digit tables of the FP64 transforms
   size_t pstride = 0, sstride = 0;
   std::vector<double> mesh;  // user radial mesh (empty: the default points)
   // trajectory 0's work buffers (trajectory b: + b * sstride bytes)
@@ -135,7 +136,9 @@ struct Group {
 void group_free(Group* g) {
   if (g->sarena) cudaFree(g->sarena);
   if (g->parena) cudaFree(g->parena);
+  if (g->dft_tab) cudaFree(g->dft_tab);
   g->sarena = g->parena = nullptr;
+  g->dft_tab = nullptr;
 }
 
 struct Layout {
@@ -357,6 +360,12 @@ int group_build(Group* g, int N, int K, int M, int m_p, double alpha, int B, con
     g->ds.spkP = (double*)(P + g->o_spkP);
     g->ds.rH = (double*)(P + g->o_rH);
     g->ds.rP = (double*)(P + g->o_rP);
+  }
+  if (const size_t bytes = opf::dft_table_bytes(K, M)) {
+    if (cudaMalloc(&g->dft_tab, bytes) != cudaSuccess) return fail(OPF_ENOMEM, "cudaMalloc of transform tables failed");
+    std::vector<char> host(bytes);
+    opf::dft_host_tables(K, M, d.inv_grid, host.data(), g->dft_tab, &g->ds.dft);
+    CU(cudaMemcpy(g->dft_tab, host.data(), bytes, cudaMemcpyHostToDevice));
   }
   d.spike = g->spike_default ? 1 : 0;
   d.ps = g->shared_setup ? 0 : (long)g->pstride;

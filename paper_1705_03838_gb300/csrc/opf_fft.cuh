@@ -289,4 +289,15 @@ inline void with_fft_length(int n, F&& f) {
   }
 }
 
+// The same for FP64, where lengths up to 96 are products with digit tables
+// (opf_dft.cu) and only longer ones come here.
+template <class F>
+inline void with_long_fft_length(int n, F&& f) {
+  switch (n) {
+    case 192: f(std::integral_constant<int, 192>{}); break;
+    case 384: f(std::integral_constant<int, 384>{}); break;
+    default: f(std::integral_constant<int, 0>{}); break;
+  }
+}
+
 }  // namespace opf

@@ -57,7 +57,17 @@ bool build_setup(Setup* s, std::string* err);
 // Per-trajectory scalars at the head of each trajectory's setup arrays.
 constexpr int kPrmRe = 0, kPrmDt = 1, kPrmC = 2, kPrmSumWG = 3, kPrmCi = 4, kPrmCu = 5, kPrmCount = 8;
 
+// Digit tables of the FP64 transforms on the tensor cores (opf_dft.cuh): z
+// synthesis, theta synthesis, theta analysis, z analysis, each cosine then
+// sine; null where the transform's length takes the FFT.  Shared by the
+// trajectories of a group.
+struct DftTables {
+  const uint2* m[8] = {};
+  int zshift = 0;  // the z analysis' results count 2^zshift
+};
+
 struct DevSetup {
+  DftTables dft;
   double* prm = nullptr;  // [kPrmCount] Re, dt, c, sum(wq G)
   double* rinv = nullptr;
   double* d1 = nullptr;
@@ -156,6 +166,17 @@ void launch_zanalysis32(const Dims& d, const DevSetup& s, const FftPlan& pz, con
 bool launch_nl_fused32(const Dims& d, const DevSetup& s, const float2* W6, const double2* Nlin, double2* Nout,
                        cudaStream_t st);
 int fused32_cluster(const Dims& d);
+// The FP64 transforms of lengths up to 96 (opf_dft.cu).  Table sizes and
+// contents for a resolution: built on the host (host: dft_table_bytes bytes to
+// be copied to dev) or by a kernel on st from the twiddles of 3K and 3M.
+size_t dft_table_bytes(int K, int M);
+void dft_host_tables(int K, int M, double inv_grid, void* host, void* dev, DftTables* t);
+void dft_device_tables(int K, int M, double inv_grid, const double2* twz, const double2* twth, void* dev,
+                       DftTables* t, cudaStream_t st);
+bool dft_prepare_attrs();
+void launch_dft_zsynth(const Dims& d, const DevSetup& s, const double2* W6, double2* Z6, cudaStream_t st);
+void launch_dft_product(const Dims& d, const DevSetup& s, const double2* Z6, double2* ZN, cudaStream_t st);
+void launch_dft_zanalysis(const Dims& d, const DevSetup& s, const double2* ZN, double2* Nout, cudaStream_t st);
 struct SolveArgs {
   const double2* Uj;
   const double2* Na;

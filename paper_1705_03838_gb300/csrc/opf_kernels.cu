@@ -14,53 +14,14 @@
 #include <algorithm>
 #include <cstdio>
 
+#include "opf_dft.cuh"
 #include "opf_fft.cuh"
 #include "opf_internal.h"
+#include "opf_step.cuh"
 
 namespace opf {
 
 __device__ __forceinline__ int row_lo_d(int i, int N) { return min(max(i - 4, 0), N - 9); }
-
-// Programmatic dependent launch between the kernels of a step: each step
-// kernel lets its successor launch once all of its own blocks have reached
-// the trigger (d.pdl = 1: at the top; 2: before the final store phase), and
-// waits for its predecessor grid to complete -- with its memory visible --
-// before it reads or writes any buffer another kernel of the step touches
-// (grid_dep_wait after a prologue that reads only setup data: twiddles,
-// stencils, factors).  Every step kernel waits, so the ordering is
-// transitive along the stream.  Without a programmatic launch both are
-// no-ops.
-__device__ __forceinline__ void grid_dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_trigger_at(const Dims& d, int where) {
-  if (d.pdl == where) grid_dep_trigger();
-}
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// Launch with the programmatic-serialisation attribute when d.pdl is set
-// (captured into a graph, the edge to the previous kernel becomes a
-// programmatic dependency), plainly otherwise.
-template <typename... KArgs, typename... Args>
-void launch_step_kernel(const Dims& d, void (*kern)(KArgs...), dim3 g, dim3 b, size_t sm, cudaStream_t st,
-                        Args&&... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = g;
-  cfg.blockDim = b;
-  cfg.dynamicSmemBytes = sm;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = d.pdl ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
-}
-
-// Batched launches: trajectory b = blockIdx.z; its buffers sit `stride` bytes
-// after trajectory b-1's (stride 0: shared).  Null stays null.
-template <typename P>
-__device__ __forceinline__ P* bofs(P* p, long stride) {
-  return p ? (P*)((char*)p + (long)blockIdx.z * stride) : p;
-}
 
 // ------------------------------------------------------------------ ABI <-> internal
 // abi: [3][M][nk][N] (u_r, u_theta, u_z); internal: [3][M][N][nk] (u+, u-, u_z).
@@ -183,15 +144,6 @@ void launch_internal_to_abi(const Dims& d, const double2* U, double2* abi, int, 
 // scalings by two, so the results are those of the halved values).  Without
 // SPLIT everything is FP64.
 constexpr int kCurlThreads = 128;
-
-static int device_sms() {
-  static const int sms = [] {
-    int dev = 0, n = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    return n > 0 ? n : 152;
-  }();
-  return sms;
-}
 
 // Blocks per trajectory and the most columns one block takes.
 struct CurlShape {
@@ -483,9 +435,10 @@ void launch_zsynth32(const Dims& d, const DevSetup& s, const FftPlan& pz, const 
 
 void launch_zsynth(const Dims& d, const DevSetup& s, const FftPlan& pz, const double2* W6,
                    double2* Z6, cudaStream_t st) {
+  if (s.dft.m[0]) return launch_dft_zsynth(d, s, W6, Z6, st);
   dim3 g((d.M + d.mcz - 1) / d.mcz, d.N * 6, d.B);
   const size_t sm = zsynth_smem(d, d.mcz, sizeof(double2));
-  with_fft_length(d.nz, [&](auto n) {
+  with_long_fft_length(d.nz, [&](auto n) {
     launch_step_kernel(d, k_zsynth<double2, decltype(n)::value>, g, dim3(transform_threads(g)), sm, st, d, pz,
                        (const double2*)s.tw_z, W6, Z6);
   });
@@ -635,9 +588,10 @@ void launch_product32(const Dims& d, const DevSetup& s, const FftPlan& pth, cons
 
 void launch_product(const Dims& d, const DevSetup& s, const FftPlan& pth, const double2* Z6,
                     double2* ZN, cudaStream_t st) {
+  if (s.dft.m[2]) return launch_dft_product(d, s, Z6, ZN, st);
   dim3 g((d.nz + d.zc - 1) / d.zc, d.N, d.B);
   const size_t sm = product_smem(d, d.zc, sizeof(double2));
-  with_fft_length(d.nth, [&](auto n) {
+  with_long_fft_length(d.nth, [&](auto n) {
     launch_step_kernel(d, k_product<double2, decltype(n)::value>, g, dim3(transform_threads(g)), sm, st, d, pth,
                        (const double2*)s.tw_th, Z6, ZN);
   });
@@ -749,9 +703,10 @@ size_t zanalysis_smem(const Dims& d, int mc, size_t vb) {
 
 void launch_zanalysis(const Dims& d, const DevSetup& s, const FftPlan& pz, const double2* ZN,
                       double2* Nout, cudaStream_t st) {
+  if (s.dft.m[6]) return launch_dft_zanalysis(d, s, ZN, Nout, st);
   dim3 g((d.M + d.mca - 1) / d.mca, d.N, d.B);
   const size_t sm = zanalysis_smem(d, d.mca, sizeof(double2));
-  with_fft_length(d.nz, [&](auto n) {
+  with_long_fft_length(d.nz, [&](auto n) {
     launch_step_kernel(d, k_zanalysis<double2, decltype(n)::value>, g, dim3(transform_threads(g)), sm, st, d, pz,
                        (const double2*)s.tw_z, ZN, (const double2*)nullptr, Nout);
   });
@@ -1762,18 +1717,24 @@ bool prepare_kernel_attrs(const Dims& d) {
       product_smem(d, d.zc, vb) > lim || solve_smem(d.N, solve_tile(d)) > lim)
     return false;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  bool ok = cudaFuncSetAttribute(k_curl<double2, false>, a, optin) == cudaSuccess;
+  bool ok = dft_prepare_attrs();
+  ok = ok && cudaFuncSetAttribute(k_curl<double2, false>, a, optin) == cudaSuccess;
   ok = ok && cudaFuncSetAttribute(k_curl<float2, true>, a, optin) == cudaSuccess;
-  with_fft_length(d.nz, [&](auto n) {
+  with_long_fft_length(d.nz, [&](auto n) {
     constexpr int L = decltype(n)::value;
     ok = ok && cudaFuncSetAttribute(k_zsynth<double2, L>, a, optin) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(k_zanalysis<double2, L>, a, optin) == cudaSuccess;
+  });
+  with_fft_length(d.nz, [&](auto n) {
+    constexpr int L = decltype(n)::value;
     ok = ok && cudaFuncSetAttribute(k_zsynth<float2, L>, a, optin) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(k_zanalysis<float2, L>, a, optin) == cudaSuccess;
   });
+  with_long_fft_length(d.nth, [&](auto n) {
+    ok = ok && cudaFuncSetAttribute(k_product<double2, decltype(n)::value>, a, optin) == cudaSuccess;
+  });
   with_fft_length(d.nth, [&](auto n) {
     constexpr int L = decltype(n)::value;
-    ok = ok && cudaFuncSetAttribute(k_product<double2, L>, a, optin) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(k_product<float2, L>, a, optin) == cudaSuccess;
   });
   ok = ok && cudaFuncSetAttribute(k_solve<16>, a, optin) == cudaSuccess;
@@ -1803,13 +1764,14 @@ bool prepare_nonlinear_attrs(const Dims& d) {
       product_smem(d, d.zc, vb) > lim)
     return false;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  bool ok = cudaFuncSetAttribute(k_curl<double2, false>, a, optin) == cudaSuccess;
-  with_fft_length(d.nz, [&](auto n) {
+  bool ok = dft_prepare_attrs();
+  ok = ok && cudaFuncSetAttribute(k_curl<double2, false>, a, optin) == cudaSuccess;
+  with_long_fft_length(d.nz, [&](auto n) {
     constexpr int L = decltype(n)::value;
     ok = ok && cudaFuncSetAttribute(k_zsynth<double2, L>, a, optin) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(k_zanalysis<double2, L>, a, optin) == cudaSuccess;
   });
-  with_fft_length(d.nth, [&](auto n) {
+  with_long_fft_length(d.nth, [&](auto n) {
     constexpr int L = decltype(n)::value;
     ok = ok && cudaFuncSetAttribute(k_product<double2, L>, a, optin) == cudaSuccess;
   });

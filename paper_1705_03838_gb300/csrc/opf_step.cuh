@@ -1,0 +1,62 @@
+// Helpers shared by the kernels of a time step: programmatic dependent launch
+// and the per-trajectory offsets of a batched launch.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <utility>
+
+#include "opf_internal.h"
+
+namespace opf {
+
+// Programmatic dependent launch between the kernels of a step: each step
+// kernel lets its successor launch once all of its own blocks have reached
+// the trigger (d.pdl = 1: at the top; 2: before the final store phase), and
+// waits for its predecessor grid to complete -- with its memory visible --
+// before it reads or writes any buffer another kernel of the step touches
+// (grid_dep_wait after a prologue that reads only setup data: twiddles,
+// stencils, factors).  Every step kernel waits, so the ordering is
+// transitive along the stream.  Without a programmatic launch both are
+// no-ops.
+__device__ __forceinline__ void grid_dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_trigger_at(const Dims& d, int where) {
+  if (d.pdl == where) grid_dep_trigger();
+}
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch with the programmatic-serialisation attribute when d.pdl is set
+// (captured into a graph, the edge to the previous kernel becomes a
+// programmatic dependency), plainly otherwise.
+template <typename... KArgs, typename... Args>
+void launch_step_kernel(const Dims& d, void (*kern)(KArgs...), dim3 g, dim3 b, size_t sm, cudaStream_t st,
+                        Args&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = g;
+  cfg.blockDim = b;
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = d.pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+
+// Batched launches: trajectory b = blockIdx.z; its buffers sit `stride` bytes
+// after trajectory b-1's (stride 0: shared).  Null stays null.
+template <typename P>
+__device__ __forceinline__ P* bofs(P* p, long stride) {
+  return p ? (P*)((char*)p + (long)blockIdx.z * stride) : p;
+}
+
+inline int device_sms() {
+  static const int sms = [] {
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 0 ? n : 152;
+  }();
+  return sms;
+}
+
+}  // namespace opf
