@@ -62,10 +62,18 @@ bool smooth235(int n) {
 }
 
 // Radial points, 9-point first-derivative stencils for both axis parities
-// (Fornberg's recursion, same points and folding as the handle's setup) and
-// the z / theta twiddle tables, computed on the device into the scratch.
-__global__ void k_noalloc_consts(int N, int nz, int nth, double Re, double* prm, double* d1,
-                                 double* rinv, double2* twz, double2* twth) {
+// (same points and folding as the handle's setup) and the z / theta twiddle
+// tables, computed on the device into the scratch.  One thread per weight:
+// with a_i = prod_(j != i) (x_i - x_j), the weight of node i at node c is
+// a_c / (a_i (x_c - x_i)), that of c itself sum_(j != c) 1 / (x_c - x_j).  (A
+// thread per row running a recursion over the nodes took 101 us at N = 32 on
+// chains of divisions, more than the rest of the call.)
+constexpr int kConstRows = 16;                   // radial rows per block
+constexpr int kConstThreads = kConstRows * 9;    // a thread per (row, node)
+__global__ void __launch_bounds__(kConstThreads)
+    k_noalloc_consts(int N, int nz, int nth, double Re, double* prm, double* d1, double* rinv, double2* twz,
+                     double2* twth) {
+  __shared__ double xs[kConstRows + 16], as[kConstRows][9], ws[kConstRows][9];
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < opf::kPrmCount) prm[t] = t == opf::kPrmRe ? Re : 0.0;
   if (t < nz) {
@@ -78,47 +86,51 @@ __global__ void k_noalloc_consts(int N, int nz, int nth, double Re, double* prm,
     sincospi(2.0 * t / nth, &s, &c);
     twth[t] = double2{c, s};
   }
-  if (t >= N) return;
+  const int n0 = blockIdx.x * kConstRows;
+  if (n0 >= N) return;
+  // extended nodes e0, e0 + 1, .. of the block's rows: e < N is -r_(N-1-e)
+  const int e0 = min(N + n0 - 4, 2 * N - 9);
   auto rad = [&](int j) { return j == N - 1 ? 1.0 : cospi((double)(N - 1 - j) / (2.0 * N - 1.0)); };
-  rinv[t] = 1.0 / rad(t);
-  const int q = N + t;
-  const int e0 = (q + 4 > 2 * N - 1) ? 2 * N - 9 : q - 4;
-  const int lo = min(max(t - 4, 0), N - 9);
-  double x[9], c[9][3];
-  for (int u = 0; u < 9; ++u) {
-    const int e = e0 + u;
-    x[u] = e < N ? -rad(N - 1 - e) : rad(e - N);
+  if (threadIdx.x < kConstRows + 8 && e0 + (int)threadIdx.x < 2 * N) {
+    const int e = e0 + threadIdx.x;
+    xs[threadIdx.x] = e < N ? -rad(N - 1 - e) : rad(e - N);
   }
-  const double z = rad(t);
-  for (int u = 0; u < 9; ++u) c[u][0] = c[u][1] = c[u][2] = 0.0;
-  double c1 = 1.0, c4 = x[0] - z;
-  c[0][0] = 1.0;
-  for (int i = 1; i < 9; ++i) {
-    const int mn = min(i, 2);
-    double c2 = 1.0;
-    const double c5 = c4;
-    c4 = x[i] - z;
-    for (int j = 0; j < i; ++j) {
-      const double c3 = x[i] - x[j];
-      c2 *= c3;
-      if (j == i - 1) {
-        for (int k = mn; k >= 1; --k) c[i][k] = c1 * (k * c[i - 1][k - 1] - c5 * c[i - 1][k]) / c2;
-        c[i][0] = -c1 * c5 * c[i - 1][0] / c2;
-      }
-      for (int k = mn; k >= 1; --k) c[j][k] = (c4 * c[j][k] - k * c[j][k - 1]) / c3;
-      c[j][0] = c4 * c[j][0] / c3;
-    }
-    c1 = c2;
+  __syncthreads();
+  const int row = threadIdx.x / 9, u = threadIdx.x - row * 9, n = n0 + row;
+  const bool in = n < N;
+  const int first = min(N + n - 4, 2 * N - 9);  // this row's first node
+  const double* x = xs + (in ? first - e0 : 0);
+  const int c = in ? N + n - first : 0;
+  if (in) {
+    double a = 1.0;
+    for (int j = 0; j < 9; ++j)
+      if (j != u) a *= x[u] - x[j];
+    as[row][u] = a;
+    if (u == 0) rinv[n] = 1.0 / rad(n);
   }
-  for (int par = 0; par < 2; ++par)
-    for (int u = 0; u < 9; ++u) d1[(par * N + t) * 9 + u] = 0.0;
-  for (int u = 0; u < 9; ++u) {
-    const int e = e0 + u;
-    const bool ghost = e < N;
-    const int slot = (ghost ? N - 1 - e : e - N) - lo;
-    d1[(0 * N + t) * 9 + slot] += c[u][1];
-    d1[(1 * N + t) * 9 + slot] += ghost ? -c[u][1] : c[u][1];
+  __syncthreads();
+  if (in) ws[row][u] = u == c ? 0.0 : as[row][c] / (as[row][u] * (x[c] - x[u]));
+  __syncthreads();
+  if (in && u == c) {  // the derivative of a constant is zero: sum the inverse distances
+    double s = 0.0;
+    for (int j = 0; j < 9; ++j)
+      if (j != c) s += 1.0 / (x[c] - x[j]);
+    ws[row][c] = s;
   }
+  __syncthreads();
+  if (!in) return;
+  // slot u of the row's columns lo .. lo + 8: the real node there, plus the
+  // ghost that folds onto it
+  const int lo = min(max(n - 4, 0), N - 9), col = lo + u;
+  double even = 0.0, odd = 0.0;
+  const int real = N + col - first, ghost = N - 1 - col - first;
+  if (real >= 0 && real < 9) even = odd = ws[row][real];
+  if (ghost >= 0 && ghost < 9 && ghost + first < N) {
+    even += ws[row][ghost];
+    odd -= ws[row][ghost];
+  }
+  d1[(0 * N + n) * 9 + u] = even;
+  d1[(1 * N + n) * 9 + u] = odd;
 }
 
 int fail(int code, const std::string& m) {
@@ -219,11 +231,16 @@ extern "C" int opf_nonlinear_noalloc(int N, int K, int M, int m_p, double alpha,
   double2* ZN = (double2*)(base + o_ZN);
   double2* Nn = (double2*)(base + o_N);
 
-  const int nc = std::max(N, std::max(d.nz, d.nth));
-  k_noalloc_consts<<<(nc + 127) / 128, 128, 0, st>>>(N, d.nz, d.nth, Re, s.prm, s.d1, s.rinv, s.tw_z,
-                                                      s.tw_th);
+  const int nb = std::max((N + kConstRows - 1) / kConstRows,
+                          (std::max(d.nz, d.nth) + kConstThreads - 1) / kConstThreads);
+  k_noalloc_consts<<<nb, kConstThreads, 0, st>>>(N, d.nz, d.nth, Re, s.prm, s.d1, s.rinv, s.tw_z, s.tw_th);
   opf::launch_abi_to_internal(d, (const double2*)d_state, U, st);
   opf::launch_curl(d, s, U, W6, st);
+  // the transforms' tables: behind the other regions, or over U, which the
+  // curl has read, where the scratch ends before (a working set that fills it
+  // has a U of a megabyte and more)
+  unsigned char* tab = need + opf::dft_table_bytes(K, M) <= kNoallocScratchBytes ? base + need : base + o_U;
+  opf::dft_device_tables(K, M, d.inv_grid, s.tw_z, s.tw_th, tab, &s.dft, st);
   opf::launch_zsynth(d, s, pz, W6, Z6, st);
   opf::launch_product(d, s, pth, Z6, ZN, st);
   opf::launch_zanalysis(d, s, pz, ZN, Nn, st);
