@@ -202,21 +202,28 @@ void launch_nan_check(const double* x, long n, int* flag, cudaStream_t st);
 // C[m][n] = sum_k A[m][k] B[n][k] for m < M, n < N; A [Mp][Kp] and B [Np][Kp]
 // row-major BF16, zero padded (Mp, Np multiples of 128, Kp of 64), 16-byte
 // aligned.  Epilogue per (m, n): x = C + bias[n]; pre_f32 = x; x = gelu(x)
-// if gelu; out_f32 = x (+= x if accumulate); out_bf16 = bf16(x); outputs
-// have row stride ldo.  d_err (device int) is set on a timed-out wait.
-// work (device, work_floats floats; may be null) lets plain FP32 outputs (no
-// bias, GELU or BF16 copy) split K across CTAs; the partial sums are added in
-// a fixed order, so results do not depend on scheduling.
+// if gelu; out_f32 = x; col: bf16(x) into the im2col rows of a width-3
+// convolution of C channels over rows of L points (row stride ldc; zeros past
+// the ends); FP32 outputs have row stride ldo.  d_err (device int) is set on
+// a timed-out wait.
+// splits (may be null): lets K be split over *splits ranges whose raw sums go
+// to work (work_floats floats) as [split][M][N] and no epilogue is applied
+// when *splits > 1; added in split order, results do not depend on scheduling.
 struct TcEpilogue {
   const float* bias;
   int gelu;
   float* pre_f32;
   float* out_f32;
-  int accumulate;
-  void* out_bf16;
   long ldo;
+  void* col;
+  int C, L;
+  long ldc;
 };
 int tc_gemm(const void* A, const void* B, int M, int N, int Mp, int Np, int Kp, const TcEpilogue& e, int* d_err,
-            cudaStream_t st, float* work = nullptr, long work_floats = 0);
+            cudaStream_t st, float* work = nullptr, long work_floats = 0, int* splits = nullptr);
+// out[m][n] (row stride ldo) = sum over k < k_rows of A[k][m] B[k][n], row-major
+// BF16 with row strides lda, ldb (multiples of 8), 16-byte aligned.
+int tc_gemm_columns(const void* A, long lda, const void* B, long ldb, int M, int N, int k_rows, float* out, long ldo,
+                    int* d_err, cudaStream_t st, float* work, long work_floats);
 
 }  // namespace opf

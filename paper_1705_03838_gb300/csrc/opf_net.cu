@@ -9,10 +9,11 @@
 //
 // conv3 is a width-3 convolution along l with zero padding.  Every
 // convolution and its two backward products is one GEMM on BF16 operands
-// with FP32 accumulation on the tcgen05 tensor cores (opf_tcgemm.cu), which
-// take row-major K-contiguous operands zero padded to 128-row / 64-column
-// multiples; small kernels here lay the operands out that way (im2col rows
-// x[b][l + j - 1][c] at column j*C + c, transposes, padded weights).  Master
+// with FP32 accumulation on the tcgen05 tensor cores (opf_tcgemm.cu).  The
+// products over channels take im2col rows (x[b][l + j - 1][c] at column
+// j*C + c, zero padded), which the producer of the activations -- the first
+// kernel, or the previous GEMM's epilogue -- writes directly; the weight
+// gradients take the same rows by columns, so nothing is transposed.  Master
 // weights and Adam moments are FP32.
 #include <cmath>
 #include <cstdint>
@@ -40,64 +41,37 @@ __device__ __forceinline__ float gelu_grad(float x) {
 long pad128(long v) { return (v + 127) / 128 * 128; }
 long pad64(long v) { return (v + 63) / 64 * 64; }
 
-// im2col rows: out[m][j*C + c] = x[b][l + s(j-1)][c] (m = b*L + l; s = +1, or
-// -1 for the transposed convolution), zero outside 0 <= l' < L, m >= M or
-// k >= 3C; out is [Mp][Kp]
-__global__ void k_im2col(const bf16* __restrict__ x, int L, int C, int M, int rev, bf16* __restrict__ out, int Mp,
-                         int Kp) {
-  const long n = (long)Mp * Kp;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const int m = (int)(i / Kp), k = (int)(i - (long)m * Kp);
-    bf16 v = __float2bfloat16(0.f);
-    if (m < M && k < 3 * C) {
-      const int j = k / C, c = k - j * C, b = m / L, l = m - b * L;
-      const int ls = l + (rev ? 1 - j : j - 1);
-      if (ls >= 0 && ls < L) v = x[((long)b * L + ls) * C + c];
-    }
-    out[i] = v;
-  }
-}
-
-// The same rows as k_im2col, 8 channels (16 bytes) per thread, one output
-// row per grid row (no integer division by the row length): a row of out is
-// three shifted rows of x, each C channels, then zeros to Kp.  Needs C and Kp
-// multiples of 8 and 16-byte aligned bases (see im2col()).
-__global__ void k_im2col8(const bf16* __restrict__ x, int L, int C, int M, int rev, bf16* __restrict__ out, int Kp) {
-  const int m = blockIdx.y, k8 = (blockIdx.x * blockDim.x + threadIdx.x) * 8;
-  if (k8 >= Kp) return;
-  uint4 v = make_uint4(0u, 0u, 0u, 0u);
-  if (m < M && k8 < 3 * C) {
-    const int j = k8 / C, c = k8 - j * C, b = m / L, l = m - b * L;
-    const int ls = l + (rev ? 1 - j : j - 1);
-    if (ls >= 0 && ls < L) v = *(const uint4*)(x + ((long)b * L + ls) * C + c);
-  }
-  *(uint4*)(out + (long)m * Kp + k8) = v;
-}
-
 int gs(long n);
 
-void im2col(cudaStream_t st, const bf16* x, int L, int C, int M, int rev, bf16* out, int Mp, int Kp) {
-  if (C % 8 == 0 && Kp % 8 == 0 && !((uintptr_t)x & 15) && !((uintptr_t)out & 15)) {
-    const int kv = Kp / 8;
-    k_im2col8<<<dim3((unsigned)((kv + 127) / 128), (unsigned)Mp), 128, 0, st>>>(x, L, C, M, rev, out, Kp);
-  } else {
-    k_im2col<<<gs((long)Mp * Kp), 256, 0, st>>>(x, L, C, M, rev, out, Mp, Kp);
-  }
+// V channels at c of one row's BF16 values into the im2col rows of a width-3
+// convolution: row m's block j holds x[l + s (j - 1)], s = +1 (forward) or -1
+// (its transpose), zeros past the ends.  col: row m, channel c of block 0.
+template <typename T>
+__device__ __forceinline__ void put_cols(T v, T zero, bf16* col, long ldc, int C, int l, int L, bool rev) {
+  const int up = rev ? 2 : 0, down = 2 - up;  // the block in row l + 1 and in row l - 1
+  *(T*)(col + C) = v;
+  if (l + 1 < L) *(T*)(col + ldc + up * C) = v;
+  else *(T*)(col + down * C) = zero;
+  if (l > 0) *(T*)(col - ldc + down * C) = v;
+  else *(T*)(col + up * C) = zero;
 }
 
-// out[c][r] = src[r][c] (r < R, c < C, row stride lds), zero padded; out is [Cp][Rp]
-__global__ void k_transpose(const bf16* __restrict__ src, int R, int C, long lds, bf16* __restrict__ out, int Rp,
-                            int Cp) {
-  __shared__ bf16 tile[32][33];
-  const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
-    const int r = r0 + q, c = c0 + threadIdx.x;
-    tile[q][threadIdx.x] = (r < R && c < C) ? src[(long)r * lds + c] : __float2bfloat16(0.f);
-  }
-  __syncthreads();
-  for (int q = threadIdx.y; q < 32; q += blockDim.y) {
-    const int c = c0 + q, r = r0 + threadIdx.x;
-    if (c < Cp && r < Rp) out[(long)c * Rp + r] = tile[threadIdx.x][q];
+// x (FP32 [BL][C]) as BF16 im2col rows; VEC: eight channels per thread (C a
+// multiple of 8, x 16-byte aligned).
+template <bool VEC>
+__global__ void k_x_cols(const float* __restrict__ x, int L, int C, bf16* __restrict__ col, long ldc) {
+  const long m = blockIdx.x;
+  const int l = (int)(m % L), c = (blockIdx.y * blockDim.x + threadIdx.x) * (VEC ? 8 : 1);
+  if (c >= C) return;
+  const float* s = x + m * C + c;
+  bf16* d = col + m * ldc + c;
+  if constexpr (VEC) {
+    const float4 a = *(const float4*)s, b = *(const float4*)(s + 4);
+    const __nv_bfloat162 p[4] = {__floats2bfloat162_rn(a.x, a.y), __floats2bfloat162_rn(a.z, a.w),
+                                 __floats2bfloat162_rn(b.x, b.y), __floats2bfloat162_rn(b.z, b.w)};
+    put_cols(*(const uint4*)p, make_uint4(0u, 0u, 0u, 0u), d, ldc, C, l, L, false);
+  } else {
+    put_cols(__float2bfloat16(*s), __float2bfloat16(0.f), d, ldc, C, l, L, false);
   }
 }
 
@@ -130,103 +104,211 @@ __global__ void k_to_bf16(const float* __restrict__ x, bf16* __restrict__ y, lon
     y[i] = __float2bfloat16(x[i]);
 }
 
-// dZ = dY * gelu'(pre), stored as bf16 (operand of the next GEMMs) and f32
-__global__ void k_gelu_back(const float* __restrict__ dy, const float* __restrict__ pre, bf16* __restrict__ dz,
-                            float* __restrict__ dzf, long n) {
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const float v = dy[i] * gelu_grad(pre[i]);
-    dz[i] = __float2bfloat16(v);
-    if (dzf) dzf[i] = v;
+// mean over l of h2 (the middle block of its im2col rows) and the head:
+// pooled[b][c], z[b][o] = sum_c Wh[o][c] pooled[b][c] + bh[o]; one block per
+// b, two thirds of a channel's rows in flight at a time
+constexpr int kPoolThreads = 512;
+__global__ void __launch_bounds__(kPoolThreads) k_pool_head(const bf16* __restrict__ col, long ldc, int L, int C,
+                                                            int O, const float* __restrict__ Wh,
+                                                            const float* __restrict__ bh, float* pooled,
+                                                            float* __restrict__ z) {
+  const long b = blockIdx.x;
+  float* sp = pooled + b * C;
+  const bf16* h = col + b * L * ldc + C;
+  for (int c = threadIdx.x; c < C; c += blockDim.x) {
+    float s = 0.f;
+    for (int l0 = 0; l0 < L; l0 += 32) {
+      bf16 v[32];
+#pragma unroll
+      for (int q = 0; q < 32; ++q) v[q] = l0 + q < L ? h[(l0 + q) * ldc + c] : __float2bfloat16(0.f);
+#pragma unroll
+      for (int q = 0; q < 32; ++q) s += __bfloat162float(v[q]);
+    }
+    sp[c] = s / L;
   }
-}
-
-// column sums (bias gradients): out[n] = sum_m x[m][n]; block (32 columns x
-// 32 row groups), partial sums reduced in shared memory
-__global__ void __launch_bounds__(1024) k_colsum(const float* __restrict__ x, int M, int N, float* __restrict__ out) {
-  __shared__ float part[32][33];
-  const int n = blockIdx.x * 32 + threadIdx.x;
-  float s = 0.f;
-  if (n < N)
-    for (int m = threadIdx.y; m < M; m += 32) s += x[(long)m * N + n];
-  part[threadIdx.y][threadIdx.x] = s;
   __syncthreads();
-  if (threadIdx.y == 0 && n < N) {
-    float t = 0.f;
-    for (int q = 0; q < 32; ++q) t += part[q][threadIdx.x];
-    out[n] = t;
+  for (int o = threadIdx.x >> 5; o < O; o += blockDim.x >> 5) {
+    float s = 0.f;
+#pragma unroll 8
+    for (int c = threadIdx.x & 31; c < C; c += 32) s += Wh[(long)o * C + c] * sp[c];
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    if ((threadIdx.x & 31) == 0) z[b * O + o] = bh[o] + s;
   }
 }
 
-// mean over l of h2 (bf16 -> f32): pooled[b][c]
-__global__ void k_pool(const bf16* __restrict__ h, int B, int L, int C, float* __restrict__ pooled) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= B * C) return;
-  const int b = i / C, c = i % C;
-  float s = 0.f;
-  for (int l = 0; l < L; ++l) s += __bfloat162float(h[((long)b * L + l) * C + c]);
-  pooled[i] = s / L;
+// Gradient tiles: a block takes 32 rows x 64 columns, thread (tx, ty) columns
+// 2 tx, 2 tx + 1 of rows ty, ty + 8, ..; column sums (bias gradients) of the
+// block go to csum[block row][C], added up by k_bias_sum in a fixed order.
+constexpr int kGradRows = 32;
+
+__device__ __forceinline__ void grad_column_sums(float s0, float s1, int c, int C, float* csum) {
+  __shared__ float2 part[8][32];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  part[ty][tx] = make_float2(s0, s1);
+  __syncthreads();
+  if (ty == 0) {
+    for (int q = 1; q < 8; ++q) {
+      s0 += part[q][tx].x;
+      s1 += part[q][tx].y;
+    }
+    if (c < C) csum[(long)blockIdx.y * C + c] = s0;
+    if (c + 1 < C) csum[(long)blockIdx.y * C + c + 1] = s1;
+  }
 }
 
-// head: z[b][o] = sum_c Wh[o][c] pooled[b][c] + bh[o]; loss terms and gradients
-__global__ void k_head(const float* __restrict__ pooled, const float* __restrict__ Wh, const float* __restrict__ bh,
-                       int B, int C, int O, float* __restrict__ z) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= B * O) return;
-  const int b = i / O, o = i % O;
-  float s = bh[o];
-  for (int c = 0; c < C; ++c) s += Wh[o * C + c] * pooled[b * C + c];
-  z[i] = s;
+// one gradient pair as BF16: rows dz (ldz apart, an even number) and, if
+// dzcol, the im2col rows of the transposed convolution
+__device__ __forceinline__ void put_grad(float v0, float v1, long m, int c, int C, int L, bf16* dz, long ldz,
+                                         bf16* dzcol, long ldc) {
+  const __nv_bfloat162 p = __floats2bfloat162_rn(v0, v1);
+  const int l = (int)(m % L);
+  if (c + 1 < C) {
+    *(__nv_bfloat162*)(dz + m * ldz + c) = p;
+  } else {
+    dz[m * ldz + c] = p.x;
+  }
+  if (!dzcol) return;
+  bf16* d = dzcol + m * ldc + c;
+  if (!(C & 1)) {
+    put_cols(*reinterpret_cast<const unsigned*>(&p), 0u, d, ldc, C, l, L, true);
+  } else {
+    put_cols(p.x, __float2bfloat16(0.f), d, ldc, C, l, L, true);
+    if (c + 1 < C) put_cols(p.y, __float2bfloat16(0.f), d + 1, ldc, C, l, L, true);
+  }
 }
 
-// residuals r = pred - target and their squared sums (two partial sums)
-__global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ tgt, long n, float scale,
-                      float* __restrict__ grad, double* __restrict__ sum) {
-  __shared__ double sh[256];
+// dL/dy = 2 scale (y - t) of the output layer, and sum (y - t)^2
+__global__ void __launch_bounds__(256) k_out_grad(const float* __restrict__ y, const float* __restrict__ t, int BL,
+                                                  int L, int C, float scale, bf16* __restrict__ dz, long ldz,
+                                                  bf16* __restrict__ dzcol, long ldc, float* __restrict__ csum,
+                                                  double* __restrict__ sum) {
+  const int c = blockIdx.x * 64 + 2 * (threadIdx.x & 31);
   double acc = 0.0;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const float r = pred[i] - tgt[i];
-    acc += (double)r * r;
-    grad[i] = 2.f * scale * r;
+  float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+  for (int q = 0; q < kGradRows / 8; ++q) {
+    const long m = (long)blockIdx.y * kGradRows + q * 8 + (threadIdx.x >> 5);
+    if (m >= BL || c >= C) continue;
+    const long i = m * C + c;
+    const float r0 = y[i] - t[i], r1 = c + 1 < C ? y[i + 1] - t[i + 1] : 0.f;
+    acc += (double)r0 * r0;
+    acc += (double)r1 * r1;
+    const float g0 = 2.f * scale * r0, g1 = 2.f * scale * r1;
+    s0 += g0;
+    s1 += g1;
+    put_grad(g0, g1, m, c, C, L, dz, ldz, dzcol, ldc);
   }
-  sh[threadIdx.x] = acc;
+  grad_column_sums(s0, s1, c, C, csum);
+  __shared__ double sh[8];
+  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
   __syncthreads();
-  for (int h = 128; h > 0; h >>= 1) {
-    if (threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) acc += sh[q];
+    atomicAdd(sum, acc);
+  }
+}
+
+// dZ = dH gelu'(pre) of a hidden layer; dH = sum over splits of dh [split][BL][C]
+// plus, under the head, the pooled mean's gradient dpool[b][c]
+__global__ void __launch_bounds__(256) k_hidden_grad(const float* __restrict__ dh, int nsplit,
+                                                     const float* __restrict__ pre, int BL, int L, int C,
+                                                     const float* __restrict__ dpool, bf16* __restrict__ dz, long ldz,
+                                                     bf16* __restrict__ dzcol, long ldc, float* __restrict__ csum) {
+  const int c = blockIdx.x * 64 + 2 * (threadIdx.x & 31);
+  const long total = (long)BL * C;
+  float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+  for (int q = 0; q < kGradRows / 8; ++q) {
+    const long m = (long)blockIdx.y * kGradRows + q * 8 + (threadIdx.x >> 5);
+    if (m >= BL || c >= C) continue;
+    const long i = m * C + c;
+    float v[2] = {0.f, 0.f};
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (c + u >= C) continue;
+      float h = 0.f;
+      for (int k = 0; k < nsplit; ++k) h += dh[k * total + i + u];
+      if (dpool) h += dpool[m / L * C + c + u];
+      v[u] = h * gelu_grad(pre[i + u]);
+    }
+    s0 += v[0];
+    s1 += v[1];
+    put_grad(v[0], v[1], m, c, C, L, dz, ldz, dzcol, ldc);
+  }
+  grad_column_sums(s0, s1, c, C, csum);
+}
+
+// head, dz = 2 zscale (z - tz).  Grid y < O: dWh[o][c] = sum_b dz[b][o]
+// pooled[b][c], dbh[o] and sum (z - tz)^2; then one grid row per sample:
+// dpool[b][c] = sum_o dz[b][o] Wh[o][c] / L.
+__global__ void __launch_bounds__(128) k_head_grad(const float* __restrict__ z, const float* __restrict__ tz,
+                                                   float zscale, const float* __restrict__ pooled,
+                                                   const float* __restrict__ Wh, int B, int L, int C, int O,
+                                                   float* __restrict__ dWh, float* __restrict__ dbh,
+                                                   float* __restrict__ dpool, double* __restrict__ sum) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x, o = blockIdx.y;
+  if (o >= O) {
+    const long b = o - O;
+    if (c >= C) return;
+    float p = 0.f;
+#pragma unroll 4
+    for (int q = 0; q < O; ++q) p += 2.f * zscale * (z[b * O + q] - tz[b * O + q]) * Wh[(long)q * C + c];
+    dpool[b * C + c] = p / L;
+    return;
+  }
+  __shared__ float dz[128];
+  float s = 0.f;
+  for (int b0 = 0; b0 < B; b0 += 128) {
+    const int nb = min(128, B - b0), b = b0 + threadIdx.x;
     __syncthreads();
+    if ((int)threadIdx.x < nb) dz[threadIdx.x] = 2.f * zscale * (z[(long)b * O + o] - tz[(long)b * O + o]);
+    __syncthreads();
+    if (c < C) {
+#pragma unroll 16
+      for (int q = 0; q < nb; ++q) s += dz[q] * pooled[(long)(b0 + q) * C + c];
+    }
   }
-  if (threadIdx.x == 0) atomicAdd(sum, sh[0]);
+  if (c < C) dWh[(long)o * C + c] = s;
+  if (blockIdx.x == 0 && threadIdx.x < 32) {  // one warp per output
+    double acc = 0.0;
+    float t = 0.f;
+    for (int b = threadIdx.x; b < B; b += 32) {
+      const float r = z[(long)b * O + o] - tz[(long)b * O + o];
+      acc += (double)r * r;
+      t += 2.f * zscale * r;
+    }
+    for (int d = 16; d > 0; d >>= 1) {
+      acc += __shfl_xor_sync(0xffffffffu, acc, d);
+      t += __shfl_xor_sync(0xffffffffu, t, d);
+    }
+    if (threadIdx.x == 0) {
+      dbh[o] = t;
+      atomicAdd(sum, acc);
+    }
+  }
 }
 
-// head backward: dWh[o][c] = sum_b dz[b][o] pooled[b][c]; dbh; dpooled[b][c]
-__global__ void k_head_back(const float* __restrict__ dz, const float* __restrict__ pooled,
-                            const float* __restrict__ Wh, int B, int C, int O, float* __restrict__ dWh,
-                            float* __restrict__ dbh, float* __restrict__ dpooled) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < O * C) {
-    const int o = i / C, c = i % C;
-    float s = 0.f;
-    for (int b = 0; b < B; ++b) s += dz[b * O + o] * pooled[b * C + c];
-    dWh[i] = s;
+// bias gradients of the three layers (grid y): db[c] = sum of the tiles' sums;
+// block of 32 channels x 8 groups of tiles
+struct BiasSums {
+  const float* csum[3];
+  float* db[3];
+  int C[3];
+};
+__global__ void __launch_bounds__(256) k_bias_sum(BiasSums a, int rows) {
+  __shared__ float part[8][32];
+  const int q = blockIdx.y, tx = threadIdx.x & 31, ty = threadIdx.x >> 5, c = blockIdx.x * 32 + tx, C = a.C[q];
+  float s = 0.f;
+  if (c < C) {
+#pragma unroll 4
+    for (int r = ty; r < rows; r += 8) s += a.csum[q][(long)r * C + c];
   }
-  if (i < O) {
-    float s = 0.f;
-    for (int b = 0; b < B; ++b) s += dz[b * O + i];
-    dbh[i] = s;
-  }
-  if (i < B * C) {
-    const int b = i / C, c = i % C;
-    float s = 0.f;
-    for (int o = 0; o < O; ++o) s += dz[b * O + o] * Wh[o * C + c];
-    dpooled[i] = s;
-  }
-}
-
-// add the pooled-mean gradient to dh2 (broadcast over l, divided by L)
-__global__ void k_unpool_add(const float* __restrict__ dpooled, int B, int L, int C, float* __restrict__ dh) {
-  const long n = (long)B * L * C;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const long b = i / ((long)L * C), c = i % C;
-    dh[i] += dpooled[b * C + c] / L;
+  part[ty][tx] = s;
+  __syncthreads();
+  if (ty == 0 && c < C) {
+    for (int u = 1; u < 8; ++u) s += part[u][tx];
+    a.db[q][c] = s;
   }
 }
 
@@ -254,19 +336,17 @@ struct opf_net {
   bf16* Pb = nullptr;  // bf16 copies of the weight matrices (same offsets)
   long step = 0;
   int Bcap = 0;
-  // activations / workspace for batch capacity Bcap
-  bf16 *xb = nullptr, *h1 = nullptr, *h2 = nullptr, *dz = nullptr, *dz2 = nullptr;
-  // GEMM operands (row-major, K contiguous, zero padded): im2col rows of the
-  // three layer inputs, their transposes, transposed / shifted output
-  // gradients, padded and shifted weights
-  bf16 *col[3] = {nullptr, nullptr, nullptr}, *colT = nullptr, *dzT = nullptr, *dzcol = nullptr;
+  // activations / workspace for batch capacity Bcap: im2col rows of the three
+  // layer inputs, an output gradient by rows (ldz apart), im2col rows of the
+  // transposed convolution for layers 2 and 3, padded and shifted weights
+  bf16 *col[3] = {nullptr, nullptr, nullptr}, *dz = nullptr, *dzcol[2] = {nullptr, nullptr};
   bf16 *wp[3] = {nullptr, nullptr, nullptr}, *ws[2] = {nullptr, nullptr};
-  int* err = nullptr;
   float* gwork = nullptr;  // split-K partial sums of the weight-gradient GEMMs
   long gwork_floats = 0;
-  float *pre1 = nullptr, *pre2 = nullptr, *y = nullptr, *dy = nullptr, *dh = nullptr;
-  float *pooled = nullptr, *z = nullptr, *dzh = nullptr, *dpooled = nullptr;
-  double* sums = nullptr;
+  float *pre1 = nullptr, *pre2 = nullptr, *y = nullptr, *dh = nullptr;
+  float *pooled = nullptr, *dpool = nullptr, *z = nullptr, *csum = nullptr;
+  double* sums = nullptr;  // the two loss sums, then the GEMMs' error flag
+  double* read = nullptr;  // pinned host copy of sums and flag
   int* aug_idx = nullptr;    // minibatch rows of opf_net_gather_augment (device)
   float* aug_ang = nullptr;  // their shift / rotation phases
   int aug_cap = 0;
@@ -284,38 +364,39 @@ int nfail(const std::string& m) {
     if (e_ != cudaSuccess) return nfail(std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
+long net_ldz(const opf_net* n) { return pad64(std::max(n->H, n->Cin)); }
+
 int net_reserve(opf_net* n, int B) {
   if (B <= n->Bcap) return OPF_OK;
-  auto fr = [](void* p) {
-    if (p) cudaFree(p);
-  };
-  fr(n->xb), fr(n->h1), fr(n->h2), fr(n->dz), fr(n->dz2), fr(n->pre1), fr(n->pre2), fr(n->y);
-  fr(n->dy), fr(n->dh), fr(n->pooled), fr(n->z), fr(n->dzh), fr(n->dpooled), fr(n->sums);
-  for (int i = 0; i < 3; ++i) fr(n->col[i]);
-  fr(n->colT), fr(n->dzT), fr(n->dzcol);
+  n->Bcap = 0;
+  for (void** p : {(void**)&n->col[0], (void**)&n->col[1], (void**)&n->col[2], (void**)&n->dz, (void**)&n->dzcol[0],
+                   (void**)&n->dzcol[1],
+                   (void**)&n->pre1, (void**)&n->pre2, (void**)&n->y, (void**)&n->dh, (void**)&n->pooled,
+                   (void**)&n->dpool, (void**)&n->z, (void**)&n->csum}) {
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+  }
   const long BL = (long)B * n->L, W = std::max(n->H, n->Cin);
-  const long BLp = pad128(BL), K1 = pad64(3L * n->Cin), K2 = pad64(3L * n->H);
-  NCU(cudaMalloc(&n->col[0], BLp * K1 * sizeof(bf16)));
-  NCU(cudaMalloc(&n->col[1], BLp * K2 * sizeof(bf16)));
-  NCU(cudaMalloc(&n->col[2], BLp * K2 * sizeof(bf16)));
-  NCU(cudaMalloc(&n->colT, pad128(3L * W) * BLp * sizeof(bf16)));
-  NCU(cudaMalloc(&n->dzT, pad128(W) * BLp * sizeof(bf16)));
-  NCU(cudaMalloc(&n->dzcol, BLp * pad64(3L * W) * sizeof(bf16)));
-  NCU(cudaMalloc(&n->xb, BL * n->Cin * sizeof(bf16)));
-  NCU(cudaMalloc(&n->h1, BL * n->H * sizeof(bf16)));
-  NCU(cudaMalloc(&n->h2, BL * n->H * sizeof(bf16)));
-  NCU(cudaMalloc(&n->dz, BL * W * sizeof(bf16)));
-  NCU(cudaMalloc(&n->dz2, BL * W * sizeof(bf16)));
+  const long BLp = pad128(BL), K1 = pad64(3L * n->Cin), K2 = pad64(3L * n->H), ldz = net_ldz(n);
+  // the BF16 rows' padding is zero and stays so
+  auto zeroed = [&](bf16** p, long count) {
+    NCU(cudaMalloc(p, count * sizeof(bf16)));
+    NCU(cudaMemsetAsync(*p, 0, count * sizeof(bf16), n->st));
+    return (int)OPF_OK;
+  };
+  int rc;
+  if ((rc = zeroed(&n->col[0], BLp * K1)) || (rc = zeroed(&n->col[1], BLp * K2)) ||
+      (rc = zeroed(&n->col[2], BLp * K2)) || (rc = zeroed(&n->dz, BLp * ldz)) ||
+      (rc = zeroed(&n->dzcol[0], BLp * K2)) || (rc = zeroed(&n->dzcol[1], BLp * K1)))
+    return rc;
   NCU(cudaMalloc(&n->pre1, BL * n->H * sizeof(float)));
   NCU(cudaMalloc(&n->pre2, BL * n->H * sizeof(float)));
   NCU(cudaMalloc(&n->y, BL * n->Cin * sizeof(float)));
-  NCU(cudaMalloc(&n->dy, BL * W * sizeof(float)));
   NCU(cudaMalloc(&n->dh, BL * W * sizeof(float)));
   NCU(cudaMalloc(&n->pooled, (long)B * n->H * sizeof(float)));
+  NCU(cudaMalloc(&n->dpool, (long)B * n->H * sizeof(float)));
   NCU(cudaMalloc(&n->z, (long)B * n->O * sizeof(float)));
-  NCU(cudaMalloc(&n->dzh, (long)B * n->O * sizeof(float)));
-  NCU(cudaMalloc(&n->dpooled, (long)B * n->H * sizeof(float)));
-  NCU(cudaMalloc(&n->sums, 2 * sizeof(double)));
+  NCU(cudaMalloc(&n->csum, (BL + kGradRows - 1) / kGradRows * (n->Cin + 2L * n->H) * sizeof(float)));
   n->Bcap = B;
   return OPF_OK;
 }
@@ -324,16 +405,26 @@ float* Pf(opf_net* n, int i) { return n->P + n->off[i]; }
 float* Gf(opf_net* n, int i) { return n->G + n->off[i]; }
 bf16* Pbf(opf_net* n, int i) { return n->Pb + n->off[i]; }
 
+int* net_err(opf_net* n) { return (int*)(n->sums + 2); }
+
 // C = A B^T on padded operands with the given epilogue
-int gemm(opf_net* n, const bf16* A, const bf16* Bm, int M, int N, int Kp, const opf::TcEpilogue& e) {
-  return opf::tc_gemm(A, Bm, M, N, (int)pad128(M), (int)pad128(N), Kp, e, n->err, n->st, n->gwork,
-                      n->gwork_floats);
+int gemm(opf_net* n, const bf16* A, const bf16* Bm, int M, int N, int Kp, const opf::TcEpilogue& e,
+         int* splits = nullptr) {
+  return opf::tc_gemm(A, Bm, M, N, (int)pad128(M), (int)pad128(N), Kp, e, net_err(n), n->st, n->gwork,
+                      n->gwork_floats, splits);
 }
 
-opf::TcEpilogue epi(long ldo) {
-  opf::TcEpilogue e;
-  std::memset(&e, 0, sizeof e);
-  e.ldo = ldo;
+// the epilogue of a hidden layer: bias, GELU, the next layer's im2col rows
+opf::TcEpilogue hidden_epilogue(opf_net* n, const float* bias, float* pre, bf16* col) {
+  opf::TcEpilogue e{};
+  e.ldo = n->H;
+  e.bias = bias;
+  e.gelu = 1;
+  e.pre_f32 = pre;
+  e.col = col;
+  e.C = n->H;
+  e.L = n->L;
+  e.ldc = pad64(3L * n->H);
   return e;
 }
 
@@ -352,95 +443,79 @@ void prepare_weights(opf_net* n) {
                                                               (int)pad64(3L * H));
 }
 
-// forward for B samples whose features are at x (f32 [B][L][Cin])
-int net_forward(opf_net* n, const float* x, int B) {
-  const int L = n->L, Ci = n->Cin, H = n->H, O = n->O;
-  const long BL = (long)B * L, BLp = pad128(BL), K1 = pad64(3L * Ci), K2 = pad64(3L * H);
-  k_to_bf16<<<gs(BL * Ci), 256, 0, n->st>>>(x, n->xb, BL * Ci);
-  int rc;
-  // layer 1: h1 = gelu(col(x) W1^T + b1)
-  im2col(n->st, n->xb, L, Ci, (int)BL, 0, n->col[0], (int)BLp, (int)K1);
-  opf::TcEpilogue e = epi(H);
-  e.bias = Pf(n, 1), e.gelu = 1, e.pre_f32 = n->pre1, e.out_bf16 = n->h1;
-  if ((rc = gemm(n, n->col[0], n->wp[0], (int)BL, H, (int)K1, e))) return rc;
-  // layer 2
-  im2col(n->st, n->h1, L, H, (int)BL, 0, n->col[1], (int)BLp, (int)K2);
-  e = epi(H);
-  e.bias = Pf(n, 3), e.gelu = 1, e.pre_f32 = n->pre2, e.out_bf16 = n->h2;
-  if ((rc = gemm(n, n->col[1], n->wp[1], (int)BL, H, (int)K2, e))) return rc;
-  // layer 3 (linear)
-  im2col(n->st, n->h2, L, H, (int)BL, 0, n->col[2], (int)BLp, (int)K2);
-  e = epi(Ci);
-  e.bias = Pf(n, 5), e.out_f32 = n->y;
-  if ((rc = gemm(n, n->col[2], n->wp[2], (int)BL, Ci, (int)K2, e))) return rc;
-  k_pool<<<(B * H + 255) / 256, 256, 0, n->st>>>(n->h2, B, L, H, n->pooled);
-  k_head<<<(B * O + 255) / 256, 256, 0, n->st>>>(n->pooled, Pf(n, 6), Pf(n, 7), B, H, O, n->z);
-  return OPF_OK;
-}
-
-// gradient of one width-3 conv layer (input width Cin, output Cout) given
-// dZ (bf16 [BL][Cout], f32 copy dZf) and the layer's im2col rows col:
-//   dW[o][k] = sum_m dZ[m][o] col[m][k]        (operands dZ^T, col^T; K = BL)
-//   db[o]    = sum_m dZ[m][o]
-//   dx[m][c] = sum_{j,o} dZ[(b, l + 1 - j)][o] W[o][j*Cin + c]   (operands col_rev(dZ), ws)
-int conv_backward(opf_net* n, int B, const bf16* col, int Kc, int Cin, int Cout, const bf16* dZ, const float* dZf,
-                  const bf16* wsh, float* dW, float* db, float* dx) {
-  const int L = n->L;
-  const long BL = (long)B * L, BLp = pad128(BL);
-  int rc;
-  dim3 tb(32, 8);
-  k_transpose<<<dim3((unsigned)(BLp / 32), (unsigned)(pad128(Cout) / 32)), tb, 0, n->st>>>(
-      dZ, (int)BL, Cout, Cout, n->dzT, (int)BLp, (int)pad128(Cout));
-  k_transpose<<<dim3((unsigned)(BLp / 32), (unsigned)(pad128(3L * Cin) / 32)), tb, 0, n->st>>>(
-      col, (int)BL, 3 * Cin, Kc, n->colT, (int)BLp, (int)pad128(3L * Cin));
-  opf::TcEpilogue e = epi(3L * Cin);
-  e.out_f32 = dW;
-  if ((rc = gemm(n, n->dzT, n->colT, Cout, 3 * Cin, (int)BLp, e))) return rc;
-  k_colsum<<<(Cout + 31) / 32, dim3(32, 32), 0, n->st>>>(dZf, (int)BL, Cout, db);
-  if (dx) {
-    const long Kd = pad64(3L * Cout);
-    im2col(n->st, dZ, L, Cout, (int)BL, 1, n->dzcol, (int)BLp, (int)Kd);
-    e = epi(Cin);
-    e.out_f32 = dx;
-    if ((rc = gemm(n, n->dzcol, wsh, (int)BL, Cin, (int)Kd, e))) return rc;
-  }
-  return OPF_OK;
-}
-
-// loss and all parameter gradients into n->G for targets ty [B][L][Cin], tz [B][O]
-int net_gradients(opf_net* n, const float* x, const float* ty, const float* tz, int B, float lambda,
-                  double* loss) {
+// forward for B samples whose features are at x (f32 [B][L][Cin]) into y and
+// z; grad: the hidden layers' inputs to the GELU are kept for the gradients
+int net_forward(opf_net* n, const float* x, int B, float* y, float* z, bool grad) {
   const int L = n->L, Ci = n->Cin, H = n->H, O = n->O;
   const long BL = (long)B * L, K1 = pad64(3L * Ci), K2 = pad64(3L * H);
-  int rc = net_forward(n, x, B);
-  if (rc) return rc;
+  int rc;
+  if (Ci % 8 == 0 && !((uintptr_t)x & 15))
+    k_x_cols<true><<<dim3((unsigned)BL, (unsigned)((Ci / 8 + 127) / 128)), 128, 0, n->st>>>(x, L, Ci, n->col[0], K1);
+  else
+    k_x_cols<false><<<dim3((unsigned)BL, (unsigned)((Ci + 127) / 128)), 128, 0, n->st>>>(x, L, Ci, n->col[0], K1);
+  // h1 = gelu(col(x) W1^T + b1), h2 likewise, y linear
+  if ((rc = gemm(n, n->col[0], n->wp[0], (int)BL, H, (int)K1,
+                 hidden_epilogue(n, Pf(n, 1), grad ? n->pre1 : nullptr, n->col[1]))))
+    return rc;
+  if ((rc = gemm(n, n->col[1], n->wp[1], (int)BL, H, (int)K2,
+                 hidden_epilogue(n, Pf(n, 3), grad ? n->pre2 : nullptr, n->col[2]))))
+    return rc;
+  opf::TcEpilogue e{};
+  e.ldo = Ci;
+  e.bias = Pf(n, 5);
+  e.out_f32 = y;
+  if ((rc = gemm(n, n->col[2], n->wp[2], (int)BL, Ci, (int)K2, e))) return rc;
+  k_pool_head<<<B, kPoolThreads, 0, n->st>>>(n->col[2], K2, L, H, O, Pf(n, 6), Pf(n, 7), n->pooled, z);
+  return OPF_OK;
+}
+
+// loss and all parameter gradients into n->G for targets ty [B][L][Cin], tz [B][O]:
+//   dW[o][k] = sum_m dZ[m][o] col[m][k],  db[o] = sum_m dZ[m][o],
+//   dx[m][c] = sum_{j,o} dZ[(b, l + 1 - j)][o] W[o][j*Cin + c]
+int net_gradients(opf_net* n, const float* x, const float* ty, const float* tz, int B, float lambda) {
+  const int L = n->L, Ci = n->Cin, H = n->H, O = n->O;
+  const long BL = (long)B * L, K1 = pad64(3L * Ci), K2 = pad64(3L * H), ldz = net_ldz(n);
+  const int rows = (int)((BL + kGradRows - 1) / kGradRows);
+  const float zscale = lambda / (float)(B * O);
+  float *cs3 = n->csum, *cs2 = cs3 + (long)rows * Ci, *cs1 = cs2 + (long)rows * H;
   NCU(cudaMemsetAsync(n->sums, 0, 2 * sizeof(double), n->st));
-  // dL/dy = 2 (y - ty) / (BL Ci); dL/dz = 2 lambda (z - tz) / (B O)
-  k_mse<<<gs(BL * Ci), 256, 0, n->st>>>(n->y, ty, BL * Ci, 1.f / (float)(BL * Ci), n->dy, n->sums);
-  k_mse<<<1, 256, 0, n->st>>>(n->z, tz, (long)B * O, lambda / (float)(B * O), n->dzh, n->sums + 1);
-  // layer 3 (linear): dZ3 = dy
-  k_to_bf16<<<gs(BL * Ci), 256, 0, n->st>>>(n->dy, n->dz, BL * Ci);
-  if ((rc = conv_backward(n, B, n->col[2], (int)K2, H, Ci, n->dz, n->dy, n->ws[1], Gf(n, 4), Gf(n, 5), n->dh)))
-    return rc;
-  // head: pooled mean of h2
-  const int hb = (int)std::max<long>((long)O * H, (long)B * H);
-  k_head_back<<<(hb + 255) / 256, 256, 0, n->st>>>(n->dzh, n->pooled, Pf(n, 6), B, H, O, Gf(n, 6), Gf(n, 7),
-                                                   n->dpooled);
-  k_unpool_add<<<gs(BL * H), 256, 0, n->st>>>(n->dpooled, B, L, H, n->dh);
+  int rc = net_forward(n, x, B, n->y, n->z, true);
+  if (rc) return rc;
+  auto weights = [&](const bf16* col, long ldc, int Cin, int Cout, float* dW) {
+    return opf::tc_gemm_columns(n->dz, ldz, col, ldc, Cout, 3 * Cin, (int)BL, dW, 3L * Cin, net_err(n), n->st,
+                                n->gwork, n->gwork_floats);
+  };
+  // the gradient of the layer's input: dh, or split sums in the work space
+  const float* dh = nullptr;
+  int nsplit = 1;
+  auto inputs = [&](const bf16* dzcol, const bf16* ws, int Cin, int Kd) {
+    opf::TcEpilogue e{};
+    e.ldo = Cin;
+    e.out_f32 = n->dh;
+    const int r = gemm(n, dzcol, ws, (int)BL, Cin, Kd, e, &nsplit);
+    dh = nsplit > 1 ? n->gwork : n->dh;
+    return r;
+  };
+  auto hidden = [&](const float* pre, bool head, bf16* dzcol, float* csum) {
+    k_hidden_grad<<<dim3((unsigned)((H + 63) / 64), (unsigned)rows), 256, 0, n->st>>>(
+        dh, nsplit, pre, (int)BL, L, H, head ? n->dpool : nullptr, n->dz, ldz, dzcol, K2, csum);
+  };
+  // layer 3 (linear): dZ = dL/dy = 2 (y - ty) / (BL Ci); head: dL/dz = 2 lambda (z - tz) / (B O)
+  k_out_grad<<<dim3((unsigned)((Ci + 63) / 64), (unsigned)rows), 256, 0, n->st>>>(
+      n->y, ty, (int)BL, L, Ci, 1.f / (float)(BL * Ci), n->dz, ldz, n->dzcol[1], K1, cs3, n->sums);
+  k_head_grad<<<dim3((unsigned)((H + 127) / 128), (unsigned)(O + B)), 128, 0, n->st>>>(
+      n->z, tz, zscale, n->pooled, Pf(n, 6), B, L, H, O, Gf(n, 6), Gf(n, 7), n->dpool, n->sums + 1);
+  if ((rc = weights(n->col[2], K2, H, Ci, Gf(n, 4)))) return rc;
+  if ((rc = inputs(n->dzcol[1], n->ws[1], H, (int)K1))) return rc;
   // layer 2
-  k_gelu_back<<<gs(BL * H), 256, 0, n->st>>>(n->dh, n->pre2, n->dz, n->dy, BL * H);
-  if ((rc = conv_backward(n, B, n->col[1], (int)K2, H, H, n->dz, n->dy, n->ws[0], Gf(n, 2), Gf(n, 3), n->dh)))
-    return rc;
+  hidden(n->pre2, true, n->dzcol[0], cs2);
+  if ((rc = weights(n->col[1], K2, H, H, Gf(n, 2)))) return rc;
+  if ((rc = inputs(n->dzcol[0], n->ws[0], H, (int)K2))) return rc;
   // layer 1 (input gradient not needed)
-  k_gelu_back<<<gs(BL * H), 256, 0, n->st>>>(n->dh, n->pre1, n->dz2, n->dy, BL * H);
-  if ((rc = conv_backward(n, B, n->col[0], (int)K1, Ci, H, n->dz2, n->dy, nullptr, Gf(n, 0), Gf(n, 1), nullptr)))
-    return rc;
-  if (loss) {
-    double h[2];
-    NCU(cudaMemcpyAsync(h, n->sums, sizeof h, cudaMemcpyDeviceToHost, n->st));
-    NCU(cudaStreamSynchronize(n->st));
-    *loss = h[0] / (double)(BL * Ci) + lambda * h[1] / (double)(B * O);
-  }
+  hidden(n->pre1, false, nullptr, cs1);
+  if ((rc = weights(n->col[0], K1, Ci, H, Gf(n, 0)))) return rc;
+  const BiasSums bs{{cs3, cs2, cs1}, {Gf(n, 5), Gf(n, 3), Gf(n, 1)}, {Ci, H, H}};
+  k_bias_sum<<<dim3((unsigned)((std::max(Ci, H) + 31) / 32), 3), 256, 0, n->st>>>(bs, rows);
   NCU(cudaGetLastError());
   return OPF_OK;
 }
@@ -527,7 +602,8 @@ opf_net_t* opf_net_create(int cin, int hidden, int L, int nout, unsigned long lo
       cudaMalloc(&n->wp[2], pad128(cin) * pad64(3L * hidden) * sizeof(bf16)) != cudaSuccess ||
       cudaMalloc(&n->ws[0], pad128(hidden) * pad64(3L * hidden) * sizeof(bf16)) != cudaSuccess ||
       cudaMalloc(&n->ws[1], pad128(hidden) * pad64(3L * cin) * sizeof(bf16)) != cudaSuccess ||
-      cudaMalloc(&n->err, sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&n->sums, 3 * sizeof(double)) != cudaSuccess ||
+      cudaMallocHost(&n->read, 3 * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&n->gwork, (n->gwork_floats = 8L * std::max(3L * hidden * std::max(cin, hidden), 1L)) *
                                 sizeof(float)) != cudaSuccess) {
     opf::set_last_error("opf_net_create: device allocation failed");
@@ -538,7 +614,7 @@ opf_net_t* opf_net_create(int cin, int hidden, int L, int nout, unsigned long lo
   cudaMemset(n->G, 0, t * sizeof(float));
   cudaMemset(n->M1, 0, t * sizeof(float));
   cudaMemset(n->M2, 0, t * sizeof(float));
-  cudaMemset(n->err, 0, sizeof(int));
+  cudaMemset(n->sums, 0, 3 * sizeof(double));
   refresh_bf16(n);
   if (cudaStreamSynchronize(n->st) != cudaSuccess) {
     opf::set_last_error("opf_net_create: initialisation failed");
@@ -551,14 +627,13 @@ opf_net_t* opf_net_create(int cin, int hidden, int L, int nout, unsigned long lo
 void opf_net_destroy(opf_net_t* n) {
   if (!n) return;
   if (n->st) cudaStreamSynchronize(n->st);
-  for (void* p : {(void*)n->P, (void*)n->G, (void*)n->M1, (void*)n->M2, (void*)n->Pb, (void*)n->xb,
-                  (void*)n->h1, (void*)n->h2, (void*)n->dz, (void*)n->dz2, (void*)n->pre1, (void*)n->pre2,
-                  (void*)n->y, (void*)n->dy, (void*)n->dh, (void*)n->pooled, (void*)n->z, (void*)n->dzh,
-                  (void*)n->dpooled, (void*)n->sums, (void*)n->col[0], (void*)n->col[1], (void*)n->col[2],
-                  (void*)n->colT, (void*)n->dzT, (void*)n->dzcol, (void*)n->wp[0], (void*)n->wp[1],
-                  (void*)n->wp[2], (void*)n->ws[0], (void*)n->ws[1], (void*)n->err, (void*)n->gwork,
-                  (void*)n->aug_idx, (void*)n->aug_ang})
+  for (void* p : {(void*)n->P, (void*)n->G, (void*)n->M1, (void*)n->M2, (void*)n->Pb, (void*)n->pre1,
+                  (void*)n->pre2, (void*)n->y, (void*)n->dh, (void*)n->pooled, (void*)n->dpool, (void*)n->z, (void*)n->csum,
+                  (void*)n->sums, (void*)n->col[0], (void*)n->col[1], (void*)n->col[2], (void*)n->dz,
+                  (void*)n->dzcol[0], (void*)n->dzcol[1], (void*)n->wp[0], (void*)n->wp[1], (void*)n->wp[2], (void*)n->ws[0],
+                  (void*)n->ws[1], (void*)n->gwork, (void*)n->aug_idx, (void*)n->aug_ang})
     if (p) cudaFree(p);
+  if (n->read) cudaFreeHost(n->read);
   if (n->st) cudaStreamDestroy(n->st);
   delete n;
 }
@@ -596,12 +671,16 @@ int opf_net_set_params(opf_net_t* n, const float* host) {
   return OPF_OK;
 }
 
-// a tensor-core GEMM whose bounded wait ran out leaves the flag set
-static int net_check(opf_net_t* n) {
-  int h = 0;
-  NCU(cudaMemcpy(&h, n->err, sizeof(int), cudaMemcpyDeviceToHost));
+// Waits for the stream with the loss sums and the error flag in n->read; a
+// tensor-core GEMM whose bounded wait ran out leaves the flag set.
+static int net_finish(opf_net_t* n) {
+  NCU(cudaMemcpyAsync(n->read, n->sums, 3 * sizeof(double), cudaMemcpyDeviceToHost, n->st));
+  NCU(cudaStreamSynchronize(n->st));
+  NCU(cudaGetLastError());
+  int h;
+  std::memcpy(&h, n->read + 2, sizeof h);
   if (h) {
-    cudaMemset(n->err, 0, sizeof(int));
+    cudaMemset(net_err(n), 0, sizeof(int));
     opf::set_last_error("proposal network: a tensor-core GEMM timed out waiting for its operands");
     return OPF_ETIMEOUT;
   }
@@ -612,14 +691,9 @@ int opf_net_forward(opf_net_t* n, const float* d_x, int B, float* d_y, float* d_
   if (!n || !d_x || B < 1) return OPF_EINVAL;
   int rc = net_reserve(n, B);
   if (rc) return rc;
-  rc = net_forward(n, d_x, B);
+  rc = net_forward(n, d_x, B, d_y ? d_y : n->y, d_z ? d_z : n->z, false);
   if (rc) return rc;
-  const long BL = (long)B * n->L;
-  if (d_y) NCU(cudaMemcpyAsync(d_y, n->y, BL * n->Cin * sizeof(float), cudaMemcpyDeviceToDevice, n->st));
-  if (d_z) NCU(cudaMemcpyAsync(d_z, n->z, (long)B * n->O * sizeof(float), cudaMemcpyDeviceToDevice, n->st));
-  NCU(cudaStreamSynchronize(n->st));
-  NCU(cudaGetLastError());
-  return net_check(n);
+  return net_finish(n);
 }
 
 int opf_net_gradients(opf_net_t* n, const float* d_x, const float* d_ty, const float* d_tz, int B,
@@ -627,10 +701,12 @@ int opf_net_gradients(opf_net_t* n, const float* d_x, const float* d_ty, const f
   if (!n || !d_x || !d_ty || !d_tz || B < 1) return OPF_EINVAL;
   int rc = net_reserve(n, B);
   if (rc) return rc;
-  rc = net_gradients(n, d_x, d_ty, d_tz, B, lambda, loss);
+  rc = net_gradients(n, d_x, d_ty, d_tz, B, lambda);
   if (rc) return rc;
-  NCU(cudaStreamSynchronize(n->st));
-  return net_check(n);
+  rc = net_finish(n);
+  if (rc) return rc;
+  if (loss) *loss = n->read[0] / (double)((long)B * n->L * n->Cin) + lambda * n->read[1] / (double)(B * n->O);
+  return OPF_OK;
 }
 
 int opf_net_train_step(opf_net_t* n, const float* d_x, const float* d_ty, const float* d_tz, int B,
