@@ -205,8 +205,9 @@ int group_fill_setups(Group* g, bool first) {
   g->o_hop = pl.add(s0.hop.size() * sizeof(int));
   g->o_luH = pl.add(s0.luH.size() * 8);
   g->o_luP = pl.add(s0.luP.size() * 8);
-  g->o_basis = pl.add(s0.basis.size() * 8);
-  g->o_ainv = pl.add(s0.ainv.size() * 8);
+  const size_t nmode = (size_t)K * M;
+  g->o_basis = pl.add(nmode * opf::basis_ld(N) * 8);
+  g->o_ainv = pl.add((size_t)M * d.nk * sizeof(double2));
   g->o_G = pl.add(s0.G.size() * 8);
   g->o_twz = pl.add(d.nz * sizeof(double2));
   g->o_twt = pl.add(d.nth * sizeof(double2));
@@ -254,15 +255,15 @@ int group_fill_setups(Group* g, bool first) {
     put(g->o_hop, s.hop.data(), s.hop.size() * sizeof(int));
     put(g->o_luH, s.luH.data(), s.luH.size() * 8);
     put(g->o_luP, s.luP.data(), s.luP.size() * 8);
-    {  // device order [K][M][N][6]: the six responses of one radial row together
-      const size_t nmode = s.basis.size() / (6 * (size_t)d.N);
-      std::vector<double> bt(s.basis.size());
+    {  // the pressure's responses, the three of one radial row together
+      const int ld = opf::basis_ld(N);
+      double* out = (double*)(host.data() + g->o_basis);
       for (size_t q = 0; q < nmode; ++q)
-        for (int v = 0; v < 6; ++v)
-          for (int i = 0; i < d.N; ++i) bt[(q * d.N + i) * 6 + v] = s.basis[(q * 6 + v) * d.N + i];
-      put(g->o_basis, bt.data(), bt.size() * 8);
+        for (int i = 0; i < N; ++i)
+          for (int v = 0; v < 3; ++v) out[q * ld + i * 3 + v] = s.basis[(q * 6 + v) * N + i];
+      double2* ai = (double2*)(host.data() + g->o_ainv);
+      for (size_t q = 0; q < (size_t)M * d.nk; ++q) ai[q] = double2{s.ainv[q * 32 + 6], s.ainv[q * 32 + 7]};
     }
-    put(g->o_ainv, s.ainv.data(), s.ainv.size() * 8);
     put(g->o_G, s.G.data(), s.G.size() * 8);
     put(g->o_twz, twz.data(), d.nz * sizeof(double2));
     put(g->o_twt, twt.data(), d.nth * sizeof(double2));
@@ -538,13 +539,9 @@ void enqueue_nonlinear(Runner* r, const Group& g, const double2* U, double2* Nou
 bool fused_curl(const Runner* r) { return r->precision == 0; }
 
 // Solve pass into Uout (and, fused, the curl of Uout into W6).
-void enqueue_solve(Runner* r, const Group& g, const double2* Na, const double2* Nb, double wa,
-                   double wb, double2* Uout) {
-  opf::SolveArgs a{g.U, Na, Nb, wa, wb, Uout, g.beta_p};
-  if (fused_curl(r)) {
-    a.curl = 1;
-    a.W6 = (void*)g.W6;
-  }
+void enqueue_solve(Runner* r, const Group& g, const double2* Na, const double2* Nb, double2* Uout) {
+  opf::SolveArgs a{g.U, Na, Nb, Uout, g.beta_p};
+  if (fused_curl(r)) a.W6 = g.W6;
   r->begin(4);
   opf::launch_solve(g.d, g.ds, a, g.nJ, r->st());
   r->end();
@@ -589,19 +586,18 @@ void enqueue_step(Runner* r) {
       r->cur = r->side[i - 1];
       cudaStreamWaitEvent(r->cur, r->fork_ev, 0);
     }
-    const double c = g->d.c;
     if (g->d.cfl) cudaMemsetAsync(g->cfl, 0, sizeof(double), r->st());
     // fused: W6 holds the curl of U at the start of a step (runner_step) and
     // the solves leave the curl of their output
     const bool curl = !fused_curl(r);
     enqueue_nonlinear(r, *g, g->U, g->Nj, curl);
-    enqueue_solve(r, *g, g->Nj, nullptr, 1.0, 0.0, g->U1);
+    enqueue_solve(r, *g, g->Nj, nullptr, g->U1);
     if (r->n_corr == 0)  // predictor only: its output (3F per trajectory) is the new state
       cudaMemcpy2DAsync(g->U, g->sstride, g->U1, g->sstride, 3 * (size_t)g->d.F * sizeof(double2), g->d.B,
                         cudaMemcpyDeviceToDevice, r->st());
     for (int q = 0; q < r->n_corr; ++q) {
       enqueue_nonlinear(r, *g, g->U1, g->Nq, curl);
-      enqueue_solve(r, *g, g->Nq, g->Nj, c, 1.0 - c, q == r->n_corr - 1 ? g->U : g->U1);
+      enqueue_solve(r, *g, g->Nq, g->Nj, q == r->n_corr - 1 ? g->U : g->U1);
     }
     if (fork && i > 0) cudaEventRecord(r->join_ev[i - 1], r->cur);
   }
@@ -709,7 +705,7 @@ int tune_group(Runner* r, Group* g) {
     if (d.spike) break;
     if (opf::solve_smem_bytes(d.N, T) > (size_t)optin) continue;
     d.tile = T;
-    opf::SolveArgs a{g->U, g->Nj, nullptr, 1.0, 0.0, g->U1, g->beta_p};
+    opf::SolveArgs a{g->U, g->Nj, nullptr, g->U1, g->beta_p};
     const float t = time_launch(r, [&] { opf::launch_solve(d, g->ds, a, g->nJ, st); });
     if (t < best) best = t, pick = T;
   }

@@ -66,6 +66,9 @@ struct DftTables {
   int zshift = 0;  // the z analysis' results count 2^zshift
 };
 
+// Doubles per mode of the device's influence responses: N rows of 3, an even number.
+__host__ __device__ constexpr int basis_ld(int N) { return (3 * N + 1) & ~1; }
+
 struct DevSetup {
   DftTables dft;
   double* prm = nullptr;  // [kPrmCount] Re, dt, c, sum(wq G)
@@ -75,8 +78,10 @@ struct DevSetup {
   int* hop = nullptr;
   double* luH = nullptr;
   double* luP = nullptr;
-  double* basis = nullptr;  // device order [K][M][N][6] (host Setup: [K][M][6][N])
-  double2* ainv = nullptr;
+  // pressure responses of (u+, u-, u_z), [K][M][basis_ld(N)] with rows of 3
+  // (host Setup: [K][M][6][N], with the unit wall responses)
+  double* basis = nullptr;
+  double2* ainv = nullptr;  // [M][2K-1]: the pressure response's entry for the wall divergence
   double* G = nullptr;
   double2* tw_z = nullptr;   // e^{+2 pi i t / nz}, t < nz
   double2* tw_th = nullptr;  // e^{+2 pi i t / nth}
@@ -180,16 +185,12 @@ void launch_dft_zanalysis(const Dims& d, const DevSetup& s, const double2* ZN, d
 struct SolveArgs {
   const double2* Uj;
   const double2* Na;
-  const double2* Nb;
-  double wa, wb;
+  const double2* Nb;  // null: N_eff = N_a, else (N_a + N_b) / 2
   double2* Uout;
   double* beta_p;  // device scalar: beta' of this solve (written by the (0,0) mode)
-  // curl of the solved state for the next nonlinear evaluation, computed by
-  // the same blocks from their radial columns: 0 none, 1 FP64 into W6
-  // (double2), 2 mixed precision into W6 (float2) and the FP64 linear terms Nlin
-  int curl = 0;
-  void* W6 = nullptr;
-  double2* Nlin = nullptr;
+  // FP64 curl of the solved state for the next nonlinear evaluation, computed
+  // by the same blocks from their radial columns (null: none)
+  double2* W6 = nullptr;
 };
 void launch_solve(const Dims& d, const DevSetup& s, const SolveArgs& a, int nJ, cudaStream_t st);
 void launch_energy(const Dims& d, const DevSetup& s, const double2* U, const double2* W6,

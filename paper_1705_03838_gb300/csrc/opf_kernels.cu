@@ -1008,8 +1008,6 @@ struct SolveDev {
   const double* prm;
   int nJ;
   int stage;  // u_j and the influence responses staged in shared memory
-  const float* d1f;
-  const double* r;
   // split solve: both blocks' factors, spikes, interface inverses
   const double* luH2;
   const double* luP2;
@@ -1018,6 +1016,13 @@ struct SolveDev {
   const double* rH;
   const double* rP;
 };
+
+// x / 2 by its exponent (an FP64 multiplication takes as long as an addition).
+__device__ __forceinline__ double halved(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+  return e - 2u < 0x7fdu ? __hiloint2double(hi - 0x100000, __double2loint(x)) : 0.5 * x;
+}
 
 // Bulk L2 prefetch by the TMA unit: p 16-byte aligned, bytes a multiple of 16.
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, unsigned bytes) {
@@ -1044,18 +1049,14 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // the influence step and the write-out read them from shared memory.
 // The host stages only where that costs no resident blocks (see
 // launch_solve); the launch gives the staged size then, the base size else.
-// Rows of P: the pressure, later the influence step's scratch (12 complex per mode).
-__host__ __device__ constexpr int solve_prows(int N) { return N > 12 ? N : 12; }
 // sp: the split solve's interface values (6T chains x 8 doubles) after misc.
 __host__ __device__ constexpr size_t solve_smem_base(int N, int T, bool sp = false) {
-  return (size_t)(N * T + solve_prows(N) * T + 4 * T) * 16 + (size_t)6 * N * T * 8 +
+  return (size_t)(2 * N * T + T) * 16 + (size_t)6 * N * T * 8 +
          (size_t)(2 * N * 9 + 3 * N + 2) * 8 + 16 + (sp ? (size_t)48 * T * 8 : 0);
 }
 __host__ __device__ constexpr size_t solve_smem_staged(int N, int T, bool sp = false) {
-  return solve_smem_base(N, T, sp) + (size_t)96 * N * T;
+  return solve_smem_base(N, T, sp) + (size_t)48 * N * T + (size_t)8 * basis_ld(N) * T;
 }
-// The FP32 copy of u_theta for the mixed-precision curl of the solved state.
-__host__ __device__ constexpr size_t solve_smem_curl32(int N, int T) { return (size_t)8 * N * T; }
 __host__ __device__ constexpr bool solve_stage_fits(int N, int T) { return solve_smem_staged(N, T) <= 100 * 1024; }
 
 // Banded substitution on one real right-hand side held in shared memory at
@@ -1247,9 +1248,9 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   // the velocity right-hand sides built on it in place, then the chains'
   // solutions; S and P are reused by the influence step and the curl.
   double2* S = (double2*)smraw;                // [N][T]     N+ + N- (later u_j near the wall, u_r)
-  double2* P = S + N * T;                      // [N][T]     pressure (later influence scratch, u_theta)
-  double2* coef = P + solve_prows(N) * T;      // [T][4]     influence coefficients
-  double* X = (double*)(coef + 4 * T);         // [N][6T]    N_eff -> right-hand sides -> velocity chains
+  double2* P = S + N * T;                      // [N][T]     pressure (later u_theta)
+  double2* coef = P + N * T;                   // [T]        influence coefficients
+  double* X = (double*)(coef + T);             // [N][6T]    N_eff -> right-hand sides -> velocity chains
   double* W1 = X + N * NT;                     // [2][N][9]  first-derivative stencils
   double* RI = W1 + 2 * N * 9;                 // [N]        1/r
   double* RIp = RI + N;                        // [N]        (1 + m~) / (2r)
@@ -1257,13 +1258,12 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   double* misc = RIm + N;                      // [2]        flux correction
   const bool stage = s.stage;
   // u_j near the wall for the influence step, when not staged: in S (free
-  // after the pressure right-hand side) if it holds [T][19], else from global
+  // after the pressure right-hand side) if it holds [T][16], else from global
   double2* UW = S;
-  const bool uw_in_s = !stage && N >= 19;
+  const bool uw_in_s = !stage && N >= 16;
   double* Zs = misc + 2;                       // [6T][8]    split-solve interface values (SP)
   double2* UJ = (double2*)(((size_t)(Zs + (SP ? 48 * T : 0)) + 15) & ~(size_t)15);  // [3][N][T] u_j (stage)
-  double* BS = (double*)(UJ + 3 * N * T);                             // [T][6N]   responses (stage)
-  float2* UT32 = stage ? (float2*)(BS + 6 * N * T) : (float2*)UJ;     // [N][T] FP32 u_theta (curl 2)
+  double* BS = (double*)(UJ + 3 * N * T);                             // [T][basis_ld] responses (stage)
   // N_eff of field f, row i, mode mi as a complex pair in X's chain layout
   auto ne_at = [&](int f, int i, int mi) -> double2& {
     return *(double2*)(X + (long)i * NT + ((f * T + mi) << 1));
@@ -1280,8 +1280,6 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   s.ainv = bofs(s.ainv, d.ps);
   s.G = bofs(s.G, d.ps);
   s.prm = bofs(s.prm, d.ps);
-  s.d1f = bofs(s.d1f, d.ps);
-  s.r = bofs(s.r, d.ps);
   if constexpr (SP) {
     s.luH2 = bofs(s.luH2, d.ps);
     s.luP2 = bofs(s.luP2, d.ps);
@@ -1291,7 +1289,6 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     s.rP = bofs(s.rP, d.ps);
   }
   a.W6 = bofs(a.W6, d.ss);
-  a.Nlin = bofs(a.Nlin, d.ss);
   a.Uj = bofs(a.Uj, d.ss);
   a.Na = bofs(a.Na, d.ss);
   a.Nb = bofs(a.Nb, d.ss);
@@ -1311,12 +1308,12 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   // Pull this block's factor blocks (pressure, u+, u-, u_z per mode) and
   // basis blocks towards L2 with one bulk prefetch each, so they arrive while
   // the right-hand sides are assembled.  Factor blocks start on 16 bytes only
-  // for even N (104 N bytes per operator); basis blocks (48 N bytes) always do.
+  // for even N (104 N bytes per operator); basis blocks always do.
   if (tid < 5 * T) {
     const int mi = tid % T, which = tid / T;
     const int ik = abs(min(kk0 + mi, nk - 1) - (K - 1));
     if (which == 4) {
-      if (!stage) prefetch_l2_bulk(s.basis + (long)(ik * M + m) * 6 * N, 48u * N);
+      if (!stage) prefetch_l2_bulk(s.basis + (long)(ik * M + m) * basis_ld(N), 8u * basis_ld(N));
     } else if (!(N & 1)) {
       const long op = which == 0 ? ((ik == 0 && m == 0) ? K * M : ik * M + m) : ik * s.nJ + s.hop[3 * m + which - 1];
       prefetch_l2_bulk((which == 0 ? (SP ? s.luP2 : s.luP) : (SP ? s.luH2 : s.luH)) + op * N * kLuSlots,
@@ -1328,7 +1325,8 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   for (int e = tid; e < 2 * N * 9; e += NB) cp_async8(W1 + e, s.d1 + e);
   cp_async_commit();
 
-  // ---- N_eff = wa N_a + wb N_b, and N+ + N- for the divergence
+  // ---- N_eff = N_a (predictor) or (N_a + N_b) / 2 (corrector, c = 1/2), and
+  //      N+ + N- for the divergence
   for (int e = tid; e < N; e += NB) {
     const double ri = s.rinv[e];
     RI[e] = ri;
@@ -1340,13 +1338,10 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   for (int e = tid; e < 3 * N * T; e += NB) {
     const int mi = e % T, i = (e / T) % N, f = e / (T * N);
     const long g = f * fs + base + (long)i * nk + min(kk0 + mi, nk - 1);
-    const double2 u = a.Na[g];
-    double2 v = u;
-    if (a.wa != 1.0) v = double2{a.wa * u.x, a.wa * u.y};  // (the predictor takes N_a as it is)
+    double2 v = a.Na[g];
     if (a.Nb) {
       const double2 w = a.Nb[g];
-      v.x += a.wb * w.x;
-      v.y += a.wb * w.y;
+      v = double2{halved(v.x + w.x), halved(v.y + w.y)};
     }
     ne_at(f, i, mi) = v;
   }
@@ -1402,36 +1397,30 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     for (int e = tid - NP; e < N * NT; e += NB - NP) {
       const int c = e % NT, i = e / NT;
       const int part = c & 1, mi = (c >> 1) % T, f = (c >> 1) / T;
-      double b = 0.0;
-      if (i < N - 1) {
-        const double2 u = uj(f, i, mi);
-        if (stage && part == 0) UJ[(f * N + i) * T + mi] = u;
-        b = fma(ci, part ? u.y : u.x, X[i * NT + c]);  // X held N_eff of this chain's element
-      }
+      const double2 u = uj(f, i, mi);
+      if (stage && part == 0) UJ[(f * N + i) * T + mi] = u;
+      const double w = part ? u.y : u.x;
+      double b;
+      if (i < N - 1) b = fma(ci, w, X[i * NT + c]);  // X held N_eff of this chain's element
+      else b = m == 0 && kk0 + mi == K - 1 ? 0.0 : cu * w;
       X[i * NT + c] = b;
     }
-    // u_j near the wall and the inverse influence matrices of the tile, for
-    // the influence step (rows N-9..N-1 of u+, u-; row N-1 of u_z)
-    // (staged: u_j of the wall row and the influence responses of the tile
-    // into shared memory instead, for the influence step and the write-out)
+    // u_j near the wall for the influence step (rows N-9..N-2 of u+, u-), or,
+    // staged, the influence responses of the tile
     if (stage) {
-      for (int e = tid - NP; e < 3 * T; e += NB - NP) {
-        const int mi = e % T, f = e / T;
-        UJ[(f * N + N - 1) * T + mi] = uj(f, N - 1, mi);
-      }
-      for (int e = tid - NP; e < 3 * N * T; e += NB - NP) {  // 16-byte chunks, 3N per mode
-        const int mi = e / (3 * N), ch = e % (3 * N);
+      const int nch = basis_ld(N) / 2;  // 16-byte chunks per mode
+      for (int e = tid - NP; e < nch * T; e += NB - NP) {
+        const int mi = e / nch, ch = e - mi * nch;
         const int ik = abs(min(kk0 + mi, nk - 1) - (K - 1));
-        cp_async16(BS + (long)mi * 6 * N + 2 * ch, s.basis + (long)(ik * M + m) * 6 * N + 2 * ch);
+        cp_async16(BS + (long)mi * basis_ld(N) + 2 * ch, s.basis + (long)(ik * M + m) * basis_ld(N) + 2 * ch);
       }
       cp_async_commit();
       cp_async_wait<0>();
     }
     if (uw_in_s) {
-      for (int e = tid - NP; e < 19 * T; e += NB - NP) {
+      for (int e = tid - NP; e < 16 * T; e += NB - NP) {
         const int mi = e % T, w = e / T;
-        const int f = w < 18 ? w / 9 : 2, i = w < 18 ? N - 9 + w % 9 : N - 1;
-        UW[mi * 19 + w] = uj(f, i, mi);
+        UW[mi * 16 + w] = uj(w >> 3, N - 9 + (w & 7), mi);
       }
     }
   }
@@ -1468,7 +1457,7 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   }
   __syncthreads();
 
-  // ---- implicit viscous solves (1/dt - cL) v = rhs, Dirichlet 0
+  // ---- implicit viscous solves (1/dt - cL) v = rhs, v(1) = ((1-c)/c) u_j(1)
   {  // 6T chains x 4 (SP: 8) lanes = all threads
     const int c = tid >> (SP ? 3 : 2);
     const int mi = (c >> 1) % T, f = (c >> 1) / T;
@@ -1488,83 +1477,46 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
       return ik * s.nJ + s.hop[3 * m + (c >> 1) / T];
     });
 
-  // ---- influence matrix on u = v - ((1-c)/c) u_j:
-  //      g = (u+(1), u-(1), u_z(1), div u(1)),  a = -A^{-1} g.
-  //      A warp issues one FP64 instruction per ~64 cycles on GB300 whatever
-  //      its active lanes, so the work is spread: step 1, one thread per
-  //      (mode, tap) of the wall divergence stencil and per (mode, field) of
-  //      u(1); step 2, one thread per (mode, row of A^{-1}, re/im part), the
-  //      tap sum reduced over the mode's 8 lanes.  (P is free by now.)
-  {
-    double2* Dt = P;          // [T][9] w_q (u+ + u-)(N-9+q)
-    double2* Gw = P + 9 * T;  // [T][3] u+-, u_z at the wall
-    auto uv = [&](int ff, int i, int mj) {  // rows N-9.. of u+-, row N-1 of u_z
+  // ---- influence matrix on u = v - ((1-c)/c) u_j.  The wall value of v makes
+  //      u(1) = 0 exactly, so of the boundary vector g = (u+(1), u-(1), u_z(1),
+  //      div u(1)) only the divergence is left, and of the coefficients
+  //      a = -A^{-1} g only the pressure response's (the unit wall responses
+  //      have zero there).  Eight threads per mode, one per row of the wall
+  //      stencil (its ninth row is the wall).
+  if (tid < 8 * T) {  // whole warps (T >= 4)
+    const int mj = tid >> 3, q = tid & 7, i = N - 9 + q;
+    const double2 A = s.ainv[(long)m * nk + min(kk0 + mj, nk - 1)];
+    auto uv = [&](int ff) {
       const int c = (ff * T + mj) << 1;
       const double2 w = stage     ? UJ[(ff * N + i) * T + mj]
-                        : uw_in_s ? UW[mj * 19 + (ff < 2 ? ff * 9 + i - (N - 9) : 18)]
+                        : uw_in_s ? UW[mj * 16 + ff * 8 + q]
                                   : uj(ff, i, mj);
       return double2{X[i * NT + c] - cu * w.x, X[i * NT + c + 1] - cu * w.y};
     };
-    // row r of A^{-1} for the step-2 threads, loaded while step 1 runs
-    double2 Ar[4];
-    if (tid < 8 * T) {
-      const int mj = tid >> 3, r = (tid >> 1) & 3;
-      const double2* Ag = s.ainv + ((long)m * nk + min(kk0 + mj, nk - 1)) * 16 + r * 4;
+    const double2 p = uv(0), mm = uv(1);
+    const double w = 0.5 * wv[(N - 1) * 9 + q];
+    double2 g = double2{w * (p.x + mm.x), w * (p.y + mm.y)};
 #pragma unroll
-      for (int c = 0; c < 4; ++c) Ar[c] = Ag[c];
+    for (int o = 4; o > 0; o >>= 1) {
+      g.x += __shfl_xor_sync(0xffffffffu, g.x, o, 8);
+      g.y += __shfl_xor_sync(0xffffffffu, g.y, o, 8);
     }
-    if (tid < 9 * T) {
-      const int mj = tid / 9, q = tid % 9, i = N - 9 + q;
-      const double2 p = uv(0, i, mj), mm = uv(1, i, mj);
-      const double w = wv[(N - 1) * 9 + q];
-      Dt[tid] = double2{w * (p.x + mm.x), w * (p.y + mm.y)};
-    } else if (tid < 12 * T) {
-      const int e = tid - 9 * T, mj = e / 3, f = e % 3;
-      Gw[e] = uv(f, N - 1, mj);
-    }
-    __syncthreads();
-    if (tid < 8 * T) {  // whole warps (T >= 4)
-      const int mj = tid >> 3, l = tid & 7, r = (tid >> 1) & 3, part = tid & 1;
-      double2 sum = Dt[mj * 9 + l];
-      if (l == 0) {
-        const double2 t8 = Dt[mj * 9 + 8];
-        sum = double2{sum.x + t8.x, sum.y + t8.y};
-      }
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) {
-        sum.x += __shfl_xor_sync(0xffffffffu, sum.x, o, 8);
-        sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o, 8);
-      }
-      const double2 g0 = Gw[mj * 3], g1 = Gw[mj * 3 + 1], g2 = Gw[mj * 3 + 2];
-      const double akj = d.alpha * (min(kk0 + mj, nk - 1) - (K - 1));
-      const double rp = RIp[N - 1], rm = RIm[N - 1];
-      const double2 g[4] = {g0, g1, g2,
-                            double2{fma(0.5, sum.x, fma(rp, g0.x, fma(rm, g1.x, -akj * g2.y))),
-                                    fma(0.5, sum.y, fma(rp, g0.y, fma(rm, g1.y, akj * g2.x)))}};
-      double acc = 0.0;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const double2 A = Ar[c];
-        acc = part ? fma(A.x, g[c].y, fma(A.y, g[c].x, acc)) : fma(A.x, g[c].x, fma(-A.y, g[c].y, acc));
-      }
-      ((double*)coef)[(mj * 4 + r) * 2 + part] = -acc;
-    }
-    __syncthreads();
+    if (q == 0) coef[mj] = double2{fma(A.y, g.y, -A.x * g.x), -fma(A.x, g.y, A.y * g.x)};
   }
+  __syncthreads();
 
-  // final value of chain c at row i: v - ((1-c)/c) u_j + basis responses
+  // final value of chain c at row i: v - ((1-c)/c) u_j + pressure response
   auto final_value = [&](int i, int c) {
     const int part = c & 1, mi = (c >> 1) % T, f = (c >> 1) / T;
     const int kk = min(kk0 + mi, nk - 1), k = kk - (K - 1);
-    const double* Bv = s.basis + (long)(abs(k) * M + m) * 6 * N;
-    const double2 a0 = coef[mi * 4 + 0], ax = coef[mi * 4 + 1 + f];
+    const double* Bv = s.basis + (long)(abs(k) * M + m) * basis_ld(N);
+    const double2 a0 = coef[mi];
     // u_z responses carry i sign(k): coefficient sign(k) (a0.x, -a0.y) swapped
     const double az = part ? a0.x : -a0.y;
     const double c0 = f == 2 ? (k > 0 ? az : (k < 0 ? -az : 0.0)) : (part ? a0.y : a0.x);
-    const double c1 = part ? ax.y : ax.x;
     const double2 w = stage ? UJ[(f * N + i) * T + mi] : a.Uj[f * fs + base + (long)i * nk + kk];
-    const double* B = stage ? BS + (long)mi * 6 * N : Bv;
-    return X[i * NT + c] - cu * (part ? w.y : w.x) + c0 * B[i * 6 + f] + c1 * B[i * 6 + 3 + f];
+    const double* B = stage ? BS + (long)mi * basis_ld(N) : Bv;
+    return fma(c0, B[i * 3 + f], X[i * NT + c] - cu * (part ? w.y : w.x));
   };
 
   // ---- fixed flux on (0,0): beta' so that 2 pi int u_z r dr = pi/2
@@ -1597,17 +1549,13 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     if (has_mean && c == cz) v += bp * s.G[i];
     double* out = (double*)(a.Uout + f * fs + base + (long)i * nk + kk0 + mi) + part;
     *out = v;
-    if (a.curl) X[i * NT + c] = v;  // (only this element's own X is read above)
+    if (a.W6) X[i * NT + c] = v;  // (only this element's own X is read above)
   }
 
   // ---- the curl of the new state (A1) for the next nonlinear evaluation, from
-  //      the block's radial columns (S and P are free: u_r, u_theta; the FP32
-  //      u_theta of the mixed-precision curl sits in the tail of shared memory).
-  //      The mixed-precision form (curl 2) is built into the 4-mode tile only:
-  //      the library's steps take it from k_curl, and in the larger tiles its
-  //      code made the solve spill more registers.
-  constexpr bool kMixedCurl = T == 4;
-  if (a.curl) {
+  //      the block's radial columns (S and P are free: u_r, u_theta).  FP64
+  //      steps only: mixed ones take it from k_curl.
+  if (a.W6) {
     __syncthreads();
     double2* UR = S;
     double2* UT = P;
@@ -1615,25 +1563,18 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     for (int i = tid / T; i < N; i += NB / T) {
       const double* xr = X + i * NT;
       const double2 up = double2{xr[c0], xr[c0 + 1]}, um = double2{xr[c1], xr[c1 + 1]};
-      const double2 ut = double2{0.5 * (up.y - um.y), -0.5 * (up.x - um.x)};
       UR[i * T + mi_t] = double2{0.5 * (up.x + um.x), 0.5 * (up.y + um.y)};
-      UT[i * T + mi_t] = ut;
-      if (kMixedCurl && a.curl == 2) UT32[i * T + mi_t] = float2{(float)ut.x, (float)ut.y};  // (curl 2 only)
+      UT[i * T + mi_t] = double2{0.5 * (up.y - um.y), -0.5 * (up.x - um.x)};
     }
     __syncthreads();
     const int kk = kk0 + mi_t;
     if (kk < nk) {
       auto uz_at = [&](int i) { return double2{X[i * NT + c2], X[i * NT + c2 + 1]}; };
       auto ut_at = [&](int i) { return UT[i * T + mi_t]; };
-      auto ut32_at = [&](int i) { return UT32[i * T + mi_t]; };
-      for (int i = tid / T; i < N; i += NB / T) {
-        if (kMixedCurl && a.curl == 2)
-          curl_point<float2, true>(d, m, kk, i, ak_t, W1, s.d1f, s.r, RI, uz_at, ut_at, ut32_at, UR[i * T + mi_t],
-                                   UT[i * T + mi_t], uz_at(i), (float2*)a.W6, a.Nlin);
-        else
-          curl_point<double2, false>(d, m, kk, i, ak_t, W1, s.d1f, s.r, RI, uz_at, ut_at, ut32_at,
-                                     UR[i * T + mi_t], UT[i * T + mi_t], uz_at(i), (double2*)a.W6, nullptr);
-      }
+      auto none = [](int) { return float2{}; };
+      for (int i = tid / T; i < N; i += NB / T)
+        curl_point<double2, false>(d, m, kk, i, ak_t, W1, nullptr, nullptr, RI, uz_at, ut_at, none, UR[i * T + mi_t],
+                                   UT[i * T + mi_t], uz_at(i), a.W6, nullptr);
     }
   }
 }
@@ -1784,9 +1725,8 @@ void launch_solve(const Dims& d, const DevSetup& s, const SolveArgs& a, int nJ, 
   dim3 g((d.nk + T - 1) / T, d.M, d.B);
   const bool stage = solve_use_stage(d, T, (long)g.x * g.y * g.z, sp);
   SolveDev sd{s.d1,  s.rinv, s.wq,   s.hop,  s.luH,  s.luP,  s.basis, s.ainv, s.G,  s.prm,
-              nJ,    stage ? 1 : 0,  s.d1f,  s.r,    s.luH2, s.luP2, s.spkH,  s.spkP, s.rH, s.rP};
-  const size_t sm = (stage ? solve_smem_staged(d.N, T, sp) : solve_smem_base(d.N, T, sp)) +
-                    (a.curl == 2 ? solve_smem_curl32(d.N, T) : 0);
+              nJ,    stage ? 1 : 0,  s.luH2, s.luP2, s.spkH,  s.spkP, s.rH, s.rP};
+  const size_t sm = stage ? solve_smem_staged(d.N, T, sp) : solve_smem_base(d.N, T, sp);
   if (T == 16) launch_step_kernel(d, k_solve<16>, g, dim3(24 * 16), sm, st, d, sd, a);
   else if (T == 8) launch_step_kernel(d, k_solve<8>, g, dim3(24 * 8), sm, st, d, sd, a);
   else if (sp) launch_step_kernel(d, k_solve<4, true>, g, dim3(48 * 4), sm, st, d, sd, a);
