@@ -265,12 +265,13 @@ __device__ __forceinline__ void curl_point(const Dims& d, int m, int kk, int n, 
     // w_z = d_r u_theta + u_theta / r - i m~ u_r / r, in FP32
     const float ri32 = d1f[2 * 9 * N + n], mri32 = (float)mt * ri32;
     const float2 ut32 = ut32_at(n);
-    const float urx = SUMS ? 0.5f * (float)ur.x : (float)ur.x, ury = SUMS ? 0.5f * (float)ur.y : (float)ur.y;
+    const float half = SUMS ? 0.5f : 1.f;
+    const float urx = half * to_float(ur.x), ury = half * to_float(ur.y);
     W6[0 * fs + w] = float2{urx, ury};
     W6[1 * fs + w] = ut32;
-    W6[2 * fs + w] = float2{(float)uzx, (float)uz.y};
-    W6[3 * fs + w] = float2{(float)(-xi), (float)xr};
-    W6[4 * fs + w] = float2{(float)wtx, (float)wty};
+    W6[2 * fs + w] = float2{to_float(uzx), to_float(uz.y)};
+    W6[3 * fs + w] = float2{-to_float(xi), to_float(xr)};
+    W6[4 * fs + w] = float2{to_float(wtx), to_float(wty)};
     W6[5 * fs + w] = float2{fmaf(mri32, ury, fmaf(ri32, ut32.x, dtx)), fmaf(-mri32, urx, fmaf(ri32, ut32.y, dty))};
   } else {
     W6[0 * fs + w] = ur;
@@ -336,7 +337,7 @@ __global__ void __launch_bounds__(kCurlThreads) k_curl(Dims d, int kc, const dou
       const double2 ut2 = double2{a.y - b.y, b.x - a.x};
       s_ur[e] = double2{a.x + b.x, a.y + b.y};
       s_ut[e] = ut2;
-      s_ut32[e] = float2{0.5f * (float)ut2.x, 0.5f * (float)ut2.y};
+      s_ut32[e] = float2{0.5f * to_float(ut2.x), 0.5f * to_float(ut2.y)};
     } else {
       s_ur[e] = double2{0.5 * (a.x + b.x), 0.5 * (a.y + b.y)};
       s_ut[e] = double2{0.5 * (a.y - b.y), -0.5 * (a.x - b.x)};
@@ -598,6 +599,9 @@ void launch_product(const Dims& d, const DevSetup& s, const FftPlan& pth, const 
 }
 
 // ------------------------------------------------------------------ z analysis (A4)
+__device__ __forceinline__ double wide(double x) { return x; }
+__device__ __forceinline__ double wide(float x) { return to_double(x); }
+
 template <typename V, int NZ>
 __global__ void __launch_bounds__(256) k_zanalysis(Dims d, FftPlan pz, const V* __restrict__ twz,
                                                    const V* __restrict__ ZN, const double2* __restrict__ Nlin,
@@ -670,9 +674,9 @@ __global__ void __launch_bounds__(256) k_zanalysis(Dims d, FftPlan pz, const V* 
     const int zp = k < 0 ? k + nz : k;
     const V r_ = res[(0 * MC + mc) * ld + zp], t_ = res[(1 * MC + mc) * ld + zp];
     const V z_ = res[(2 * MC + mc) * ld + zp];
-    double2 np = double2{(double)(sc * (r_.x - t_.y)), (double)(sc * (r_.y + t_.x))};  // N+ = N_r + i N_theta
-    double2 nm = double2{(double)(sc * (r_.x + t_.y)), (double)(sc * (r_.y - t_.x))};  // N- = N_r - i N_theta
-    double2 nz2 = double2{(double)(sc * z_.x), (double)(sc * z_.y)};
+    double2 np = double2{wide(sc * (r_.x - t_.y)), wide(sc * (r_.y + t_.x))};  // N+ = N_r + i N_theta
+    double2 nm = double2{wide(sc * (r_.x + t_.y)), wide(sc * (r_.y - t_.x))};  // N- = N_r - i N_theta
+    double2 nz2 = double2{wide(sc * z_.x), wide(sc * z_.y)};
     if (k == 0 && m == 0) nz2.x += 4.0 / Re;  // base driving force (laminar balance)
     const long o = ((long)m * d.N + n) * nk + kk;
     if (Nlin || d.forcing) {
@@ -901,9 +905,9 @@ __global__ void __launch_bounds__(256) k_nl_fused32(Dims d, int C, const float2*
     const int zp = k < 0 ? k + NZ : k;
     const V r_ = res3[(0 * MC + mc) * LDZ + zp], t_ = res3[(1 * MC + mc) * LDZ + zp];
     const V z_ = res3[(2 * MC + mc) * LDZ + zp];
-    double2 np = double2{(double)(sc * (r_.x - t_.y)), (double)(sc * (r_.y + t_.x))};  // N+ = N_r + i N_theta
-    double2 nm = double2{(double)(sc * (r_.x + t_.y)), (double)(sc * (r_.y - t_.x))};  // N- = N_r - i N_theta
-    double2 nz2 = double2{(double)(sc * z_.x), (double)(sc * z_.y)};
+    double2 np = double2{wide(sc * (r_.x - t_.y)), wide(sc * (r_.y + t_.x))};  // N+ = N_r + i N_theta
+    double2 nm = double2{wide(sc * (r_.x + t_.y)), wide(sc * (r_.y - t_.x))};  // N- = N_r - i N_theta
+    double2 nz2 = double2{wide(sc * z_.x), wide(sc * z_.y)};
     if (k == 0 && m == 0) nz2.x += 4.0 / Re;  // base driving force (laminar balance)
     const long o = ((long)m * N + n) * nk + kk;
     double2 ap = double2{0.0, 0.0}, am = ap, az = ap;

@@ -43,6 +43,30 @@ void launch_step_kernel(const Dims& d, void (*kern)(KArgs...), dim3 g, dim3 b, s
   cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
+// FP64 <-> FP32 by integer operations: the conversion instructions run on the
+// FP64 unit at its two lanes per clock, these at 64 a clock and more.  Same
+// results; the rare ranges (FP32 subnormals, infinities, NaN) take the
+// instruction.
+__device__ __forceinline__ float to_float(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+  unsigned f = __funnelshift_r(lo, hi, 29) + 0x40000000u;      // exponent less 896 (mod 512)
+  f += ((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29;    // to nearest, ties to even
+  f = (f & 0x7fffffffu) | sign;
+  if (e < 873u) f = sign;                                      // below half of the least subnormal
+  else if (e - 897u > 253u) f = __float_as_uint((float)x);
+  return __uint_as_float(f);
+}
+__device__ __forceinline__ double to_double(float x) {
+  const unsigned f = __float_as_uint(x), e = (f >> 23) & 0xffu;
+  unsigned hi = ((f & 0x7fffffffu) >> 3) + 0x38000000u, lo = f << 29;
+  if (e - 1u > 253u) {
+    if (f << 1) return (double)x;
+    hi = lo = 0u;
+  }
+  return __hiloint2double((int)(hi | (f & 0x80000000u)), (int)lo);
+}
+
 // Batched launches: trajectory b = blockIdx.z; its buffers sit `stride` bytes
 // after trajectory b-1's (stride 0: shared).  Null stays null.
 template <typename P>
