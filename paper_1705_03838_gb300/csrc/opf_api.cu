@@ -60,9 +60,9 @@ struct Group {
   opf::FftPlan pz{}, pth{};
   int nJ = 0;
   bool shared_setup = false;
-  // FP64 steps: W6 holds the curl of U, as the last solve of a step leaves
-  // it; anything else that writes U, W6 or an option clears this, and the
-  // next step then starts with a curl launch
+  // steps whose solves take the curl: W6 holds the curl of U, as the last
+  // solve of a step leaves it; anything else that writes U, W6 or an option
+  // clears this, and the next step then starts with a curl launch
   bool w6_valid = false;
   std::vector<double> Re, dt, time;  // per trajectory
   opf::DevSetup ds;                  // trajectory 0's setup arrays
@@ -82,7 +82,7 @@ struct Group {
   // setup-arena offsets (same for every trajectory), for in-place rebuilds
   size_t o_prm = 0, o_rinv = 0, o_d1 = 0, o_wq = 0, o_hop = 0, o_luH = 0, o_luP = 0;
   size_t o_basis = 0, o_ainv = 0, o_G = 0, o_twz = 0, o_twt = 0, o_twz32 = 0, o_twt32 = 0;
-  size_t o_r = 0, o_d1f = 0;
+  size_t o_r = 0, o_stab = 0;
   size_t o_luH2 = 0, o_luP2 = 0, o_spkH = 0, o_spkP = 0, o_rH = 0, o_rP = 0;
   bool spike_built = false;  // split factors built (decided once, at creation)
   bool spike_default = false;  // the split solve is on unless the option says otherwise
@@ -111,7 +111,7 @@ struct Group {
     s.tw_z32 = sh(s.tw_z32);
     s.tw_th32 = sh(s.tw_th32);
     s.r = sh(s.r);
-    s.d1f = sh(s.d1f);
+    s.stab = (char*)s.stab + o;
     if (spike_built) {
       s.luH2 = sh(s.luH2);
       s.luP2 = sh(s.luP2);
@@ -214,7 +214,7 @@ int group_fill_setups(Group* g, bool first) {
   g->o_twz32 = pl.add(d.nz * sizeof(float2));
   g->o_twt32 = pl.add(d.nth * sizeof(float2));
   g->o_r = pl.add(s0.r.size() * 8);
-  g->o_d1f = pl.add((s0.d1.size() + s0.rinv.size()) * sizeof(float));
+  g->o_stab = pl.add(opf::stencil_bytes(N));
   g->o_luH2 = pl.add(s0.luH2.size() * 8);
   g->o_luP2 = pl.add(s0.luP2.size() * 8);
   g->o_spkH = pl.add(s0.spkH.size() * 8);
@@ -270,9 +270,7 @@ int group_fill_setups(Group* g, bool first) {
     put(g->o_twz32, twz32.data(), d.nz * sizeof(float2));
     put(g->o_twt32, twt32.data(), d.nth * sizeof(float2));
     put(g->o_r, s.r.data(), s.r.size() * 8);
-    std::vector<float> d1f(s.d1.begin(), s.d1.end());  // FP32 stencils, then FP32 1/r
-    d1f.insert(d1f.end(), s.rinv.begin(), s.rinv.end());
-    put(g->o_d1f, d1f.data(), d1f.size() * sizeof(float));
+    opf::stencil_host_table(s.d1.data(), d.N, host.data() + g->o_stab);
     put(g->o_luH2, s.luH2.data(), s.luH2.size() * 8);
     put(g->o_luP2, s.luP2.data(), s.luP2.size() * 8);
     put(g->o_spkH, s.spkH.data(), s.spkH.size() * 8);
@@ -353,7 +351,7 @@ int group_build(Group* g, int N, int K, int M, int m_p, double alpha, int B, con
   g->ds.tw_z32 = (float2*)(P + g->o_twz32);
   g->ds.tw_th32 = (float2*)(P + g->o_twt32);
   g->ds.r = (double*)(P + g->o_r);
-  g->ds.d1f = (float*)(P + g->o_d1f);
+  g->ds.stab = P + g->o_stab;
   if (g->spike_built) {
     g->ds.luH2 = (double*)(P + g->o_luH2);
     g->ds.luP2 = (double*)(P + g->o_luP2);
@@ -488,8 +486,8 @@ void runner_free(Runner* r) {
   r->own = nullptr;
 }
 
-// The curl of U (A1) into the group's W6 (and Nlin in mixed precision);
-// timed: inside the per-kernel event slots.
+// The curl of U (A1) into W6 (and Nlin in mixed precision); timed: inside the
+// per-kernel event slots.
 void enqueue_curl(Runner* r, const Group& g, const double2* U, bool timed = true) {
   if (timed) r->begin(0);
   if (r->precision == 1) opf::launch_curl_split32(g.d, g.ds, U, g.W6f, g.Nlin, r->st());
@@ -531,17 +529,12 @@ void enqueue_nonlinear(Runner* r, const Group& g, const double2* U, double2* Nou
   r->end();
 }
 
-// FP64 steps fuse the curl into the solve: the solve blocks leave the curl
-// of their output in W6 for the next nonlinear evaluation (measured: FP64
-// medium step 441 -> 394 us).  Mixed-precision steps keep the separate split
-// curl: there the fused form cost the solve about as much as the curl launch
-// it saved.
-bool fused_curl(const Runner* r) { return r->precision == 0; }
+bool fused_curl(const Runner* r, const Group& g) { return r->precision == 0 && opf::solve_takes_curl(g.d); }
 
 // Solve pass into Uout (and, fused, the curl of Uout into W6).
 void enqueue_solve(Runner* r, const Group& g, const double2* Na, const double2* Nb, double2* Uout) {
   opf::SolveArgs a{g.U, Na, Nb, Uout, g.beta_p};
-  if (fused_curl(r)) a.W6 = g.W6;
+  if (fused_curl(r, g)) a.W6 = g.W6;
   r->begin(4);
   opf::launch_solve(g.d, g.ds, a, g.nJ, r->st());
   r->end();
@@ -587,9 +580,7 @@ void enqueue_step(Runner* r) {
       cudaStreamWaitEvent(r->cur, r->fork_ev, 0);
     }
     if (g->d.cfl) cudaMemsetAsync(g->cfl, 0, sizeof(double), r->st());
-    // fused: W6 holds the curl of U at the start of a step (runner_step) and
-    // the solves leave the curl of their output
-    const bool curl = !fused_curl(r);
+    const bool curl = !fused_curl(r, *g);  // (else W6 holds the curl of U: runner_step)
     enqueue_nonlinear(r, *g, g->U, g->Nj, curl);
     enqueue_solve(r, *g, g->Nj, nullptr, g->U1);
     if (r->n_corr == 0)  // predictor only: its output (3F per trajectory) is the new state
@@ -753,7 +744,7 @@ int runner_step(Runner* r, int n) {
   for (int s = 0; s < n; ++s) {
     r->nslots = 0;
     for (Group* g : r->groups)
-      if (fused_curl(r) && !g->w6_valid) {  // the step graph starts from the curl of U (untimed)
+      if (fused_curl(r, *g) && !g->w6_valid) {  // the step starts from the curl of U (untimed)
         enqueue_curl(r, *g, g->U, false);
         g->w6_valid = true;
       }
@@ -1011,7 +1002,7 @@ int traj_energy(Group* g, int b, double out[3], cudaStream_t st) {
   const opf::DevSetup s = g->setup_of(b);
   double2* U = g->at(g->U, b);
   double2* W6 = g->at(g->W6, b);
-  g->w6_valid = false;  // FP64 curl of this trajectory only
+  g->w6_valid = false;  // the curl of this trajectory only
   opf::launch_curl(d, s, U, W6, st);
   opf::launch_energy(d, s, U, W6, g->at(g->beta_p, b), g->at(g->partial, b), g->nblk_energy,
                      g->at(g->out3, b), st);

@@ -16,32 +16,6 @@ namespace {
 constexpr int kThreads = 256, kWarps = kThreads / 32;
 
 // ------------------------------------------------------------------ tables
-// Entry (k, n) of a table in fixed point: v(k, n), zero outside K x N.
-#pragma nv_exec_check_disable
-template <class V>
-__host__ __device__ void table_entry(long idx, int KT, V v, uint2* out) {
-  // idx = (nt * KT + kt) * 32 + lane
-  const int lane = (int)(idx % 32), kt = (int)(idx / 32 % KT), nt = (int)(idx / 32 / KT);
-  const int t = lane & 3, n = nt * 8 + (lane >> 2), k0 = kt * 16 + 2 * t;
-  const long long f[4] = {v(k0, n), v(k0 + 1, n), v(k0 + 8, n), v(k0 + 9, n)};
-  for (int i = 0; i < kDig; ++i) {
-    unsigned short h[4];
-    for (int q = 0; q < 4; ++q) {  // a small integer as a half
-      const int d = dft_digit(f[q], i);
-#ifdef __CUDA_ARCH__
-      h[q] = __half_as_ushort(__int2half_rn(d));
-#else
-      const int a = d < 0 ? -d : d;
-      int e = 0;
-      while ((a >> e) > 1) ++e;
-      h[q] = a ? (unsigned short)((d < 0 ? 0x8000 : 0) | ((15 + e) << 10) | ((a << (10 - e)) & 0x3ff)) : 0;
-#endif
-    }
-    out[((long)nt * KT + kt) * kTileB + i * 32 + lane] =
-        make_uint2(h[0] | (unsigned)h[1] << 16, h[2] | (unsigned)h[3] << 16);
-  }
-}
-
 // The eight matrices of a handle, in the order of DftTables.
 struct TableShape {
   int H, n, anal, sine;
@@ -150,6 +124,18 @@ void dft_device_tables(int K, int M, double inv_grid, const double2* twz, const 
   if (most) k_dft_tables<<<dim3((unsigned)((most + 127) / 128), 8), 128, 0, st>>>(jobs);
 }
 
+size_t stencil_bytes(int N) {
+  return (size_t)stencil_table_size(N) * sizeof(uint2) + (size_t)16 * stencil_tiles(N) * sizeof(int);
+}
+StencilTable stencil_at(const void* p, int N) {
+  const uint2* tab = (const uint2*)p;
+  return StencilTable{tab, (const int*)(tab + stencil_table_size(N)), stencil_tiles(N), 8 * stencil_tiles(N) - N};
+}
+void stencil_host_table(const double* d1, int N, void* host) {
+  uint2* tab = (uint2*)host;
+  for (long idx = 0; idx < 64L * stencil_tiles(N); ++idx)
+    stencil_entry(idx, d1, N, tab, (int*)(tab + stencil_table_size(N)));
+}
 // ------------------------------------------------------------------ z synthesis
 // Block: up to 32 m columns of one field and radial row.  A row tile is eight
 // columns: rows 0-7 their real parts, 8-15 the imaginary ones; the sums over

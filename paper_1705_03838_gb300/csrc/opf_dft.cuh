@@ -29,7 +29,9 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdint>
+#include <cstring>
 
 namespace opf {
 
@@ -60,6 +62,96 @@ __host__ __device__ constexpr long dft_anal_size(int H, int n) {
 __host__ __device__ inline int dft_digit(long long v, int i) {
   const unsigned long long y = (unsigned long long)v + 0x0080808080808080ull;
   return (i == 0 ? (int)(y >> 48) : (int)((y >> (8 * (6 - i))) & 255)) - 128;
+}
+
+struct StencilTable {
+  const uint2* tab;  // [parity][tile][digit][lane]
+  const int* ew;     // [parity][8 tiles]
+  int tiles, off;    // row i sits at i + off of the tiles
+};
+StencilTable stencil_at(const void* p, int N);  // p as filled by stencil_host_table
+__host__ __device__ constexpr int stencil_tiles(int N) { return (N + 7) / 8; }
+__host__ __device__ constexpr long stencil_table_size(int N) { return 2L * stencil_tiles(N) * kTileB; }
+// Mesh row of lane t's value q = 0..3 in a tile whose first row is i0.
+__host__ __device__ constexpr int stencil_row(int i0, int t, int q) {
+  return q < 2 ? i0 + 2 * t + q : (t < 2 ? i0 - 4 + 2 * t : i0 + 4 + 2 * t) + q - 2;
+}
+__host__ __device__ inline unsigned long long dft_bits(double x) {
+#ifdef __CUDA_ARCH__
+  return (unsigned long long)__double_as_longlong(x);
+#else
+  unsigned long long b;
+  std::memcpy(&b, &x, sizeof b);
+  return b;
+#endif
+}
+// x in fixed point, rounded to nearest: units of 2^(emax - 1022 - 55 + half),
+// emax the largest biased exponent among the values that share it (200 at
+// least), |result| <= 2^(55 - half); half = 1 leaves room for the sum of two.
+__host__ __device__ inline long long dft_fixed(double x, int emax, int half) {
+  const unsigned long long b = dft_bits(x);
+  const unsigned h = (unsigned)(b >> 32);
+  const int e = (h >> 20) & 0x7ff;
+  const unsigned hm = e ? ((h & 0xfffffu) | 0x100000u) : 0u;
+  const unsigned long long m = ((unsigned long long)hm << 32) | (e ? (unsigned)b : 0u);
+  const int s0 = (emax < 200 ? 200 : emax) - e + half, sh = s0 < 63 ? s0 : 63;
+  const unsigned long long r = (((m << 3) >> sh) + 1) >> 1;
+  return (h & 0x80000000u) ? -(long long)r : (long long)r;
+}
+// Table entry of (parity's) stencils d1 = [N][9]: fixed point of the weight
+// that output row i gives row j, and the largest biased exponent of row i.
+__host__ __device__ inline int stencil_exponent(const double* d1, int i) {
+  int e = 0;
+  for (int q = 0; q < 9; ++q) {
+    const int f = (int)(dft_bits(d1[i * 9 + q]) >> 52) & 0x7ff;
+    e = f > e ? f : e;
+  }
+  return e;
+}
+__host__ __device__ inline long long stencil_weight(const double* d1, int N, int i, int j) {
+  const int lo = i - 4 < 0 ? 0 : (i - 4 > N - 9 ? N - 9 : i - 4);
+  if (i < 0 || i >= N || j < 0 || j >= N || j < lo || j > lo + 8) return 0;
+  return dft_fixed(d1[i * 9 + j - lo], stencil_exponent(d1, i), 0);
+}
+
+// Entry (k, n) of a table in fixed point: v(k, n), zero outside K x N.
+#pragma nv_exec_check_disable
+template <class V>
+__host__ __device__ inline void table_entry(long idx, int KT, V v, uint2* out) {
+  // idx = (nt * KT + kt) * 32 + lane
+  const int lane = (int)(idx % 32), kt = (int)(idx / 32 % KT), nt = (int)(idx / 32 / KT);
+  const int t = lane & 3, n = nt * 8 + (lane >> 2), k0 = kt * 16 + 2 * t;
+  const long long f[4] = {v(k0, n), v(k0 + 1, n), v(k0 + 8, n), v(k0 + 9, n)};
+  for (int i = 0; i < kDig; ++i) {
+    unsigned short h[4];
+    for (int q = 0; q < 4; ++q) {  // a small integer as a half
+      const int d = dft_digit(f[q], i);
+#ifdef __CUDA_ARCH__
+      h[q] = __half_as_ushort(__int2half_rn(d));
+#else
+      const int a = d < 0 ? -d : d;
+      int e = 0;
+      while ((a >> e) > 1) ++e;
+      h[q] = a ? (unsigned short)((d < 0 ? 0x8000 : 0) | ((15 + e) << 10) | ((a << (10 - e)) & 0x3ff)) : 0;
+#endif
+    }
+    out[((long)nt * KT + kt) * kTileB + i * 32 + lane] =
+        make_uint2(h[0] | (unsigned)h[1] << 16, h[2] | (unsigned)h[3] << 16);
+  }
+}
+
+// Entry idx = (parity * tiles + tile) * 32 + lane of the stencil table.
+__host__ __device__ inline void stencil_entry(long idx, const double* d1, int N, uint2* tab, int* ew) {
+  const int NT = stencil_tiles(N), off = 8 * NT - N;
+  const int nt = (int)(idx / 32 % NT), par = (int)(idx / 32 / NT);
+  const double* w = d1 + (long)par * N * 9;
+  // a table of one k tile and NT column tiles: k, n of the tile -> row, weight
+  table_entry(idx % (32L * NT), 1, [=](int k, int n) -> long long {
+    const int i0 = (n >> 3) * 8 - off, t = (k & 7) >> 1, q = (k & 1) + (k >> 3) * 2;
+    return stencil_weight(w, N, i0 + (n & 7), stencil_row(i0, t, q));
+  }, tab + (long)par * NT * kTileB);
+  const int lane = (int)(idx % 32), i = nt * 8 + lane - off;
+  if (lane < 8) ew[(par * NT + nt) * 8 + lane] = i < 0 ? 0 : stencil_exponent(w, i) - 1022;
 }
 
 #ifdef __CUDACC__
@@ -148,18 +240,6 @@ __device__ __forceinline__ double dft_negative(const unsigned (&a)[4], const Dft
 
 __device__ __forceinline__ int dft_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
-// x in fixed point, rounded to nearest: |result| <= 2^(55 - half), half = 1
-// leaves room for the sum of two.  emax as in dft_scale (there shift = half).
-__device__ __forceinline__ long long dft_fixed(double x, int emax, int half) {
-  const unsigned h = (unsigned)__double2hiint(x);
-  const int e = (h >> 20) & 0x7ff;
-  const unsigned hm = e ? ((h & 0xfffffu) | 0x100000u) : 0u;
-  const unsigned long long m = ((unsigned long long)hm << 32) | (e ? (unsigned)__double2loint(x) : 0u);
-  const int sh = min(max(emax, 200) - e + half, 63);
-  const unsigned long long r = (((m << 3) >> sh) + 1) >> 1;
-  return (h & 0x80000000u) ? -(long long)r : (long long)r;
-}
-
 // One fragment register per digit from two neighbouring k (va at the even one):
 // bytes of the offset values, made halves 1024 + byte and brought to -128..128.
 __device__ __forceinline__ void dft_split(long long va, long long vb, unsigned (&out)[kDig]) {
@@ -188,6 +268,98 @@ __device__ __forceinline__ void dft_put(uint4* tile, int lane, const long long (
   dft_split(y[2], y[3], r3);
 #pragma unroll
   for (int i = 0; i < kDig; ++i) tile[i * 32 + lane] = make_uint4(r0[i], r1[i], r2[i], r3[i]);
+}
+
+// ---------------------------------------------------------------- radial stencils
+// The 9-point first derivative of eight complex columns at eight rows, by the
+// same digit products: the rows of the 16 x 16 data tile are the columns' real
+// (0-7) and imaginary (8-15) parts, its k the 16 rows that the eight outputs
+// reach -- k = 0..7 the output rows themselves, 8..15 the four below and the
+// four above, so that a lane's first two values are the points it gets the
+// derivative of.  Rows are counted in tiles of eight back from the wall (the
+// wall rows' shifted stencils then stay within the window); rows outside the
+// mesh have weight zero.  One exponent per column and window, one per row of
+// the stencil.  Nine FP64 multiply-adds per point and part become none.
+//
+// x: this lane's column (lane = 4 g + t) at rows 2t, 2t+1 of the tile, then of
+// its halo (stencil_row); tab: the tile's table plus lane; ew: the exponents
+// of output rows 2t, 2t+1.
+// The window's digits as a fragment, DIG of them; er, ei: the columns' exponents.
+template <int DIG>
+__device__ __forceinline__ void stencil_digits(const double2 (&x)[4], uint4 (&a)[DIG], int* er_out, int* ei_out) {
+  int er = 0, ei = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    er = max(er, dft_exponent(x[q].x));
+    ei = max(ei, dft_exponent(x[q].y));
+  }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    er = max(er, __shfl_xor_sync(0xffffffffu, er, o));
+    ei = max(ei, __shfl_xor_sync(0xffffffffu, ei, o));
+  }
+  unsigned r[kDig];
+  dft_split(dft_fixed(x[0].x, er, 0), dft_fixed(x[1].x, er, 0), r);
+#pragma unroll
+  for (int i = 0; i < DIG; ++i) a[i].x = r[i];
+  dft_split(dft_fixed(x[0].y, ei, 0), dft_fixed(x[1].y, ei, 0), r);
+#pragma unroll
+  for (int i = 0; i < DIG; ++i) a[i].y = r[i];
+  dft_split(dft_fixed(x[2].x, er, 0), dft_fixed(x[3].x, er, 0), r);
+#pragma unroll
+  for (int i = 0; i < DIG; ++i) a[i].z = r[i];
+  dft_split(dft_fixed(x[2].y, ei, 0), dft_fixed(x[3].y, ei, 0), r);
+#pragma unroll
+  for (int i = 0; i < DIG; ++i) a[i].w = r[i];
+  *er_out = er;
+  *ei_out = ei;
+}
+template <int DIG, int LEV>
+__device__ __forceinline__ void stencil_products(const uint4 (&a)[DIG], const uint2* __restrict__ tab,
+                                                 float (&acc)[LEV][4]) {
+#pragma unroll
+  for (int l = 0; l < LEV; ++l)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[l][q] = kDftBias;
+#pragma unroll
+  for (int j = 0; j < DIG; ++j) {
+    const uint2 b = __ldg(tab + j * 32);
+#pragma unroll
+    for (int i = 0; i < DIG; ++i)
+      if (i + j < LEV) dft_mma(acc[i + j], a[i], b);
+  }
+}
+__device__ __forceinline__ void dft_stencil(const double2 (&x)[4], const uint2* __restrict__ tab, int ew0, int ew1,
+                                            double2 (&out)[2]) {
+  uint4 a[kDig];
+  float acc[kLev][4];
+  int er, ei;
+  stencil_digits<kDig>(x, a, &er, &ei);
+  stencil_products<kDig, kLev>(a, tab, acc);
+  unsigned w[4][kLev / 2];
+  dft_pairs(acc, w);
+  out[0] = double2{dft_value(w[0], dft_scale(er, ew0)), dft_value(w[2], dft_scale(ei, ew0))};
+  out[1] = double2{dft_value(w[1], dft_scale(er, ew1)), dft_value(w[3], dft_scale(ei, ew1))};
+}
+// The same to FP32: five digits and levels are 2^-39 of the largest term.
+__device__ __forceinline__ void dft_stencil32(const double2 (&x)[4], const uint2* __restrict__ tab, int ew0, int ew1,
+                                              float2 (&out)[2]) {
+  constexpr int kD = 5;
+  uint4 a[kD];
+  float acc[kD][4];
+  int er, ei;
+  stencil_digits<kD>(x, a, &er, &ei);
+  stencil_products<kD, kD>(a, tab, acc);
+  auto value = [&](int q, int emax, int shift) {  // in units of level 3, 2^(e - 38)
+    const unsigned hi = (unsigned)__float_as_int(acc[0][q]) * 256u + (unsigned)__float_as_int(acc[1][q]) - kDftPair;
+    const unsigned lo = (unsigned)__float_as_int(acc[2][q]) * 256u + (unsigned)__float_as_int(acc[3][q]) - kDftPair;
+    const int low = (int)lo + (__float_as_int(acc[4][q]) - __float_as_int(kDftBias) + 128 >> 8);
+    const int e = max(emax, 200) - 1022 + shift - 38 + 127;
+    const float s = emax >= 1900 ? __int_as_float(0x7fc00000) : e > 0 ? __int_as_float(min(e, 254) << 23) : 0.f;
+    return fmaf((float)(int)hi, 65536.f, (float)low) * s;
+  };
+  out[0] = float2{value(0, er, ew0), value(2, ei, ew0)};
+  out[1] = float2{value(1, er, ew1), value(3, ei, ew1)};
 }
 #endif  // __CUDACC__
 

@@ -88,7 +88,7 @@ struct DevSetup {
   float2* tw_z32 = nullptr;
   float2* tw_th32 = nullptr;
   double* r = nullptr;    // radial points (null where the split curl is not used)
-  float* d1f = nullptr;   // d1 in FP32, then 1/r in FP32 ([2][N][9] + [N])
+  void* stab = nullptr;   // digit table of d1 (stencil_bytes)
   // two-partition (split) solve data (Setup::luH2 ...; null unless built)
   double *luH2 = nullptr, *luP2 = nullptr, *spkH = nullptr, *spkP = nullptr, *rH = nullptr, *rP = nullptr;
 };
@@ -179,6 +179,9 @@ void dft_host_tables(int K, int M, double inv_grid, void* host, void* dev, DftTa
 void dft_device_tables(int K, int M, double inv_grid, const double2* twz, const double2* twth, void* dev,
                        DftTables* t, cudaStream_t st);
 bool dft_prepare_attrs();
+// Digit table of the first-derivative stencils d1 ([2][N][9]), for the curl.
+size_t stencil_bytes(int N);
+void stencil_host_table(const double* d1, int N, void* host);
 void launch_dft_zsynth(const Dims& d, const DevSetup& s, const double2* W6, double2* Z6, cudaStream_t st);
 void launch_dft_product(const Dims& d, const DevSetup& s, const double2* Z6, double2* ZN, cudaStream_t st);
 void launch_dft_zanalysis(const Dims& d, const DevSetup& s, const double2* ZN, double2* Nout, cudaStream_t st);
@@ -188,10 +191,9 @@ struct SolveArgs {
   const double2* Nb;  // null: N_eff = N_a, else (N_a + N_b) / 2
   double2* Uout;
   double* beta_p;  // device scalar: beta' of this solve (written by the (0,0) mode)
-  // FP64 curl of the solved state for the next nonlinear evaluation, computed
-  // by the same blocks from their radial columns (null: none)
-  double2* W6 = nullptr;
+  double2* W6 = nullptr;  // the FP64 curl of the solved state too (null: no; see solve_takes_curl)
 };
+bool solve_takes_curl(const Dims& d);  // FP64 steps: the solve leaves the curl of its output
 void launch_solve(const Dims& d, const DevSetup& s, const SolveArgs& a, int nJ, cudaStream_t st);
 void launch_energy(const Dims& d, const DevSetup& s, const double2* U, const double2* W6,
                    const double* beta_p, double* partial, int nblk, double* out3, cudaStream_t st);

@@ -120,255 +120,168 @@ void launch_internal_to_abi(const Dims& d, const double2* U, double2* abi, int, 
 }
 
 // ------------------------------------------------------------------ curl (A1)
-// The radial columns of a trajectory -- column (m, kk), all N rows -- are
-// split into contiguous runs of whole columns, one per block (their count
-// differing by at most one between blocks).  A block stages its columns --
-// each u+-, u_z value read once, u_r and u_theta formed in FP64 -- in shared
-// memory, and the 9-point radial stencils read their neighbours from there.
-// Threads take the block's points row by row with the columns innermost, so
-// that a warp's stencil rows are shared by the lanes of one row and its
-// stores run along k.  Columns per block: on a grid of a few waves, the
-// count that puts the fewest warp-passes on the busiest SM (then the most
-// resident warps; the grid of four columns per block of a one-wave medium
-// trajectory left a third of the SMs' time idle), else four.
+// One warp per item of eight modes (consecutive k at one m) and eight radial
+// rows: a lane holds a mode's u+-, u_z at two of the rows and at two of the
+// halo's, the radial derivatives of u_z and u_theta are digit products on the
+// tensor cores (dft_stencil), and everything else is pointwise in the lane.
+// Nothing passes through shared memory and warps are independent; the rows of
+// neighbouring items come from L1 again.
 //
 // SPLIT (mixed precision): the laminar base flow U = (1 - r^2) z,
 // Omega = 2r theta is removed in FP64 (W6 then holds u', w' in FP32), and the
 // terms linear in the perturbation, U x w' + u' x Omega (+ U x Omega on
 // (0,0)), are evaluated here per mode in FP64 -- they are diagonal in r -- and
-// written to Nlin in +- form.  FP64 arithmetic is kept to what Nlin needs (the
-// u_z derivative, w_r, w_theta); the u_theta derivative feeds only w_z, which
-// goes to the FP32 product, and is taken in FP32 from an FP32 copy of the
-// u_theta tile.  The factor 1/2 of u_r = (u+ + u-)/2 and
-// u_theta = (u+ - u-)/(2i) goes into the constants that multiply them (exact
-// scalings by two, so the results are those of the halved values).  Without
-// SPLIT everything is FP64.
-constexpr int kCurlThreads = 128;
+// written to Nlin in +- form.  FP64 arithmetic is kept to what Nlin needs
+// (w_r, w_theta); w_z goes to the FP32 product only and is put together in
+// FP32.  The factor 1/2 of u_r = (u+ + u-)/2 and u_theta = (u+ - u-)/(2i) goes
+// into the constants that multiply them (exact scalings by two).
+//
+// What bounds it: the FP64 unit, with ~27 FP64 instructions per point left of
+// 57, then the integer units.  Against stencils as FP64 multiply-adds on
+// columns staged in shared memory (whose loads of data and weights took about
+// as long), split curl per launch: N = 128, 255 x 128 modes 440 -> 242 us,
+// groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 57 -> 35 us, N = 48,
+// 63 x 24 modes 14.8 -> 12.4 us.
+constexpr int kCurlWarps = 4;
 
-// Blocks per trajectory and the most columns one block takes.
-struct CurlShape {
-  int nbx, kc;
-};
-static CurlShape curl_shape(const Dims& d) {
-  const long sms = device_sms();
-  const long cols = (long)d.M * d.nk, B = d.B > 0 ? d.B : 1, N = d.N;
-  const long warps_max = kCurlThreads / 32;
-  long cpb = 4;
-  if ((cols + 3) / 4 * B <= 8 * sms) {
-    long best_cost = -1, best_conc = 0;
-    for (long c = 1; c <= 16 && c <= cols; ++c) {
-      const long w = (c * N + 31) / 32;  // warp-passes of a block
-      if (c * N < 32 || w > 4 * warps_max) continue;
-      const long per_sm = ((cols + c - 1) / c * B + sms - 1) / sms;
-      const long cost = per_sm * w, conc = per_sm * std::min(w, warps_max);
-      if (best_cost < 0 || cost < best_cost || (cost == best_cost && conc > best_conc)) {
-        best_cost = cost;
-        best_conc = conc;
-        cpb = c;
-      }
-    }
-  }
-  cpb = std::min(cpb, cols);
-  const long nbx = (cols + cpb - 1) / cpb;
-  return CurlShape{(int)nbx, (int)((cols + nbx - 1) / nbx)};
+// The (0,0) mode of the split curl: the base flow is taken off u_z and w_theta.
+__device__ __noinline__ void curl_mean(double Ub, double Ob, double2 uz, double wtx, double wty, long fs, long w,
+                                       float2* W6, double2* Nlin) {
+  const double uzx = uz.x - Ub;
+  wtx -= Ob;
+  const double2 nr = double2{-Ub * wtx - Ob * uzx - Ub * Ob, -Ub * wty - Ob * uz.y};  // (w_r is zero)
+  Nlin[w] = nr;
+  Nlin[fs + w] = nr;
+  W6[2 * fs + w].x = (float)uzx;
+  W6[4 * fs + w].x = (float)wtx;
+}
+// Coriolis force of the base flow on (k, m~) = (0, 1): N- gains -2 U (Omega_y + i Omega_x).
+__device__ __noinline__ void curl_rotation(double Ub, double rot_x, double rot_y, double2* nminus) {
+  const double2 n = *nminus;
+  *nminus = double2{n.x - 2.0 * Ub * rot_y, n.y - 2.0 * Ub * rot_x};
 }
 
-size_t curl_smem(const Dims& d) {
-  const size_t kc = (size_t)curl_shape(d).kc, N = (size_t)d.N;
-  return N * kc * (3 * sizeof(double2) + sizeof(float2)) + kc * sizeof(double) + 2 * N * sizeof(double) +
-         2 * kc * sizeof(int);
-}
-
-// One grid point (m, kk, radial row n) of A1 from the radial column of its
-// mode: uz_at(i), ut_at(i) (FP64) and ut32_at(i) (FP32, SPLIT) give u_z and
-// u_theta at row i; ur, ut, uz are the point's own values; ak = alpha k.
-// SPLIT with SUMS: ur and ut are 2 u_r and 2 u_theta, ak is alpha k / 2, and
-// Ub, Ob are U = 1 - r^2 and Omega = 2r at the point's row (else formed
-// here from r).  d1 = [2][N][9] stencils, d1f =
-// the FP32 stencils then FP32 1/r, rr and rinv the radial points and their
-// inverses (all of this trajectory).  Writes the six W6 components (and,
-// SPLIT, the FP64 linear terms Nlin in +- form).
-template <typename V, bool SPLIT, bool SUMS = false, typename UzAt, typename UtAt, typename Ut32At>
-__device__ __forceinline__ void curl_point(const Dims& d, int m, int kk, int n, double ak,
-                                           const double* __restrict__ d1, const float* __restrict__ d1f,
-                                           const double* __restrict__ rr, const double* __restrict__ rinv,
-                                           UzAt uz_at, UtAt ut_at, Ut32At ut32_at, double2 ur, double2 ut,
-                                           double2 uz, V* __restrict__ W6, double2* __restrict__ Nlin,
-                                           double Ub = 0.0, double Ob = 0.0) {
-  using T = typename Scalar<V>::T;
-  const int N = d.N, nk = d.nk;
-  const long fs = d.F;
-  const int mt = d.m_p * m;
-  const int ps = mt & 1, pv = ps ^ 1;
-  const int lo = row_lo_d(n, N);
-  const double* ws = d1 + ((long)ps * N + n) * 9;
-  double dzx = 0, dzy = 0;  // d/dr of u_z (FP64)
-  T dtx = 0, dty = 0;       // d/dr of u_theta
-  if constexpr (SPLIT) {
-    const float* wv = d1f + ((long)pv * N + n) * 9;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      const double2 z = uz_at(lo + q);
-      const float2 t = ut32_at(lo + q);
-      dzx = fma(ws[q], z.x, dzx);
-      dzy = fma(ws[q], z.y, dzy);
-      dtx = fmaf(wv[q], t.x, dtx);
-      dty = fmaf(wv[q], t.y, dty);
-    }
-  } else {
-    const double* wv = d1 + ((long)pv * N + n) * 9;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      const double2 z = uz_at(lo + q), t = ut_at(lo + q);
-      dzx = fma(ws[q], z.x, dzx);
-      dzy = fma(ws[q], z.y, dzy);
-      dtx = fma(wv[q], t.x, dtx);
-      dty = fma(wv[q], t.y, dty);
-    }
-  }
-  const double ri = rinv[n];
-  const double mri = mt * ri;
-  // w_r = i (m~ u_z / r - ak u_theta)
-  const double xr = mri * uz.x - ak * ut.x, xi = mri * uz.y - ak * ut.y;
-  // w_theta = i ak u_r - d_r u_z
-  double wtx = -ak * ur.y - dzx, wty = ak * ur.x - dzy;
-  const long w = ((long)m * N + n) * nk + kk;
-  double uzx = uz.x;
-  if constexpr (SPLIT) {
-    if constexpr (!SUMS) {
-      const double r = rr[n];
-      Ub = 1.0 - r * r;
-      Ob = 2.0 * r;
-    }
-    const bool mean = (m == 0 && kk == d.K - 1);
-    if (mean) {
-      uzx -= Ub;
-      wtx -= Ob;
-    }
-    // N_r = -U w'_t - Omega u'_z, N_t = U w'_r, N_z = Omega u'_r
-    double nrx = -Ub * wtx - Ob * uzx, nry = -Ub * wty - Ob * uz.y;
-    if (mean) nrx -= Ub * Ob;
-    const double ntx = Ub * (-xi), nty = Ub * xr;
-    Nlin[w] = double2{nrx - nty, nry + ntx};
-    double2 nminus = double2{nrx + nty, nry - ntx};
-    if (d.rotate && mt == 1 && kk == d.K - 1) {  // Coriolis force of U z: N- = -2 U (Omega_y + i Omega_x)
-      nminus.x -= 2.0 * Ub * d.rot_y;
-      nminus.y -= 2.0 * Ub * d.rot_x;
-    }
-    Nlin[fs + w] = nminus;
-    if constexpr (SUMS) {
-      const double r = rr[n];  // Omega u_r = r (2 u_r)
-      Nlin[2 * fs + w] = double2{r * ur.x, r * ur.y};
-    } else {
-      Nlin[2 * fs + w] = double2{Ob * ur.x, Ob * ur.y};
-    }
-    // w_z = d_r u_theta + u_theta / r - i m~ u_r / r, in FP32
-    const float ri32 = d1f[2 * 9 * N + n], mri32 = (float)mt * ri32;
-    const float2 ut32 = ut32_at(n);
-    const float half = SUMS ? 0.5f : 1.f;
-    const float urx = half * to_float(ur.x), ury = half * to_float(ur.y);
-    W6[0 * fs + w] = float2{urx, ury};
-    W6[1 * fs + w] = ut32;
-    W6[2 * fs + w] = float2{to_float(uzx), to_float(uz.y)};
-    W6[3 * fs + w] = float2{-to_float(xi), to_float(xr)};
-    W6[4 * fs + w] = float2{to_float(wtx), to_float(wty)};
-    W6[5 * fs + w] = float2{fmaf(mri32, ury, fmaf(ri32, ut32.x, dtx)), fmaf(-mri32, urx, fmaf(ri32, ut32.y, dty))};
-  } else {
-    W6[0 * fs + w] = ur;
-    W6[1 * fs + w] = ut;
-    W6[2 * fs + w] = uz;
-    W6[3 * fs + w] = V{-xi, xr};
-    W6[4 * fs + w] = V{wtx, wty};
-    W6[5 * fs + w] = V{dtx + ri * ut.x + mri * ur.y, dty + ri * ut.y - mri * ur.x};
-  }
-}
-
-// kc: the most columns of a block (curl_shape), the shared-memory size.
 template <typename V, bool SPLIT>
-__global__ void __launch_bounds__(kCurlThreads) k_curl(Dims d, int kc, const double* __restrict__ d1,
-                                                       const float* __restrict__ d1f, const double* __restrict__ rr,
-                                                       const double* __restrict__ rinv,
-                                                       const double2* __restrict__ U, V* __restrict__ W6,
-                                                       double2* __restrict__ Nlin) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int N = d.N, nk = d.nk;
-  double2* s_uz = (double2*)smraw;            // [N][ncb] u_z
-  double2* s_ur = s_uz + N * kc;              // [N][ncb] u_r (SPLIT: 2 u_r)
-  double2* s_ut = s_ur + N * kc;              // [N][ncb] u_theta (SPLIT: 2 u_theta)
-  float2* s_ut32 = (float2*)(s_ut + N * kc);  // [N][ncb] u_theta in FP32 (SPLIT)
-  double* s_ak = (double*)(s_ut32 + N * kc);  // [ncb] alpha k of the columns (SPLIT: alpha k / 2)
-  double* s_ub = s_ak + kc;                   // [N] U = 1 - r^2 (SPLIT)
-  double* s_ob = s_ub + N;                    // [N] Omega = 2r (SPLIT)
-  int* s_m = (int*)(s_ob + N);                // [ncb] m of the columns
-  int* s_kk = s_m + kc;                       // [ncb] kk of the columns
-  d1 = bofs(d1, d.ps);
-  d1f = bofs(d1f, d.ps);
+__global__ void __launch_bounds__(kCurlWarps * 32, 4)
+    k_curl(Dims d, StencilTable st, double ah, const double* __restrict__ rr, const double* __restrict__ rinv,
+           const double2* __restrict__ U, V* __restrict__ W6, double2* __restrict__ Nlin) {
+  const int N = d.N, nk = d.nk, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int G = (nk + 7) / 8;
+  long item = (long)blockIdx.x * kCurlWarps + (threadIdx.x >> 5);
+  grid_dep_trigger_at(d, 1);
+  if (item >= (long)d.M * G * st.tiles) return;
+  const int nt = (int)(item % st.tiles);
+  item /= st.tiles;
+  const int kk = (int)(item % G) * 8 + g, m = (int)(item / G);
+  const bool in = kk < nk;
+  st.tab = bofs(st.tab, d.ps);
+  st.ew = bofs(st.ew, d.ps);
   rr = bofs(rr, d.ps);
   rinv = bofs(rinv, d.ps);
   U = bofs(U, d.ss);
   W6 = bofs(W6, d.ss);
   Nlin = bofs(Nlin, d.ss);
-  const long fs = d.F, cols = (long)d.M * nk;
-  const int col0 = (int)((long)blockIdx.x * cols / gridDim.x);
-  const int ncb = (int)((long)(blockIdx.x + 1) * cols / gridDim.x) - col0;  // this block's columns, <= kc
-  grid_dep_trigger_at(d, 1);
-  if (ncb <= 0) return;
-  for (int c = threadIdx.x; c < ncb; c += blockDim.x) {
-    const int col = col0 + c, m = col / nk, kk = col - m * nk;
-    s_m[c] = m;
-    s_kk[c] = kk;
-    const double ak = d.alpha * (kk - (d.K - 1));
-    s_ak[c] = SPLIT ? 0.5 * ak : ak;
-  }
-  if constexpr (SPLIT)
-    for (int n = threadIdx.x; n < N; n += blockDim.x) {
-      const double r = rr[n];
-      s_ub[n] = 1.0 - r * r;
-      s_ob[n] = 2.0 * r;
-    }
-  __syncthreads();
+  const long fs = d.F;
+  const int i0 = nt * 8 - st.off, mt = d.m_p * m, ps = mt & 1, pv = ps ^ 1;
+  const long col = (long)m * N * nk + kk;
   grid_dep_wait();
-  for (int e = threadIdx.x; e < N * ncb; e += blockDim.x) {
-    const int n = e / ncb, c = e - n * ncb;
-    const long o = ((long)s_m[c] * N + n) * nk + s_kk[c];
-    const double2 a = U[o], b = U[fs + o];
-    s_uz[e] = U[2 * fs + o];
-    if constexpr (SPLIT) {
-      const double2 ut2 = double2{a.y - b.y, b.x - a.x};
-      s_ur[e] = double2{a.x + b.x, a.y + b.y};
-      s_ut[e] = ut2;
-      s_ut32[e] = float2{0.5f * to_float(ut2.x), 0.5f * to_float(ut2.y)};
-    } else {
-      s_ur[e] = double2{0.5 * (a.x + b.x), 0.5 * (a.y + b.y)};
-      s_ut[e] = double2{0.5 * (a.y - b.y), -0.5 * (a.x - b.x)};
+  double2 uz[4], ut[4], ur[2];  // u_z; 2 u_theta; 2 u_r
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = stencil_row(i0, t, q);
+    uz[q] = ut[q] = double2{0.0, 0.0};
+    if (q < 2) ur[q] = uz[q];
+    if (in && i >= 0 && i < N) {
+      const double2 a = U[col + (long)i * nk], b = U[fs + col + (long)i * nk];
+      uz[q] = U[2 * fs + col + (long)i * nk];
+      ut[q] = double2{a.y - b.y, b.x - a.x};
+      if (q < 2) ur[q] = double2{a.x + b.x, a.y + b.y};
     }
   }
-  __syncthreads();
-  grid_dep_trigger_at(d, 2);
-  for (int e = threadIdx.x; e < N * ncb; e += blockDim.x) {
-    const int n = e / ncb, c = e - n * ncb;
-    const double2 *cz = s_uz + c, *ct = s_ut + c;
-    const float2* ct32 = s_ut32 + c;
-    curl_point<V, SPLIT, true>(
-        d, s_m[c], s_kk[c], n, s_ak[c], d1, d1f, rr, rinv, [=](int i) { return cz[i * ncb]; },
-        [=](int i) { return ct[i * ncb]; }, [=](int i) { return ct32[i * ncb]; }, s_ur[e], s_ut[e], s_uz[e], W6,
-        Nlin, SPLIT ? s_ub[n] : 0.0, SPLIT ? s_ob[n] : 0.0);
+  double2 dz[2];  // d/dr of u_z and u_theta
+  V dt[2];
+  {
+    const int* ez = st.ew + (ps * st.tiles + nt) * 8 + 2 * t;
+    const int* et = st.ew + (pv * st.tiles + nt) * 8 + 2 * t;
+    dft_stencil(uz, st.tab + (long)(ps * st.tiles + nt) * kTileB + lane, ez[0], ez[1], dz);
+    const uint2* tt = st.tab + (long)(pv * st.tiles + nt) * kTileB + lane;
+    if constexpr (SPLIT) dft_stencil32(ut, tt, et[0] - 1, et[1] - 1, dt);
+    else dft_stencil(ut, tt, et[0] - 1, et[1] - 1, dt);
   }
+  grid_dep_trigger_at(d, 2);
+  if (!in) return;
+  const double akh = ah * (kk - (d.K - 1));  // alpha k / 2
+  const double mtd = mt;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = i0 + 2 * t + q;
+    if (i < 0) continue;
+    const double ri = rinv[i], mri = mtd * ri;
+    // w_r = i (m~ u_z / r - ak u_theta)
+    const double xr = fma(mri, uz[q].x, -akh * ut[q].x), xi = fma(mri, uz[q].y, -akh * ut[q].y);
+    // w_theta = i ak u_r - d_r u_z
+    const double wtx = fma(-akh, ur[q].y, -dz[q].x), wty = fma(akh, ur[q].x, -dz[q].y);
+    const long w = col + (long)i * nk;
+    if constexpr (SPLIT) {
+      const double r = rr[i], Ub = fma(-r, r, 1.0), Ob = __hiloint2double(__double2hiint(r) + 0x100000, __double2loint(r));
+      // N_r = -U w'_t - Omega u'_z, N_t = U w'_r, N_z = Omega u'_r
+      const double nrx = fma(-Ub, wtx, -Ob * uz[q].x), nry = fma(-Ub, wty, -Ob * uz[q].y);
+      // N- = N_r - i N_t, N+ = N_r + i N_t, N_t = U (-xi + i xr)
+      Nlin[w] = double2{fma(-Ub, xr, nrx), fma(-Ub, xi, nry)};
+      Nlin[fs + w] = double2{fma(Ub, xr, nrx), fma(Ub, xi, nry)};
+      Nlin[2 * fs + w] = double2{r * ur[q].x, r * ur[q].y};  // Omega u_r = r (2 u_r)
+      const double v[11] = {ur[q].x, ur[q].y, ut[q].x, ut[q].y, uz[q].x, uz[q].y, xi, xr, wtx, wty, ri};
+      float f[11];
+      bool rare = false;
+#pragma unroll
+      for (int u = 0; u < 11; ++u) f[u] = to_float(v[u], &rare);
+      if (rare) {
+#pragma unroll
+        for (int u = 0; u < 11; ++u) f[u] = (float)v[u];
+      }
+      // w_z = d_r u_theta + u_theta / r - i m~ u_r / r, in FP32
+      const float mri32 = (float)mt * f[10];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) f[u] *= 0.5f;
+      W6[0 * fs + w] = float2{f[0], f[1]};
+      W6[1 * fs + w] = float2{f[2], f[3]};
+      W6[2 * fs + w] = float2{f[4], f[5]};
+      W6[3 * fs + w] = float2{-f[6], f[7]};
+      W6[4 * fs + w] = float2{f[8], f[9]};
+      W6[5 * fs + w] = float2{fmaf(mri32, f[1], fmaf(f[10], f[2], dt[q].x)),
+                              fmaf(-mri32, f[0], fmaf(f[10], f[3], dt[q].y))};
+      // the few modes with a term of their own, kept out of the others' way
+      if (kk == d.K - 1) {
+        if (m == 0) curl_mean(Ub, Ob, uz[q], wtx, wty, fs, w, (float2*)W6, Nlin);
+        if (d.rotate && mt == 1) curl_rotation(Ub, d.rot_x, d.rot_y, Nlin + fs + w);
+      }
+    } else {
+      const double2 u = double2{halved(ur[q].x), halved(ur[q].y)}, v = double2{halved(ut[q].x), halved(ut[q].y)};
+      W6[0 * fs + w] = u;
+      W6[1 * fs + w] = v;
+      W6[2 * fs + w] = uz[q];
+      W6[3 * fs + w] = V{-xi, xr};
+      W6[4 * fs + w] = V{wtx, wty};
+      W6[5 * fs + w] = V{fma(mri, u.y, fma(ri, v.x, dt[q].x)), fma(-mri, u.x, fma(ri, v.y, dt[q].y))};
+    }
+  }
+}
+
+template <typename V, bool SPLIT>
+static void launch_curl_as(const Dims& d, const DevSetup& s, const double2* U, V* W6, double2* Nlin, cudaStream_t st) {
+  const StencilTable tab = stencil_at(s.stab, d.N);
+  const long items = (long)d.M * ((d.nk + 7) / 8) * tab.tiles;
+  launch_step_kernel(d, k_curl<V, SPLIT>, dim3((unsigned)((items + kCurlWarps - 1) / kCurlWarps), 1, d.B),
+                     dim3(kCurlWarps * 32), 0, st, d, tab, 0.5 * d.alpha, (const double*)s.r, (const double*)s.rinv, U, W6, Nlin);
 }
 
 void launch_curl(const Dims& d, const DevSetup& s, const double2* U, double2* W6, cudaStream_t st) {
-  const CurlShape c = curl_shape(d);
-  launch_step_kernel(d, k_curl<double2, false>, dim3(c.nbx, 1, d.B), dim3(kCurlThreads), curl_smem(d), st, d,
-                     c.kc, (const double*)s.d1, (const float*)nullptr, (const double*)nullptr,
-                     (const double*)s.rinv, U, W6, (double2*)nullptr);
+  launch_curl_as<double2, false>(d, s, U, W6, nullptr, st);
 }
 
-void launch_curl_split32(const Dims& d, const DevSetup& s, const double2* U, float2* W6,
-                         double2* Nlin, cudaStream_t st) {
-  const CurlShape c = curl_shape(d);
-  launch_step_kernel(d, k_curl<float2, true>, dim3(c.nbx, 1, d.B), dim3(kCurlThreads), curl_smem(d), st, d,
-                     c.kc, (const double*)s.d1, (const float*)s.d1f, (const double*)s.r,
-                     (const double*)s.rinv, U, W6, Nlin);
+void launch_curl_split32(const Dims& d, const DevSetup& s, const double2* U, float2* W6, double2* Nlin,
+                         cudaStream_t st) {
+  launch_curl_as<float2, true>(d, s, U, W6, Nlin, st);
 }
 
 // Threads per block of the transform kernels: 256 for grids of at most four
@@ -1021,13 +934,6 @@ struct SolveDev {
   const double* rP;
 };
 
-// x / 2 by its exponent (an FP64 multiplication takes as long as an addition).
-__device__ __forceinline__ double halved(double x) {
-  const int hi = __double2hiint(x);
-  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
-  return e - 2u < 0x7fdu ? __hiloint2double(hi - 0x100000, __double2loint(x)) : 0.5 * x;
-}
-
 // Bulk L2 prefetch by the TMA unit: p 16-byte aligned, bytes a multiple of 16.
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
@@ -1250,8 +1156,8 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   constexpr int NP = (SP ? 16 : 8) * T;    // threads of the pressure substitution (2T chains)
   // X holds N_eff first (chain layout: field f, mode mi, re/im part), then
   // the velocity right-hand sides built on it in place, then the chains'
-  // solutions; S and P are reused by the influence step and the curl.
-  double2* S = (double2*)smraw;                // [N][T]     N+ + N- (later u_j near the wall, u_r)
+  // solutions; S is reused by the influence step.
+  double2* S = (double2*)smraw;                // [N][T]     N+ + N- (later u_j near the wall)
   double2* P = S + N * T;                      // [N][T]     pressure (later u_theta)
   double2* coef = P + N * T;                   // [T]        influence coefficients
   double* X = (double*)(coef + T);             // [N][6T]    N_eff -> right-hand sides -> velocity chains
@@ -1292,7 +1198,6 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     s.rH = bofs(s.rH, d.ps);
     s.rP = bofs(s.rP, d.ps);
   }
-  a.W6 = bofs(a.W6, d.ss);
   a.Uj = bofs(a.Uj, d.ss);
   a.Na = bofs(a.Na, d.ss);
   a.Nb = bofs(a.Nb, d.ss);
@@ -1553,32 +1458,46 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     if (has_mean && c == cz) v += bp * s.G[i];
     double* out = (double*)(a.Uout + f * fs + base + (long)i * nk + kk0 + mi) + part;
     *out = v;
-    if (a.W6) X[i * NT + c] = v;  // (only this element's own X is read above)
+    if (T == 4 && a.W6) X[i * NT + c] = v;  // (only this element's own X is read above)
   }
 
-  // ---- the curl of the new state (A1) for the next nonlinear evaluation, from
-  //      the block's radial columns (S and P are free: u_r, u_theta).  FP64
-  //      steps only: mixed ones take it from k_curl.
-  if (a.W6) {
+  // ---- FP64 steps on grids of at most a block per SM: the curl (A1) of the
+  //      new state for the next nonlinear evaluation from the block's radial
+  //      columns.  There the time is latency: a curl launch of its own took
+  //      3 us longer per pass at N = 32, 31 x 16 modes (on larger grids it is
+  //      the faster form).
+  if (T == 4 && a.W6) {
+    a.W6 = bofs(a.W6, d.ss);
     __syncthreads();
-    double2* UR = S;
-    double2* UT = P;
-    const int c0 = mi_t << 1, c1 = (T + mi_t) << 1, c2 = (2 * T + mi_t) << 1;
-    for (int i = tid / T; i < N; i += NB / T) {
+    const int c0 = mi_t << 1, c1 = (T + mi_t) << 1, c2 = (2 * T + mi_t) << 1, kk = kk0 + mi_t;
+    for (int i = tid / T; i < N; i += NB / T) {  // u_theta
       const double* xr = X + i * NT;
-      const double2 up = double2{xr[c0], xr[c0 + 1]}, um = double2{xr[c1], xr[c1 + 1]};
-      UR[i * T + mi_t] = double2{0.5 * (up.x + um.x), 0.5 * (up.y + um.y)};
-      UT[i * T + mi_t] = double2{0.5 * (up.y - um.y), -0.5 * (up.x - um.x)};
+      P[i * T + mi_t] = double2{0.5 * (xr[c0 + 1] - xr[c1 + 1]), -0.5 * (xr[c0] - xr[c1])};
     }
     __syncthreads();
-    const int kk = kk0 + mi_t;
-    if (kk < nk) {
-      auto uz_at = [&](int i) { return double2{X[i * NT + c2], X[i * NT + c2 + 1]}; };
-      auto ut_at = [&](int i) { return UT[i * T + mi_t]; };
-      auto none = [](int) { return float2{}; };
-      for (int i = tid / T; i < N; i += NB / T)
-        curl_point<double2, false>(d, m, kk, i, ak_t, W1, nullptr, nullptr, RI, uz_at, ut_at, none, UR[i * T + mi_t],
-                                   UT[i * T + mi_t], uz_at(i), a.W6, nullptr);
+    for (int i = tid / T; kk < nk && i < N; i += NB / T) {
+      const int lo = row_lo_d(i, N);
+      double dzx = 0.0, dzy = 0.0, dtx = 0.0, dty = 0.0;  // d/dr of u_z, u_theta
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const double* xq = X + (lo + q) * NT + c2;
+        const double2 tq = P[(lo + q) * T + mi_t];
+        dzx = fma(ws[i * 9 + q], xq[0], dzx);
+        dzy = fma(ws[i * 9 + q], xq[1], dzy);
+        dtx = fma(wv[i * 9 + q], tq.x, dtx);
+        dty = fma(wv[i * 9 + q], tq.y, dty);
+      }
+      const double* xr = X + i * NT;
+      const double2 ur = double2{0.5 * (xr[c0] + xr[c1]), 0.5 * (xr[c0 + 1] + xr[c1 + 1])};
+      const double2 ut = P[i * T + mi_t], uz = double2{xr[c2], xr[c2 + 1]};
+      const double ri = RI[i], mri = mt * ri;
+      double2* W = a.W6 + base + (long)i * nk + kk;
+      W[0] = ur;
+      W[fs] = ut;
+      W[2 * fs] = uz;
+      W[3 * fs] = double2{ak_t * ut.y - mri * uz.y, mri * uz.x - ak_t * ut.x};
+      W[4 * fs] = double2{-ak_t * ur.y - dzx, ak_t * ur.x - dzy};
+      W[5 * fs] = double2{dtx + ri * ut.x + mri * ur.y, dty + ri * ut.y - mri * ur.x};
     }
   }
 }
@@ -1599,6 +1518,10 @@ static int solve_tile(const Dims& d) {
 }
 
 size_t solve_smem_bytes(int N, int T) { return solve_smem(N, T); }
+
+bool solve_takes_curl(const Dims& d) {
+  return solve_tile(d) == 4 && (long)((d.nk + 3) / 4) * d.M * d.B <= device_sms();
+}
 
 static size_t solve_smem(int N, int T) {
   return solve_stage_fits(N, T) ? solve_smem_staged(N, T) : solve_smem_base(N, T);
@@ -1658,13 +1581,11 @@ bool prepare_kernel_attrs(const Dims& d) {
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
     return false;
   const size_t lim = (size_t)optin;
-  if (zsynth_smem(d, d.mcz, vb) > lim || zanalysis_smem(d, d.mca, vb) > lim || curl_smem(d) > lim ||
+  if (zsynth_smem(d, d.mcz, vb) > lim || zanalysis_smem(d, d.mca, vb) > lim ||
       product_smem(d, d.zc, vb) > lim || solve_smem(d.N, solve_tile(d)) > lim)
     return false;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   bool ok = dft_prepare_attrs();
-  ok = ok && cudaFuncSetAttribute(k_curl<double2, false>, a, optin) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(k_curl<float2, true>, a, optin) == cudaSuccess;
   with_long_fft_length(d.nz, [&](auto n) {
     constexpr int L = decltype(n)::value;
     ok = ok && cudaFuncSetAttribute(k_zsynth<double2, L>, a, optin) == cudaSuccess;
@@ -1705,12 +1626,11 @@ bool prepare_nonlinear_attrs(const Dims& d) {
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
     return false;
   const size_t lim = (size_t)optin;
-  if (zsynth_smem(d, d.mcz, vb) > lim || zanalysis_smem(d, d.mca, vb) > lim || curl_smem(d) > lim ||
+  if (zsynth_smem(d, d.mcz, vb) > lim || zanalysis_smem(d, d.mca, vb) > lim ||
       product_smem(d, d.zc, vb) > lim)
     return false;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   bool ok = dft_prepare_attrs();
-  ok = ok && cudaFuncSetAttribute(k_curl<double2, false>, a, optin) == cudaSuccess;
   with_long_fft_length(d.nz, [&](auto n) {
     constexpr int L = decltype(n)::value;
     ok = ok && cudaFuncSetAttribute(k_zsynth<double2, L>, a, optin) == cudaSuccess;

@@ -31,6 +31,7 @@
 #include <mutex>
 #include <string>
 
+#include "opf_dft.cuh"
 #include "opf_internal.h"
 
 namespace {
@@ -65,14 +66,15 @@ bool smooth235(int n) {
 // (same points and folding as the handle's setup) and the z / theta twiddle
 // tables, computed on the device into the scratch.  One thread per weight:
 // with a_i = prod_(j != i) (x_i - x_j), the weight of node i at node c is
-// a_c / (a_i (x_c - x_i)), that of c itself sum_(j != c) 1 / (x_c - x_j).  (A
+// a_c / (a_i (x_c - x_i)), that of c itself sum_(j != c) 1 / (x_c - x_j).  A
+// block's rows are two tiles of the curl's digit table, which it fills in.  (A
 // thread per row running a recursion over the nodes took 101 us at N = 32 on
 // chains of divisions, more than the rest of the call.)
 constexpr int kConstRows = 16;                   // radial rows per block
 constexpr int kConstThreads = kConstRows * 9;    // a thread per (row, node)
 __global__ void __launch_bounds__(kConstThreads)
     k_noalloc_consts(int N, int nz, int nth, double Re, double* prm, double* d1, double* rinv, double2* twz,
-                     double2* twth) {
+                     double2* twth, uint2* tab, int* ew) {
   __shared__ double xs[kConstRows + 16], as[kConstRows][9], ws[kConstRows][9];
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < opf::kPrmCount) prm[t] = t == opf::kPrmRe ? Re : 0.0;
@@ -86,10 +88,10 @@ __global__ void __launch_bounds__(kConstThreads)
     sincospi(2.0 * t / nth, &s, &c);
     twth[t] = double2{c, s};
   }
-  const int n0 = blockIdx.x * kConstRows;
+  const int tiles = opf::stencil_tiles(N), n0 = blockIdx.x * kConstRows - (8 * tiles - N);
   if (n0 >= N) return;
   // extended nodes e0, e0 + 1, .. of the block's rows: e < N is -r_(N-1-e)
-  const int e0 = min(N + n0 - 4, 2 * N - 9);
+  const int e0 = min(N + max(n0, 0) - 4, 2 * N - 9);
   auto rad = [&](int j) { return j == N - 1 ? 1.0 : cospi((double)(N - 1 - j) / (2.0 * N - 1.0)); };
   if (threadIdx.x < kConstRows + 8 && e0 + (int)threadIdx.x < 2 * N) {
     const int e = e0 + threadIdx.x;
@@ -97,7 +99,7 @@ __global__ void __launch_bounds__(kConstThreads)
   }
   __syncthreads();
   const int row = threadIdx.x / 9, u = threadIdx.x - row * 9, n = n0 + row;
-  const bool in = n < N;
+  const bool in = n >= 0 && n < N;
   const int first = min(N + n - 4, 2 * N - 9);  // this row's first node
   const double* x = xs + (in ? first - e0 : 0);
   const int c = in ? N + n - first : 0;
@@ -118,19 +120,24 @@ __global__ void __launch_bounds__(kConstThreads)
     ws[row][c] = s;
   }
   __syncthreads();
-  if (!in) return;
   // slot u of the row's columns lo .. lo + 8: the real node there, plus the
   // ghost that folds onto it
-  const int lo = min(max(n - 4, 0), N - 9), col = lo + u;
-  double even = 0.0, odd = 0.0;
-  const int real = N + col - first, ghost = N - 1 - col - first;
-  if (real >= 0 && real < 9) even = odd = ws[row][real];
-  if (ghost >= 0 && ghost < 9 && ghost + first < N) {
-    even += ws[row][ghost];
-    odd -= ws[row][ghost];
+  if (in) {
+    const int lo = min(max(n - 4, 0), N - 9), col = lo + u;
+    double even = 0.0, odd = 0.0;
+    const int real = N + col - first, ghost = N - 1 - col - first;
+    if (real >= 0 && real < 9) even = odd = ws[row][real];
+    if (ghost >= 0 && ghost < 9) {
+      even += ws[row][ghost];
+      odd -= ws[row][ghost];
+    }
+    d1[(0 * N + n) * 9 + u] = even;
+    d1[(1 * N + n) * 9 + u] = odd;
   }
-  d1[(0 * N + n) * 9 + u] = even;
-  d1[(1 * N + n) * 9 + u] = odd;
+  __syncthreads();  // (the tiles' weights are this block's own)
+  const int tile = blockIdx.x * 2 + (threadIdx.x >> 6), par = (threadIdx.x >> 5) & 1;
+  if (threadIdx.x < 128 && tile < tiles)
+    opf::stencil_entry((par * tiles + tile) * 32 + (threadIdx.x & 31), d1, N, tab, ew);
 }
 
 int fail(int code, const std::string& m) {
@@ -231,12 +238,16 @@ extern "C" int opf_nonlinear_noalloc(int N, int K, int M, int m_p, double alpha,
   double2* ZN = (double2*)(base + o_ZN);
   double2* Nn = (double2*)(base + o_N);
 
-  const int nb = std::max((N + kConstRows - 1) / kConstRows,
-                          (std::max(d.nz, d.nth) + kConstThreads - 1) / kConstThreads);
-  k_noalloc_consts<<<nb, kConstThreads, 0, st>>>(N, d.nz, d.nth, Re, s.prm, s.d1, s.rinv, s.tw_z, s.tw_th);
+  // the curl's digit table: behind the other regions, or in the half-physical
+  // fields', which are not in use yet, where the scratch ends before
+  s.stab = need + opf::stencil_bytes(N) <= kNoallocScratchBytes ? base + need : base + o_Z6;
+  const opf::StencilTable stab = opf::stencil_at(s.stab, N);
+  const int nb = std::max((stab.tiles + 1) / 2, (std::max(d.nz, d.nth) + kConstThreads - 1) / kConstThreads);
+  k_noalloc_consts<<<nb, kConstThreads, 0, st>>>(N, d.nz, d.nth, Re, s.prm, s.d1, s.rinv, s.tw_z, s.tw_th,
+                                                 (uint2*)stab.tab, (int*)stab.ew);
   opf::launch_abi_to_internal(d, (const double2*)d_state, U, st);
   opf::launch_curl(d, s, U, W6, st);
-  // the transforms' tables: behind the other regions, or over U, which the
+  // the transforms' tables: behind the other regions (over the curl's), or over U, which the
   // curl has read, where the scratch ends before (a working set that fills it
   // has a U of a megabyte and more)
   unsigned char* tab = need + opf::dft_table_bytes(K, M) <= kNoallocScratchBytes ? base + need : base + o_U;

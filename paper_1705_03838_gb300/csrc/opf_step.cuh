@@ -44,17 +44,18 @@ void launch_step_kernel(const Dims& d, void (*kern)(KArgs...), dim3 g, dim3 b, s
 }
 
 // FP64 <-> FP32 by integer operations: the conversion instructions run on the
-// FP64 unit at its two lanes per clock, these at 64 a clock and more.  Same
-// results; the rare ranges (FP32 subnormals, infinities, NaN) take the
-// instruction.
-__device__ __forceinline__ float to_float(double x) {
+// FP64 unit at its two lanes per clock, these at 64 a clock.  Same results;
+// FP32 subnormals, infinities and NaN take the instruction.  Narrowing only
+// sets *rare for them: where the FP64 unit is the bound, the caller converts
+// several values again in one branch (a branch per value becomes a predicated
+// instruction, which occupies the unit all the same).
+__device__ __forceinline__ float to_float(double x, bool* rare) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const unsigned e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
   unsigned f = __funnelshift_r(lo, hi, 29) + 0x40000000u;      // exponent less 896 (mod 512)
   f += ((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29;    // to nearest, ties to even
-  f = (f & 0x7fffffffu) | sign;
-  if (e < 873u) f = sign;                                      // below half of the least subnormal
-  else if (e - 897u > 253u) f = __float_as_uint((float)x);
+  f = e < 873u ? sign : (f & 0x7fffffffu) | sign;              // (below half of the least subnormal: zero)
+  *rare |= e - 873u < 24u || e > 1150u;
   return __uint_as_float(f);
 }
 __device__ __forceinline__ double to_double(float x) {
@@ -65,6 +66,14 @@ __device__ __forceinline__ double to_double(float x) {
     hi = lo = 0u;
   }
   return __hiloint2double((int)(hi | (f & 0x80000000u)), (int)lo);
+}
+
+// x / 2 by its exponent (a multiplication takes the FP64 unit as long as an
+// addition).
+__device__ __forceinline__ double halved(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+  return e - 2u < 0x7fdu ? __hiloint2double(hi - 0x100000, __double2loint(x)) : 0.5 * x;
 }
 
 // Batched launches: trajectory b = blockIdx.z; its buffers sit `stride` bytes
