@@ -75,21 +75,21 @@ constexpr int kConstThreads = kConstRows * 9;    // a thread per (row, node)
 __global__ void __launch_bounds__(kConstThreads)
     k_noalloc_consts(int N, int nz, int nth, double Re, double* prm, double* d1, double* rinv, double2* twz,
                      double2* twth, uint2* tab, int* ew) {
-  __shared__ double xs[kConstRows + 16], as[kConstRows][9], ws[kConstRows][9];
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < opf::kPrmCount) prm[t] = t == opf::kPrmRe ? Re : 0.0;
-  if (t < nz) {
-    double s, c;
-    sincospi(2.0 * t / nz, &s, &c);
-    twz[t] = double2{c, s};
-  }
-  if (t < nth) {
-    double s, c;
-    sincospi(2.0 * t / nth, &s, &c);
-    twth[t] = double2{c, s};
-  }
+  __shared__ double xs[kConstRows + 16], as[kConstRows][9], ws[kConstRows][9], inv[kConstRows][9];
   const int tiles = opf::stencil_tiles(N), n0 = blockIdx.x * kConstRows - (8 * tiles - N);
-  if (n0 >= N) return;
+  if (n0 >= N) {  // blocks behind the rows': the twiddles
+    int t = (blockIdx.x - (tiles + 1) / 2) * blockDim.x + threadIdx.x;
+    if (t < opf::kPrmCount) prm[t] = t == opf::kPrmRe ? Re : 0.0;
+    const int n = t < nz ? nz : nth;
+    double2* tw = t < nz ? twz : twth;
+    t = t < nz ? t : t - nz;
+    if (t < n) {
+      double s, c;
+      sincospi(2.0 * t / n, &s, &c);
+      tw[t] = double2{c, s};
+    }
+    return;
+  }
   // extended nodes e0, e0 + 1, .. of the block's rows: e < N is -r_(N-1-e)
   const int e0 = min(N + max(n0, 0) - 4, 2 * N - 9);
   auto rad = [&](int j) { return j == N - 1 ? 1.0 : cospi((double)(N - 1 - j) / (2.0 * N - 1.0)); };
@@ -111,12 +111,16 @@ __global__ void __launch_bounds__(kConstThreads)
     if (u == 0) rinv[n] = 1.0 / rad(n);
   }
   __syncthreads();
-  if (in) ws[row][u] = u == c ? 0.0 : as[row][c] / (as[row][u] * (x[c] - x[u]));
+  if (in && u != c) {
+    const double dist = x[c] - x[u];
+    ws[row][u] = as[row][c] / (as[row][u] * dist);
+    inv[row][u] = 1.0 / dist;
+  }
   __syncthreads();
-  if (in && u == c) {  // the derivative of a constant is zero: sum the inverse distances
+  if (in && u == c) {
     double s = 0.0;
     for (int j = 0; j < 9; ++j)
-      if (j != c) s += 1.0 / (x[c] - x[j]);
+      if (j != c) s += inv[row][j];
     ws[row][c] = s;
   }
   __syncthreads();
@@ -242,7 +246,7 @@ extern "C" int opf_nonlinear_noalloc(int N, int K, int M, int m_p, double alpha,
   // fields', which are not in use yet, where the scratch ends before
   s.stab = need + opf::stencil_bytes(N) <= kNoallocScratchBytes ? base + need : base + o_Z6;
   const opf::StencilTable stab = opf::stencil_at(s.stab, N);
-  const int nb = std::max((stab.tiles + 1) / 2, (std::max(d.nz, d.nth) + kConstThreads - 1) / kConstThreads);
+  const int nb = (stab.tiles + 1) / 2 + (d.nz + d.nth + kConstThreads - 1) / kConstThreads;
   k_noalloc_consts<<<nb, kConstThreads, 0, st>>>(N, d.nz, d.nth, Re, s.prm, s.d1, s.rinv, s.tw_z, s.tw_th,
                                                  (uint2*)stab.tab, (int*)stab.ew);
   opf::launch_abi_to_internal(d, (const double2*)d_state, U, st);
