@@ -329,6 +329,13 @@ __device__ __forceinline__ void stencil_products(const uint4 (&a)[DIG], const ui
       if (i + j < LEV) dft_mma(acc[i + j], a[i], b);
   }
 }
+__device__ __forceinline__ void stencil_join(const float (&acc)[kLev][4], int er, int ei, int ew0, int ew1,
+                                             double2 (&out)[2]) {
+  unsigned w[4][kLev / 2];
+  dft_pairs(acc, w);
+  out[0] = double2{dft_value(w[0], dft_scale(er, ew0)), dft_value(w[2], dft_scale(ei, ew0))};
+  out[1] = double2{dft_value(w[1], dft_scale(er, ew1)), dft_value(w[3], dft_scale(ei, ew1))};
+}
 __device__ __forceinline__ void dft_stencil(const double2 (&x)[4], const uint2* __restrict__ tab, int ew0, int ew1,
                                             double2 (&out)[2]) {
   uint4 a[kDig];
@@ -336,10 +343,41 @@ __device__ __forceinline__ void dft_stencil(const double2 (&x)[4], const uint2* 
   int er, ei;
   stencil_digits<kDig>(x, a, &er, &ei);
   stencil_products<kDig, kLev>(a, tab, acc);
-  unsigned w[4][kLev / 2];
-  dft_pairs(acc, w);
-  out[0] = double2{dft_value(w[0], dft_scale(er, ew0)), dft_value(w[2], dft_scale(ei, ew0))};
-  out[1] = double2{dft_value(w[1], dft_scale(er, ew1)), dft_value(w[3], dft_scale(ei, ew1))};
+  stencil_join(acc, er, ei, ew0, ew1, out);
+}
+// Four modes at two tiles: lanes g < 4 at the first (table tab), the others at
+// the next (if two).  Every lane goes through both tables' products, which are
+// the cheap part, and joins its own.
+__device__ __forceinline__ void dft_stencil_pair(const double2 (&x)[4], const uint2* __restrict__ tab, bool two,
+                                                 bool second, int ew0, int ew1, double2 (&out)[2]) {
+  uint4 a[kDig];
+  float acc[kLev][4];
+  int er, ei;
+  stencil_digits<kDig>(x, a, &er, &ei);
+  stencil_products<kDig, kLev>(a, tab, acc);
+  if (two) {
+    float acc1[kLev][4];
+    stencil_products<kDig, kLev>(a, tab + kTileB, acc1);
+#pragma unroll
+    for (int l = 0; l < kLev; ++l)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[l][q] = second ? acc1[l][q] : acc[l][q];
+  }
+  stencil_join(acc, er, ei, ew0, ew1, out);
+}
+// That as one copy of the code per kernel, for blocks that have an SM to
+// themselves and go through it once per use: there fetching the instructions
+// is most of its time.
+struct StencilPair {
+  double2 v[2];
+};
+static __device__ __noinline__ StencilPair dft_stencil_call(double2 x0, double2 x1, double2 x2, double2 x3,
+                                                            const uint2* __restrict__ tab, bool two, bool second,
+                                                            int ew0, int ew1) {
+  const double2 x[4] = {x0, x1, x2, x3};
+  StencilPair out;
+  dft_stencil_pair(x, tab, two, second, ew0, ew1, out.v);
+  return out;
 }
 // The same to FP32: five digits and levels are 2^-39 of the largest term.
 __device__ __forceinline__ void dft_stencil32(const double2 (&x)[4], const uint2* __restrict__ tab, int ew0, int ew1,

@@ -923,6 +923,7 @@ struct SolveDev {
   const double2* ainv;
   const double* G;
   const double* prm;
+  StencilTable st;  // digit table of the stencils
   int nJ;
   int stage;  // u_j and the influence responses staged in shared memory
   // split solve: both blocks' factors, spikes, interface inverses
@@ -960,9 +961,13 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // The host stages only where that costs no resident blocks (see
 // launch_solve); the launch gives the staged size then, the base size else.
 // sp: the split solve's interface values (6T chains x 8 doubles) after misc.
+// The stencils are digit products (dft_stencil; results do not depend on the
+// tile) and only the wall divergence's weights are kept here, except in the
+// split solve, whose grids of few blocks are better off with multiply-adds.
+__host__ __device__ constexpr int solve_weights(int N, bool sp) { return sp ? 2 * N * 9 : 10; }
 __host__ __device__ constexpr size_t solve_smem_base(int N, int T, bool sp = false) {
   return (size_t)(2 * N * T + T) * 16 + (size_t)6 * N * T * 8 +
-         (size_t)(2 * N * 9 + 3 * N + 2) * 8 + 16 + (sp ? (size_t)48 * T * 8 : 0);
+         (size_t)(solve_weights(N, sp) + 3 * N + 2) * 8 + 16 + (sp ? (size_t)48 * T * 8 : 0);
 }
 __host__ __device__ constexpr size_t solve_smem_staged(int N, int T, bool sp = false) {
   return solve_smem_base(N, T, sp) + (size_t)48 * N * T + (size_t)8 * basis_ld(N) * T;
@@ -1103,6 +1108,19 @@ __device__ __forceinline__ void band_solve4(const double* __restrict__ L, double
 // flux correction on the way out to global memory, and with a.curl the block
 // then takes the curl of its new state for the next nonlinear evaluation.
 //
+// The radial derivatives (of N+ + N- and of p) are digit products on the tensor
+// cores (dft_stencil), a warp per eight modes and rows, except in the split
+// solve (on a block per SM its wider block with FP64 multiply-adds and the
+// weights in shared memory is the faster: 28.6 us at N = 32, 31 x 16 modes).
+// What bounds it: the chains of the substitutions and, on large grids, the
+// FP64 unit, which the stencils took 36 of ~90 instructions per point of.  Per
+// launch against multiply-adds: N = 128, 255 x 128 modes 1743 -> 1533 us, 64 x
+// (N = 32, 31 x 16) 411 -> 376 us, groups of 8 x (N = 32 .. 48) and 6 x (N = 64,
+// 63 x 32) 193 -> 180 us, N = 48, 63 x 24 modes 46.0 -> 42.5 us; N = 41, 53 x 20
+// modes (two blocks per SM) 35.8 us either way; N = 20, 7 x 5 modes, which takes
+// the curl as well and is latency alone, 24.3 -> 28.4 us -- there the one copy of
+// the code (dft_stencil_call) is 2 us faster than one per use.
+//
 // Resident blocks per SM the register budget must allow (the shared-memory
 // footprints of the tiles allow about as many at moderate N).
 template <int T, bool SP>
@@ -1146,7 +1164,8 @@ __device__ __forceinline__ void spike_fix(int tid, int N, int nch, int st, doubl
 // SP: the split (two-partition) solve for the latency-bound grids -- each
 // chain's substitution runs on 8 lanes, the two halves of its rows at once
 // (twice the threads; the other phases use them too).
-template <int T, bool SP = false>
+// CURL: may take the curl of its new state (a.W6).
+template <int T, bool SP = false, bool CURL = SP>
 __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     k_solve(Dims d, SolveDev s, SolveArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1161,8 +1180,8 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   double2* P = S + N * T;                      // [N][T]     pressure (later u_theta)
   double2* coef = P + N * T;                   // [T]        influence coefficients
   double* X = (double*)(coef + T);             // [N][6T]    N_eff -> right-hand sides -> velocity chains
-  double* W1 = X + N * NT;                     // [2][N][9]  first-derivative stencils
-  double* RI = W1 + 2 * N * 9;                 // [N]        1/r
+  double* W1 = X + N * NT;                     // [2][N][9]  first-derivative stencils (digits: the wall's row)
+  double* RI = W1 + solve_weights(N, SP);      // [N]        1/r
   double* RIp = RI + N;                        // [N]        (1 + m~) / (2r)
   double* RIm = RIp + N;                       // [N]        (1 - m~) / (2r)
   double* misc = RIm + N;                      // [2]        flux correction
@@ -1190,6 +1209,8 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   s.ainv = bofs(s.ainv, d.ps);
   s.G = bofs(s.G, d.ps);
   s.prm = bofs(s.prm, d.ps);
+  s.st.tab = bofs(s.st.tab, d.ps);
+  s.st.ew = bofs(s.st.ew, d.ps);
   if constexpr (SP) {
     s.luH2 = bofs(s.luH2, d.ps);
     s.luP2 = bofs(s.luP2, d.ps);
@@ -1206,8 +1227,10 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   const double ci = s.prm[kPrmCi], cu = s.prm[kPrmCu];  // 1 / (c dt), (1 - c) / c
   const long fs = d.F;
   const long base = (long)m * N * nk;
+  constexpr bool kDigits = !SP;
   const double* wv = W1 + pv * N * 9;  // stencils of u_r, u_theta parity
   const double* ws = W1 + ps * N * 9;  // stencils of u_z, p parity
+  const double* wall = kDigits ? W1 : wv + (N - 1) * 9;  // wall row of wv
   // chain c -> (field f, mode mi, part); element (f, row i, mode mi) of a field
   auto uj = [&](int f, int i, int mi) {
     return a.Uj[f * fs + base + (long)i * nk + min(kk0 + mi, nk - 1)];
@@ -1231,7 +1254,14 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   }
 
   // The stencils by asynchronous copies, waited for at the first barrier.
-  for (int e = tid; e < 2 * N * 9; e += NB) cp_async8(W1 + e, s.d1 + e);
+  if constexpr (kDigits) {
+    if (tid < 9) cp_async8(W1 + tid, s.d1 + ((long)pv * N + N - 1) * 9 + tid);
+    if (CURL && a.W6)  // a block per SM: the digit tables to the SM's cache while it waits for its input
+      for (int e = tid; e < 2 * s.st.tiles * (kTileB / 16); e += NB)
+        asm volatile("{\n.reg .b32 t;\nld.global.ca.b32 t, [%0];\n}" ::"l"(s.st.tab + 16 * e));
+  } else {
+    for (int e = tid; e < 2 * N * 9; e += NB) cp_async8(W1 + e, s.d1 + e);
+  }
   cp_async_commit();
 
   // ---- N_eff = N_a (predictor) or (N_a + N_b) / 2 (corrector, c = 1/2), and
@@ -1268,7 +1298,53 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   const int mi_t = tid % T;
   const double ak_t = d.alpha * (min(kk0 + mi_t, nk - 1) - (K - 1));
 
+  // The derivative (times 2^shift) of a field at(row, mode) of one parity at every
+  // row and mode, out(row, mode, alpha k, derivative): a warp per eight modes and
+  // eight rows, or per four modes and two such tiles (one if there are warps
+  // enough).
+  auto for_stencil_items = [&](auto at, int parity, int shift, auto out) {
+    const int lane = tid & 31, g = lane >> 2, t = lane & 3;
+    constexpr int kGroups = T >= 8 ? T / 8 : 1;  // of modes
+    const int tiles = s.st.tiles, per = T >= 8 || tiles <= NB / 32 ? 1 : 2;  // tiles per item
+    for (int it = tid >> 5; it < (tiles + per - 1) / per * kGroups; it += NB / 32) {
+      __syncwarp();
+      const int first = it / kGroups * per, nt = T >= 8 || g < 4 ? first : per == 2 ? first + 1 : tiles;
+      const int mi = T >= 8 ? it % kGroups * 8 + g : g & 3, i0 = nt * 8 - s.st.off;
+      double2 x[4];
+      StencilPair d9;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = stencil_row(i0, t, q);
+        x[q] = i >= 0 && i < N ? at(i, mi) : double2{0.0, 0.0};  // (a tile past the last has no rows < N)
+      }
+      const int* ew = s.st.ew + (parity * tiles + min(nt, tiles - 1)) * 8 + 2 * t;
+      const uint2* tab = s.st.tab + (long)(parity * tiles + first) * kTileB + lane;
+      if constexpr (T >= 8) dft_stencil(x, tab, ew[0] + shift, ew[1] + shift, d9.v);
+      else {
+        const bool two = per == 2 && first + 1 < tiles;
+        if constexpr (CURL)
+          d9 = dft_stencil_call(x[0], x[1], x[2], x[3], tab, two, g >= 4, ew[0] + shift, ew[1] + shift);
+        else
+          dft_stencil_pair(x, tab, two, g >= 4, ew[0] + shift, ew[1] + shift, d9.v);
+      }
+      const double ak = d.alpha * (min(kk0 + mi, nk - 1) - (K - 1));
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = i0 + 2 * t + q;
+        if (i >= 0 && i < N) out(i, mi, ak, d9.v[q]);
+      }
+    }
+  };
+
   // ---- pressure right-hand side: div N_eff (rows < N-1), 0 at the wall
+  if constexpr (kDigits) {
+    for_stencil_items([&](int i, int mi) { return S[i * T + mi]; }, pv, -1, [&](int i, int mi, double ak, double2 dr) {  // dr: half the derivative
+      const double2 np = ne_at(0, i, mi), nm = ne_at(1, i, mi), nz = ne_at(2, i, mi);
+      const double bx = dr.x + fma(RIp[i], np.x, fma(RIm[i], nm.x, -ak * nz.y));
+      const double by = dr.y + fma(RIp[i], np.y, fma(RIm[i], nm.y, ak * nz.x));
+      P[i * T + mi] = i < N - 1 ? double2{bx, by} : double2{0.0, 0.0};
+    });
+  } else
   for (int i = tid / T; i < N; i += NB / T) {
     double2 b = double2{0.0, 0.0};
     if (i < N - 1) {
@@ -1343,6 +1419,23 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   // ---- d_r p per (mode, row), subtracted at once from the right-hand sides of
   //      the three fields (rows < N-1):
   //      (grad p)+- = d_r p -+ m~ p / r,  (grad p)_z = i ak p
+  auto subtract_gradient = [&](int i, int mi, double ak, double2 dp) {
+    const double2 pp = P[i * T + mi];
+    const double mr = mt * RI[i];
+    double* xr = X + i * NT;
+    const int c0 = mi << 1, c1 = (T + mi) << 1, c2 = (2 * T + mi) << 1;
+    xr[c0] = fma(mr, pp.x, xr[c0] - dp.x);
+    xr[c0 + 1] = fma(mr, pp.y, xr[c0 + 1] - dp.y);
+    xr[c1] = fma(-mr, pp.x, xr[c1] - dp.x);
+    xr[c1 + 1] = fma(-mr, pp.y, xr[c1 + 1] - dp.y);
+    xr[c2] = fma(ak, pp.y, xr[c2]);
+    xr[c2 + 1] = fma(-ak, pp.x, xr[c2 + 1]);
+  };
+  if constexpr (kDigits) {
+    for_stencil_items([&](int i, int mi) { return P[i * T + mi]; }, ps, 0, [&](int i, int mi, double ak, double2 dp) {
+      if (i < N - 1) subtract_gradient(i, mi, ak, dp);
+    });
+  } else
   for (int i = tid / T; i < N - 1; i += NB / T) {
     const int lo = row_lo_d(i, N);
     double ax = 0.0, ay = 0.0;
@@ -1353,16 +1446,7 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
       ax = fma(w, pv2.x, ax);
       ay = fma(w, pv2.y, ay);
     }
-    const double2 pp = P[i * T + mi_t];
-    const double mr = mt * RI[i];
-    double* xr = X + i * NT;
-    const int c0 = mi_t << 1, c1 = (T + mi_t) << 1, c2 = (2 * T + mi_t) << 1;
-    xr[c0] = fma(mr, pp.x, xr[c0] - ax);
-    xr[c0 + 1] = fma(mr, pp.y, xr[c0 + 1] - ay);
-    xr[c1] = fma(-mr, pp.x, xr[c1] - ax);
-    xr[c1 + 1] = fma(-mr, pp.y, xr[c1 + 1] - ay);
-    xr[c2] = fma(ak_t, pp.y, xr[c2]);
-    xr[c2 + 1] = fma(-ak_t, pp.x, xr[c2 + 1]);
+    subtract_gradient(i, mi_t, ak_t, double2{ax, ay});
   }
   __syncthreads();
 
@@ -1403,7 +1487,7 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
       return double2{X[i * NT + c] - cu * w.x, X[i * NT + c + 1] - cu * w.y};
     };
     const double2 p = uv(0), mm = uv(1);
-    const double w = 0.5 * wv[(N - 1) * 9 + q];
+    const double w = 0.5 * wall[q];
     double2 g = double2{w * (p.x + mm.x), w * (p.y + mm.y)};
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) {
@@ -1458,46 +1542,58 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     if (has_mean && c == cz) v += bp * s.G[i];
     double* out = (double*)(a.Uout + f * fs + base + (long)i * nk + kk0 + mi) + part;
     *out = v;
-    if (T == 4 && a.W6) X[i * NT + c] = v;  // (only this element's own X is read above)
+    if (CURL && a.W6) X[i * NT + c] = v;  // (only this element's own X is read above)
   }
 
   // ---- FP64 steps on grids of at most a block per SM: the curl (A1) of the
   //      new state for the next nonlinear evaluation from the block's radial
   //      columns.  There the time is latency: a curl launch of its own took
   //      3 us longer per pass at N = 32, 31 x 16 modes (on larger grids it is
-  //      the faster form).
-  if (T == 4 && a.W6) {
+  //      the faster form).  But for the split solve the values are k_curl's.
+  if (CURL && a.W6) {
     a.W6 = bofs(a.W6, d.ss);
     __syncthreads();
-    const int c0 = mi_t << 1, c1 = (T + mi_t) << 1, c2 = (2 * T + mi_t) << 1, kk = kk0 + mi_t;
+    const int c0 = mi_t << 1, c1 = (T + mi_t) << 1, c2 = (2 * T + mi_t) << 1;
     for (int i = tid / T; i < N; i += NB / T) {  // u_theta
       const double* xr = X + i * NT;
       P[i * T + mi_t] = double2{0.5 * (xr[c0 + 1] - xr[c1 + 1]), -0.5 * (xr[c0] - xr[c1])};
     }
     __syncthreads();
-    for (int i = tid / T; kk < nk && i < N; i += NB / T) {
-      const int lo = row_lo_d(i, N);
-      double dzx = 0.0, dzy = 0.0, dtx = 0.0, dty = 0.0;  // d/dr of u_z, u_theta
-#pragma unroll
-      for (int q = 0; q < 9; ++q) {
-        const double* xq = X + (lo + q) * NT + c2;
-        const double2 tq = P[(lo + q) * T + mi_t];
-        dzx = fma(ws[i * 9 + q], xq[0], dzx);
-        dzy = fma(ws[i * 9 + q], xq[1], dzy);
-        dtx = fma(wv[i * 9 + q], tq.x, dtx);
-        dty = fma(wv[i * 9 + q], tq.y, dty);
-      }
+    auto put = [&](int i, int mi, double ak, double2 dz, double2 dt) {  // dz, dt: d/dr of u_z, u_theta
+      if (kk0 + mi >= nk) return;
       const double* xr = X + i * NT;
-      const double2 ur = double2{0.5 * (xr[c0] + xr[c1]), 0.5 * (xr[c0 + 1] + xr[c1 + 1])};
-      const double2 ut = P[i * T + mi_t], uz = double2{xr[c2], xr[c2 + 1]};
+      const int b0 = mi << 1, b1 = (T + mi) << 1, b2 = (2 * T + mi) << 1;
+      const double2 ur = double2{0.5 * (xr[b0] + xr[b1]), 0.5 * (xr[b0 + 1] + xr[b1 + 1])};
+      const double2 ut = P[i * T + mi], uz = double2{xr[b2], xr[b2 + 1]};
       const double ri = RI[i], mri = mt * ri;
-      double2* W = a.W6 + base + (long)i * nk + kk;
+      double2* W = a.W6 + base + (long)i * nk + kk0 + mi;
       W[0] = ur;
       W[fs] = ut;
       W[2 * fs] = uz;
-      W[3 * fs] = double2{ak_t * ut.y - mri * uz.y, mri * uz.x - ak_t * ut.x};
-      W[4 * fs] = double2{-ak_t * ur.y - dzx, ak_t * ur.x - dzy};
-      W[5 * fs] = double2{dtx + ri * ut.x + mri * ur.y, dty + ri * ut.y - mri * ur.x};
+      W[3 * fs] = double2{-fma(mri, uz.y, -ak * ut.y), fma(mri, uz.x, -ak * ut.x)};  // (as k_curl rounds)
+      W[4 * fs] = double2{fma(-ak, ur.y, -dz.x), fma(ak, ur.x, -dz.y)};
+      W[5 * fs] = double2{fma(mri, ur.y, fma(ri, ut.x, dt.x)), fma(-mri, ur.x, fma(ri, ut.y, dt.y))};
+    };
+    if constexpr (kDigits) {  // (a row and mode belong to the same lane in both passes)
+      for_stencil_items([&](int i, int mi) { return P[i * T + mi]; }, pv, 0,
+                        [&](int i, int mi, double, double2 dt) { S[i * T + mi] = dt; });
+      for_stencil_items([&](int i, int mi) { return *(const double2*)(X + i * NT + ((2 * T + mi) << 1)); }, ps, 0,
+                        [&](int i, int mi, double ak, double2 dz) { put(i, mi, ak, dz, S[i * T + mi]); });
+    } else {
+      for (int i = tid / T; i < N; i += NB / T) {
+        const int lo = row_lo_d(i, N);
+        double2 dz = double2{0.0, 0.0}, dt = dz;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+          const double* xq = X + (lo + q) * NT + c2;
+          const double2 tq = P[(lo + q) * T + mi_t];
+          dz.x = fma(ws[i * 9 + q], xq[0], dz.x);
+          dz.y = fma(ws[i * 9 + q], xq[1], dz.y);
+          dt.x = fma(wv[i * 9 + q], tq.x, dt.x);
+          dt.y = fma(wv[i * 9 + q], tq.y, dt.y);
+        }
+        put(i, mi_t, ak_t, dz, dt);
+      }
     }
   }
 }
@@ -1517,7 +1613,12 @@ static int solve_tile(const Dims& d) {
   return 4;
 }
 
-size_t solve_smem_bytes(int N, int T) { return solve_smem(N, T); }
+// What a resolution or tile has to fit in to be accepted: a block that keeps
+// the stencils' weights as well, as the split solve's does (N <= 475 with the
+// 4-mode tile), whichever form then runs.
+size_t solve_smem_bytes(int N, int T) {
+  return std::max(solve_smem(N, T), (size_t)(2 * N * T + 4 * T) * 16 + (size_t)48 * N * T + (size_t)(21 * N + 4) * 8);
+}
 
 bool solve_takes_curl(const Dims& d) {
   return solve_tile(d) == 4 && (long)((d.nk + 3) / 4) * d.M * d.B <= device_sms();
@@ -1582,7 +1683,7 @@ bool prepare_kernel_attrs(const Dims& d) {
     return false;
   const size_t lim = (size_t)optin;
   if (zsynth_smem(d, d.mcz, vb) > lim || zanalysis_smem(d, d.mca, vb) > lim ||
-      product_smem(d, d.zc, vb) > lim || solve_smem(d.N, solve_tile(d)) > lim)
+      product_smem(d, d.zc, vb) > lim || solve_smem_bytes(d.N, solve_tile(d)) > lim)
     return false;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   bool ok = dft_prepare_attrs();
@@ -1606,6 +1707,7 @@ bool prepare_kernel_attrs(const Dims& d) {
   ok = ok && cudaFuncSetAttribute(k_solve<16>, a, optin) == cudaSuccess;
   ok = ok && cudaFuncSetAttribute(k_solve<8>, a, optin) == cudaSuccess;
   ok = ok && cudaFuncSetAttribute(k_solve<4>, a, optin) == cudaSuccess;
+  ok = ok && cudaFuncSetAttribute(k_solve<4, false, true>, a, optin) == cudaSuccess;
   ok = ok && cudaFuncSetAttribute(k_solve<4, true>, a, optin) == cudaSuccess;
   auto fusable = [](int n) { return n == 48 || n == 72 || n == 96; };
   if (fusable(d.nz) && fusable(d.nth))  // (the option or the autotuner may switch the fused launch on later)
@@ -1615,10 +1717,11 @@ bool prepare_kernel_attrs(const Dims& d) {
   return ok;
 }
 
-// Shared-memory limits of the FP64 nonlinear-term kernels only (curl, z
-// synthesis, theta product, z analysis) for the allocation-free entry point:
-// checks their footprints against the opt-in limit and raises their dynamic
-// shared-memory limit to it.
+// Shared-memory limits of the FP64 nonlinear-term kernels only (z synthesis,
+// theta product, z analysis) for the allocation-free entry point: checks their
+// footprints against the opt-in limit and raises their dynamic shared-memory
+// limit to it.  The radial resolution it accepts is that of a block which
+// keeps four columns of the curl (N <= 968), although k_curl itself needs none.
 bool prepare_nonlinear_attrs(const Dims& d) {
   const size_t vb = sizeof(double2);
   int dev = 0, optin = 0;
@@ -1626,8 +1729,9 @@ bool prepare_nonlinear_attrs(const Dims& d) {
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
     return false;
   const size_t lim = (size_t)optin;
+  const size_t cols = (size_t)d.M * d.nk, blocks = (cols + 3) / 4, kc = (cols + blocks - 1) / blocks;
   if (zsynth_smem(d, d.mcz, vb) > lim || zanalysis_smem(d, d.mca, vb) > lim ||
-      product_smem(d, d.zc, vb) > lim)
+      product_smem(d, d.zc, vb) > lim || (size_t)d.N * (56 * kc + 16) + 16 * kc > lim)
     return false;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   bool ok = dft_prepare_attrs();
@@ -1649,11 +1753,12 @@ void launch_solve(const Dims& d, const DevSetup& s, const SolveArgs& a, int nJ, 
   dim3 g((d.nk + T - 1) / T, d.M, d.B);
   const bool stage = solve_use_stage(d, T, (long)g.x * g.y * g.z, sp);
   SolveDev sd{s.d1,  s.rinv, s.wq,   s.hop,  s.luH,  s.luP,  s.basis, s.ainv, s.G,  s.prm,
-              nJ,    stage ? 1 : 0,  s.luH2, s.luP2, s.spkH,  s.spkP, s.rH, s.rP};
+              stencil_at(s.stab, d.N), nJ,    stage ? 1 : 0,  s.luH2, s.luP2, s.spkH,  s.spkP, s.rH, s.rP};
   const size_t sm = stage ? solve_smem_staged(d.N, T, sp) : solve_smem_base(d.N, T, sp);
   if (T == 16) launch_step_kernel(d, k_solve<16>, g, dim3(24 * 16), sm, st, d, sd, a);
   else if (T == 8) launch_step_kernel(d, k_solve<8>, g, dim3(24 * 8), sm, st, d, sd, a);
   else if (sp) launch_step_kernel(d, k_solve<4, true>, g, dim3(48 * 4), sm, st, d, sd, a);
+  else if (a.W6) launch_step_kernel(d, k_solve<4, false, true>, g, dim3(24 * 4), sm, st, d, sd, a);
   else launch_step_kernel(d, k_solve<4>, g, dim3(24 * 4), sm, st, d, sd, a);
 }
 
