@@ -137,36 +137,62 @@ void stencil_host_table(const double* d1, int N, void* host) {
     stencil_entry(idx, d1, N, tab, (int*)(tab + stencil_table_size(N)));
 }
 // ------------------------------------------------------------------ z synthesis
-// Block: up to 32 m columns of one field and radial row.  A row tile is eight
-// columns: rows 0-7 their real parts, 8-15 the imaginary ones; the sums over
-// harmonics of X_k + X_-k with cosines and of X_k - X_-k with sines give the
-// points p and n - p.
+// A row tile is eight m columns of one field and radial row: rows 0-7 their
+// real parts, 8-15 the imaginary ones; the sums over harmonics of X_k + X_-k
+// with cosines and of X_k - X_-k with sines give the points p and n - p.
+// Block: R consecutive row tiles, whose R KT digit tiles take a warp each and
+// whose R NT products are dealt out to the warps.
+namespace {
+struct SynthShape {
+  int R, blocks;
+};
+// The tiles per block that take the fewest rounds of the eight warps over the
+// waves of two blocks per SM: few on small grids, a digit tile for every warp
+// on large ones.  (64 x (N = 32, 31 x 16 modes), whose rows are two tiles of one
+// digit tile each: 184 us with a row per block, most of its warps waiting for
+// the two that cut digits; 141 us with eight tiles.)
+SynthShape synth_shape(const Dims& d) {
+  const int KT = dft_tiles(d.K, 16), NT = dft_tiles(dft_points(d.nz), 8);
+  const long tiles = 6L * d.N * ((d.M + 7) / 8), slots = 2L * device_sms();
+  SynthShape best{1, 0};
+  long cost = -1;
+  for (int R = 1; R * KT <= kWarps; ++R) {
+    const long blocks = (tiles + R - 1) / R;
+    const long c = (blocks * d.B + slots - 1) / slots * (1 + (R * NT + kWarps - 1) / kWarps);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = SynthShape{R, (int)blocks};
+    }
+  }
+  return best;
+}
+}  // namespace
 size_t dft_zsynth_smem(const Dims& d) {
-  return (size_t)std::min(4, (d.M + 7) / 8) * 2 * dft_tiles(d.K, 16) * kTileA * sizeof(uint4);
+  return (size_t)synth_shape(d).R * 2 * dft_tiles(d.K, 16) * kTileA * sizeof(uint4);
 }
 
 __global__ void __launch_bounds__(kThreads, 2)
-    k_dft_zsynth(Dims d, const uint2* __restrict__ Tc, const uint2* __restrict__ Ts, const double2* __restrict__ W6,
-                 double2* __restrict__ Z6) {
+    k_dft_zsynth(Dims d, int R, const uint2* __restrict__ Tc, const uint2* __restrict__ Ts,
+                 const double2* __restrict__ W6, double2* __restrict__ Z6) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ int emx[4][8];
+  __shared__ int emx[kWarps][8];
   const int K = d.K, M = d.M, N = d.N, nk = d.nk, nz = d.nz;
-  const int m0 = blockIdx.x * 32, n = blockIdx.y / 6, f = blockIdx.y % 6;
-  const int RT = min(4, (M - m0 + 7) / 8), KT = dft_tiles(K, 16), P = dft_points(nz), NT = dft_tiles(P, 8);
+  const int MT = (M + 7) / 8, t0 = blockIdx.x * R, RT = min(R, 6 * N * MT - t0);
+  const int KT = dft_tiles(K, 16), P = dft_points(nz), NT = dft_tiles(P, 8);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   uint4* A = (uint4*)smraw;  // [row tile][sum, difference][k tile] tiles
   W6 = bofs(W6, d.ss);
   Z6 = bofs(Z6, d.ss);
   grid_dep_trigger_at(d, 1);
-  if (threadIdx.x < 32) emx[threadIdx.x >> 3][threadIdx.x & 7] = 0;
-  __syncthreads();
-  grid_dep_wait();
+  if (threadIdx.x < kWarps * 8) emx[threadIdx.x >> 3][threadIdx.x & 7] = 0;
   double2 xp[4], xm[4];  // X_k, X_-k
   const int rt = warp / KT, kt = warp - rt * KT;  // KT <= 2: one item per warp
   const bool have = rt < RT;
+  const int fn = (t0 + rt) / MT, f = fn / N, m = (t0 + rt - fn * MT) * 8 + g;  // fn = field * N + row
+  const double2* src = W6 + (long)f * d.F + ((long)m * N + fn - f * N) * nk + K - 1;
+  __syncthreads();
+  grid_dep_wait();
   if (have) {
-    const int m = m0 + rt * 8 + g;
-    const double2* src = W6 + (long)f * d.F + ((long)m * N + n) * nk + K - 1;
     int e = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -209,9 +235,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     dft_pairs(acc, c);
     dft_gemm(acc, A + (r * 2 + 1) * KT * kTileA + lane, Ts + (long)nt * KT * kTileB + lane, KT);
     dft_pairs(acc, s);
-    const int m = m0 + r * 8 + g;
+    const int fn = (t0 + r) / MT, m = (t0 + r - fn * MT) * 8 + g;
     const DftScale sc = dft_scale(emx[r][g], 1);
-    double2* dst = Z6 + ((long)f * N + n) * nz * M + m;
+    double2* dst = Z6 + (long)fn * nz * M + m;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {  // e^{+i phi}: (c + i s) at p, (c - i s) at n - p
       const int p = nt * 8 + 2 * t + q;
@@ -235,9 +261,9 @@ struct ProductShape {
   size_t phys, a1, a2;  // bytes: one field's rows, a round's digits, the products' digits
   size_t smem;
 };
-__host__ __device__ inline ProductShape product_shape(int M, int nth, int warps) {
+__host__ __device__ inline ProductShape product_shape(int M, int nth, int fields) {
   ProductShape s;
-  s.fields = warps >= 16 ? 6 : 3;
+  s.fields = fields;
   s.ldq = (nth + 7) / 16 * 16 + 8;
   s.KT = dft_tiles(M, 16);
   s.NT = dft_tiles(dft_points(nth), 8);
@@ -253,17 +279,21 @@ __host__ __device__ inline ProductShape product_shape(int M, int nth, int warps)
 }
 }  // namespace
 
-// WARPS: 8, two blocks per SM, or 16 where there are no more blocks than SMs.
-template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, 16 / WARPS)
+// FIELDS per round.  16 warps and all six where there are no more blocks than
+// SMs.  Else 8 warps, two blocks per SM: with one k tile per row (M <= 16) and
+// its small footprint all six fields at once, 6 digit tiles and 24 products for
+// the 8 warps where two rounds of 3 and 12 left warps waiting (64 x (N = 32,
+// 31 x 16 modes) 409 -> 352 us; six warps in three blocks 379 us); else three.
+template <int WARPS, int FIELDS, int BLOCKS>
+__global__ void __launch_bounds__(WARPS * 32, BLOCKS)
     k_dft_product(Dims d, const uint2* __restrict__ Sc, const uint2* __restrict__ Ss, const uint2* __restrict__ Ac,
                   const uint2* __restrict__ As, const double2* __restrict__ tw, const double2* __restrict__ Z6,
                   double2* __restrict__ ZN) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int kFields = WARPS >= 16 ? 6 : 3;
+  constexpr int kFields = FIELDS;
   __shared__ int emx[kFields][16], emn[3][16];
   const int M = d.M, N = d.N, nz = d.nz, nth = d.nth;
-  const ProductShape ps = product_shape(M, nth, WARPS);
+  const ProductShape ps = product_shape(M, nth, FIELDS);
   const int ldq = ps.ldq, KT = ps.KT, KT2 = ps.KT2, P = dft_points(nth);
   double* ph = (double*)smraw;  // [6][16][ldq]
   uint4* A1 = (uint4*)(smraw + 6 * ps.phys);
@@ -458,7 +488,13 @@ size_t dft_zanalysis_smem(const Dims& d) {
   return std::max(a, (size_t)24 * d.nk * sizeof(double2));
 }
 
-__global__ void __launch_bounds__(kThreads, 2)
+// WARPS: its 3, 6, 9 or 12 digit tiles and as many products or fewer take
+// multiples of three; six, with a third block per SM where the digits fit, were
+// 106 -> 86 us against eight on 64 x (N = 32, 31 x 16 modes), and twelve where
+// there are no more blocks than SMs 18.3 -> 17.1 us at N = 48, 63 x 24 modes.
+// There eight do for up to 8 tiles (twelve: 1 us more per launch at N = 20, 32).
+template <int WARPS, int BLOCKS>
+__global__ void __launch_bounds__(WARPS * 32, BLOCKS)
     k_dft_zanalysis(Dims d, int zshift, const uint2* __restrict__ Tc, const uint2* __restrict__ Ts,
                     const double2* __restrict__ ZN, double2* __restrict__ Nout) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -477,11 +513,11 @@ __global__ void __launch_bounds__(kThreads, 2)
   if (threadIdx.x < 24) emx[threadIdx.x >> 3][threadIdx.x & 7] = 0;
   __syncthreads();
   grid_dep_wait();
-  constexpr int kItems = 2;  // 3 KT <= 12 items over 8 warps
+  constexpr int kItems = (12 + WARPS - 1) / WARPS;  // 3 KT <= 12 items
   double2 x[kItems][4], y[kItems][4];  // points p, n - p
 #pragma unroll
   for (int u = 0; u < kItems; ++u) {
-    const int it = warp + u * kWarps;
+    const int it = warp + u * WARPS;
     if (it < 3 * KT) {
       const int f = it / KT, kt = it - f * KT, m = m0 + g;
       const double2* src = ZN + f * fstride + (long)n * nz * M + m;
@@ -505,7 +541,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __syncthreads();
 #pragma unroll
   for (int u = 0; u < kItems; ++u) {
-    const int it = warp + u * kWarps;
+    const int it = warp + u * WARPS;
     if (it < 3 * KT) {
       const int f = it / KT, kt = it - f * KT, e = emx[f][g];
       long long sr[4], si[4], dr[4], di[4];
@@ -523,12 +559,12 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
   }
   __syncthreads();
-  // 3 NT <= 12 products over 8 warps; results stay in registers until every
+  // 3 NT <= 12 products; results stay in registers until every
   // warp has read its digits
   double2 res[kItems][4];
 #pragma unroll
   for (int u = 0; u < kItems; ++u) {
-    const int it = warp + u * kWarps;
+    const int it = warp + u * WARPS;
     if (it < 3 * NT) {
       __syncwarp();
       const int f = it % 3, nt = it / 3;
@@ -549,7 +585,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __syncthreads();
 #pragma unroll
   for (int u = 0; u < kItems; ++u) {
-    const int it = warp + u * kWarps;
+    const int it = warp + u * WARPS;
     if (it < 3 * NT) {
       const int f = it % 3, nt = it / 3;
 #pragma unroll
@@ -565,7 +601,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __syncthreads();
   grid_dep_trigger_at(d, 2);
   const int mcn = min(8, M - m0);
-  for (int e = threadIdx.x; e < mcn * nk; e += kThreads) {
+  for (int e = threadIdx.x; e < mcn * nk; e += WARPS * 32) {
     const int mc = e / nk, kk = e - mc * nk;
     const double2 r = R[mc * nk + kk], th = R[(8 + mc) * nk + kk];
     double2 z = R[(16 + mc) * nk + kk];
@@ -597,27 +633,38 @@ bool dft_prepare_attrs() {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   const int lim = optin - 1024;  // (static shared memory counts too)
   return cudaFuncSetAttribute(k_dft_zsynth, a, lim) == cudaSuccess &&
-         cudaFuncSetAttribute(k_dft_product<8>, a, lim) == cudaSuccess &&
-         cudaFuncSetAttribute(k_dft_product<16>, a, lim) == cudaSuccess &&
-         cudaFuncSetAttribute(k_dft_zanalysis, a, lim) == cudaSuccess;
+         cudaFuncSetAttribute(k_dft_product<8, 3, 2>, a, lim) == cudaSuccess &&
+         cudaFuncSetAttribute(k_dft_product<8, 6, 2>, a, lim) == cudaSuccess &&
+         cudaFuncSetAttribute(k_dft_product<16, 6, 1>, a, lim) == cudaSuccess &&
+         cudaFuncSetAttribute(k_dft_zanalysis<6, 3>, a, lim) == cudaSuccess &&
+         cudaFuncSetAttribute(k_dft_zanalysis<8, 1>, a, lim) == cudaSuccess &&
+         cudaFuncSetAttribute(k_dft_zanalysis<12, 1>, a, lim) == cudaSuccess;
 }
 
 void launch_dft_zsynth(const Dims& d, const DevSetup& s, const double2* W6, double2* Z6, cudaStream_t st) {
-  launch_step_kernel(d, k_dft_zsynth, dim3((d.M + 31) / 32, d.N * 6, d.B), dim3(kThreads), dft_zsynth_smem(d), st, d,
+  const SynthShape sh = synth_shape(d);
+  launch_step_kernel(d, k_dft_zsynth, dim3(sh.blocks, 1, d.B), dim3(kThreads), dft_zsynth_smem(d), st, d, sh.R,
                      s.dft.m[0], s.dft.m[1], W6, Z6);
 }
 void launch_dft_product(const Dims& d, const DevSetup& s, const double2* Z6, double2* ZN, cudaStream_t st) {
   const dim3 g((d.nz + 15) / 16, d.N, d.B);
-  auto go = [&](auto kern, int warps) {
-    launch_step_kernel(d, kern, g, dim3(warps * 32), product_shape(d.M, d.nth, warps).smem, st, d, s.dft.m[2],
+  auto go = [&](auto kern, int warps, int fields) {
+    launch_step_kernel(d, kern, g, dim3(warps * 32), product_shape(d.M, d.nth, fields).smem, st, d, s.dft.m[2],
                        s.dft.m[3], s.dft.m[4], s.dft.m[5], (const double2*)s.tw_th, Z6, ZN);
   };
-  if ((long)g.x * g.y * g.z <= device_sms()) go(k_dft_product<16>, 16);
-  else go(k_dft_product<8>, 8);
+  if ((long)g.x * g.y * g.z <= device_sms()) go(k_dft_product<16, 6, 1>, 16, 6);
+  else if (d.M <= 16) go(k_dft_product<8, 6, 2>, 8, 6);
+  else go(k_dft_product<8, 3, 2>, 8, 3);
 }
 void launch_dft_zanalysis(const Dims& d, const DevSetup& s, const double2* ZN, double2* Nout, cudaStream_t st) {
-  launch_step_kernel(d, k_dft_zanalysis, dim3((d.M + 7) / 8, d.N, d.B), dim3(kThreads), dft_zanalysis_smem(d), st, d,
-                     s.dft.zshift, s.dft.m[6], s.dft.m[7], ZN, Nout);
+  const dim3 g((d.M + 7) / 8, d.N, d.B);
+  auto go = [&](auto kern, int warps) {
+    launch_step_kernel(d, kern, g, dim3(warps * 32), dft_zanalysis_smem(d), st, d, s.dft.zshift, s.dft.m[6],
+                       s.dft.m[7], ZN, Nout);
+  };
+  if ((long)g.x * g.y * g.z > device_sms()) go(k_dft_zanalysis<6, 3>, 6);
+  else if (3 * dft_tiles(dft_points(d.nz), 16) > 8) go(k_dft_zanalysis<12, 1>, 12);
+  else go(k_dft_zanalysis<8, 1>, 8);
 }
 
 }  // namespace opf
