@@ -1,5 +1,5 @@
 // Batched mixed-radix FFTs in shared memory (Stockham autosort, radices
-// 2, 3, 4, 5, 8), used for the Eq. 1 transforms on the 3K x 3M grid.
+// 2, 3, 4, 5, 8 and composites of them in registers), used for the Eq. 1 transforms on the 3K x 3M grid.
 //
 // A block transforms `batch` sequences of length p.n stored at stride `ld`
 // (complex elements) in buffer a, ping-ponging with buffer b; the returned
@@ -62,10 +62,85 @@ __device__ __forceinline__ void butterfly8_zm(V* v, int sign) {
   v[7] = csub(e[3], o3);
 }
 
+// cos and sin of 2 pi i / n for the compile-time twiddles below (the series; |x| <= pi).
+__host__ __device__ constexpr double turn_cos(int i, int n) {
+  const double x = 6.283185307179586476925 * (2 * i > n ? i - n : i) / n;
+  double t = 1.0, s = 1.0;
+  for (int k = 1; k < 20; ++k) {
+    t *= -x * x / ((2 * k - 1) * (2 * k));
+    s += t;
+  }
+  return s;
+}
+__host__ __device__ constexpr double turn_sin(int i, int n) {
+  const double x = 6.283185307179586476925 * (2 * i > n ? i - n : i) / n;
+  double t = x, s = x;
+  for (int k = 1; k < 20; ++k) {
+    t *= -x * x / ((2 * k) * (2 * k + 1));
+    s += t;
+  }
+  return s;
+}
+
+template <int R, typename V>
+__device__ __forceinline__ void butterfly(V* v, int sign);
+
+// v times e^{sign 2 pi i E/R}
+template <int R, int E, typename V>
+__device__ __forceinline__ V cmul_root(V v, int sign) {
+  using T = typename Scalar<V>::T;
+  if constexpr (E % R == 0) {
+    return v;
+  } else if constexpr (4 * E % R == 0) {
+    constexpr int quarter = 4 * E / R % 4;
+    if constexpr (quarter == 2) return V{-v.x, -v.y};
+    else return cmul_si(v, quarter == 1 ? sign : -sign);
+  } else {
+    constexpr T c = (T)turn_cos(E % R, R), s = (T)turn_sin(E % R, R);
+    return cmul(v, V{c, sign > 0 ? s : -s});
+  }
+}
+
+// Size P Q in registers: P-point transforms of every Q-th value, roots of
+// unity, Q-point transforms.
+template <int P, int Q, int QI, int KI, typename V>
+__device__ __forceinline__ void butterfly_roots(V (&y)[P * Q], int sign) {  // y[q P + k]
+  if constexpr (QI < Q) {
+    y[QI * P + KI] = cmul_root<P * Q, QI * KI>(y[QI * P + KI], sign);
+    if constexpr (KI + 1 < P) butterfly_roots<P, Q, QI, KI + 1>(y, sign);
+    else butterfly_roots<P, Q, QI + 1, 0>(y, sign);
+  }
+}
+template <int P, int Q, typename V>
+__device__ __forceinline__ void butterfly_pq(V* v, int sign) {
+  V y[P * Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+#pragma unroll
+    for (int i = 0; i < P; ++i) y[q * P + i] = v[q + Q * i];
+    butterfly<P>(y + q * P, sign);
+  }
+  butterfly_roots<P, Q, 0, 0>(y, sign);
+#pragma unroll
+  for (int k = 0; k < P; ++k) {
+    V z[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) z[q] = y[q * P + k];
+    butterfly<Q>(z, sign);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) v[k + P * q] = z[q];
+  }
+}
+
 template <int R, typename V>
 __device__ __forceinline__ void butterfly(V* v, int sign) {
   using T = typename Scalar<V>::T;
-  if constexpr (R == 2) {
+  if constexpr (R == 6) butterfly_pq<2, 3>(v, sign);
+  else if constexpr (R == 9) butterfly_pq<3, 3>(v, sign);
+  else if constexpr (R == 12) butterfly_pq<4, 3>(v, sign);
+  else if constexpr (R == 16) butterfly_pq<4, 4>(v, sign);
+  else if constexpr (R == 24) butterfly_pq<8, 3>(v, sign);
+  else if constexpr (R == 2) {
     const V a = v[0], b = v[1];
     v[0] = cadd(a, b);
     v[1] = csub(a, b);
@@ -268,7 +343,18 @@ __host__ __device__ constexpr bool fft_length_compiled(int n) {
 template <int N, int SIGN, bool ZERO_MID = false, typename V>
 __device__ __forceinline__ V* block_fft_c(V* a, V* b, int batch, int ld, const V* tw) {
   static_assert(fft_length_compiled(N), "no compiled plan for this length");
-  if constexpr (N == 48) return fft_stages_c<48, 1, SIGN, ZERO_MID, 4, 4, 3>(a, b, ld, batch, tw);
+  // FP32: two passes over shared memory, whose load and store pipe bounds the
+  // transforms, with radices up to 24 in registers.  Against 8 4 4 3 (length
+  // 384; 3 or 4 passes each): z synthesis 221 -> 197 us, product 504 -> 467 us,
+  // z analysis 276 -> 256 us at N = 128, 255 x 128 modes; product of groups of 8 x
+  // (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 49.0 -> 44.6 us.  FP64 has no registers for it.
+  if constexpr (sizeof(V) == sizeof(float2)) {
+    if constexpr (N == 48) return fft_stages_c<48, 1, SIGN, ZERO_MID, 8, 6>(a, b, ld, batch, tw);
+    else if constexpr (N == 72) return fft_stages_c<72, 1, SIGN, ZERO_MID, 8, 9>(a, b, ld, batch, tw);
+    else if constexpr (N == 96) return fft_stages_c<96, 1, SIGN, ZERO_MID, 8, 12>(a, b, ld, batch, tw);
+    else if constexpr (N == 192) return fft_stages_c<192, 1, SIGN, ZERO_MID, 16, 12>(a, b, ld, batch, tw);
+    else return fft_stages_c<384, 1, SIGN, ZERO_MID, 16, 24>(a, b, ld, batch, tw);
+  } else if constexpr (N == 48) return fft_stages_c<48, 1, SIGN, ZERO_MID, 4, 4, 3>(a, b, ld, batch, tw);
   else if constexpr (N == 72) return fft_stages_c<72, 1, SIGN, ZERO_MID, 8, 3, 3>(a, b, ld, batch, tw);
   else if constexpr (N == 96) return fft_stages_c<96, 1, SIGN, ZERO_MID, 8, 4, 3>(a, b, ld, batch, tw);
   else if constexpr (N == 192) return fft_stages_c<192, 1, SIGN, ZERO_MID, 8, 8, 3>(a, b, ld, batch, tw);
