@@ -23,10 +23,16 @@ template <typename V>
 __device__ __forceinline__ V cadd(V a, V b) { return V{a.x + b.x, a.y + b.y}; }
 template <typename V>
 __device__ __forceinline__ V csub(V a, V b) { return V{a.x - b.x, a.y - b.y}; }
+// Multiply-adds are written out wherever a product meets a sum, so that every
+// kernel that inlines a transform rounds alike.
+__device__ __forceinline__ float madd(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double madd(double a, double b, double c) { return fma(a, b, c); }
 template <typename V>
 __device__ __forceinline__ V cmul(V a, V b) {
-  return V{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
+  return V{madd(a.x, b.x, -(a.y * b.y)), madd(a.x, b.y, a.y * b.x)};
 }
+template <typename V, typename T>
+__device__ __forceinline__ V cmadd(T f, V a, V b) { return V{madd(f, a.x, b.x), madd(f, a.y, b.y)}; }
 // multiply by s*i (s = +-1)
 template <typename V>
 __device__ __forceinline__ V cmul_si(V a, int s) { return s > 0 ? V{-a.y, a.x} : V{a.y, -a.x}; }
@@ -49,17 +55,17 @@ __device__ __forceinline__ void butterfly8_zm(V* v, int sign) {
   V o[4] = {cadd(oa, v[7]), cadd(ob, od), csub(oa, v[7]), csub(ob, od)};
   const T h = (T)0.70710678118654752440;  // 1 / sqrt(2)
   const T s = (T)sign;
-  const V o1 = V{h * (o[1].x - s * o[1].y), h * (o[1].y + s * o[1].x)};
+  const V o1 = csub(o[1], V{s * o[1].y, -s * o[1].x});  // (times h below)
   const V o2 = cmul_si(o[2], sign);
-  const V o3 = V{-h * (o[3].x + s * o[3].y), h * (s * o[3].x - o[3].y)};
+  const V o3 = csub(V{-s * o[3].y, s * o[3].x}, o[3]);
   v[0] = cadd(e[0], o[0]);
   v[4] = csub(e[0], o[0]);
-  v[1] = cadd(e[1], o1);
-  v[5] = csub(e[1], o1);
+  v[1] = cmadd(h, o1, e[1]);
+  v[5] = cmadd(-h, o1, e[1]);
   v[2] = cadd(e[2], o2);
   v[6] = csub(e[2], o2);
-  v[3] = cadd(e[3], o3);
-  v[7] = csub(e[3], o3);
+  v[3] = cmadd(h, o3, e[3]);
+  v[7] = cmadd(-h, o3, e[3]);
 }
 
 // cos and sin of 2 pi i / n for the compile-time twiddles below (the series; |x| <= pi).
@@ -154,11 +160,11 @@ __device__ __forceinline__ void butterfly(V* v, int sign) {
   } else if constexpr (R == 3) {
     const T h = (T)0.86602540378443864676;  // sin(2 pi / 3)
     const V t1 = cadd(v[1], v[2]), t2 = csub(v[1], v[2]);
-    const V base = V{v[0].x - (T)0.5 * t1.x, v[0].y - (T)0.5 * t1.y};
-    const V rot = cmul_si(cscale(t2, h), sign);
+    const V base = cmadd((T)-0.5, t1, v[0]);
+    const V rot = cmul_si(t2, sign);
     v[0] = cadd(v[0], t1);
-    v[1] = cadd(base, rot);
-    v[2] = csub(base, rot);
+    v[1] = cmadd(h, rot, base);
+    v[2] = cmadd(-h, rot, base);
   } else if constexpr (R == 8) {
     // two radix-4 transforms of the even and odd points, joined by the
     // eighth roots of unity w^q = e^{sign 2 pi i q/8}
@@ -167,17 +173,17 @@ __device__ __forceinline__ void butterfly(V* v, int sign) {
     butterfly<4>(o, sign);
     const T h = (T)0.70710678118654752440;  // 1 / sqrt(2)
     const T s = (T)sign;
-    const V o1 = V{h * (o[1].x - s * o[1].y), h * (o[1].y + s * o[1].x)};
+    const V o1 = csub(o[1], V{s * o[1].y, -s * o[1].x});  // (times h below)
     const V o2 = cmul_si(o[2], sign);
-    const V o3 = V{-h * (o[3].x + s * o[3].y), h * (s * o[3].x - o[3].y)};
+    const V o3 = csub(V{-s * o[3].y, s * o[3].x}, o[3]);
     v[0] = cadd(e[0], o[0]);
     v[4] = csub(e[0], o[0]);
-    v[1] = cadd(e[1], o1);
-    v[5] = csub(e[1], o1);
+    v[1] = cmadd(h, o1, e[1]);
+    v[5] = cmadd(-h, o1, e[1]);
     v[2] = cadd(e[2], o2);
     v[6] = csub(e[2], o2);
-    v[3] = cadd(e[3], o3);
-    v[7] = csub(e[3], o3);
+    v[3] = cmadd(h, o3, e[3]);
+    v[7] = cmadd(-h, o3, e[3]);
   } else if constexpr (R == 5) {
     const T c1 = (T)0.30901699437494742410, c2 = (T)-0.80901699437494742410;
     const T s1 = (T)0.95105651629515357212, s2 = (T)0.58778525229247312917;
@@ -338,22 +344,60 @@ __host__ __device__ constexpr bool fft_length_compiled(int n) {
   return n == 48 || n == 72 || n == 96 || n == 192 || n == 384;
 }
 
+// The two passes of an FP32 transform: a synthesis takes r1 then r2, an
+// analysis r2 then r1, so that the points a thread gets from the last pass of
+// one are those it needs for the first pass of the other (k_product).
+struct FftRadices {
+  int r1, r2;
+};
+__host__ __device__ constexpr FftRadices fft_radices32(int n) {
+  return n == 48 ? FftRadices{8, 6} : n == 72 ? FftRadices{9, 8} : n == 96 ? FftRadices{12, 8}
+       : n == 192 ? FftRadices{16, 12} : FftRadices{24, 16};
+}
+// Butterfly j of the first pass with inputs load(i), i = j + q N / R, into the
+// sequence dst (swizzled); of the last pass (twiddles tw) from src into v, whose
+// v[q] is output j + q N / R.  The arithmetic is fft_stage_c's.
+template <int R, int N, int SIGN, bool ZM, typename V, typename Load>
+__device__ __forceinline__ void fft_first(int j, V* __restrict__ dst, Load load) {
+  constexpr bool zm = ZM && R == 8;
+  V v[R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    if (zm && (q == 3 || q == 4)) continue;
+    v[q] = load(j + q * (N / R));
+  }
+  if constexpr (zm) butterfly8_zm(v, SIGN);
+  else butterfly<R>(v, SIGN);
+#pragma unroll
+  for (int q = 0; q < R; ++q) dst[fft_swz(j * R + q)] = v[q];
+}
+template <int R, int N, int SIGN, typename V>
+__device__ __forceinline__ void fft_last(int j, const V* __restrict__ src, const V* __restrict__ tw, V (&v)[R]) {
+  v[0] = src[fft_swz(j)];
+#pragma unroll
+  for (int q = 1; q < R; ++q) {
+    V t = tw[q * j];
+    if constexpr (SIGN < 0) t.y = -t.y;
+    v[q] = cmul(src[fft_swz(j + q * (N / R))], t);
+  }
+  butterfly<R>(v, SIGN);
+}
+
 // ZERO_MID: the inputs in the middle third, positions (N/3, 2N/3), are zero
 // (a synthesis of the 3/2 rule); the radix-8 first stages then skip them.
 template <int N, int SIGN, bool ZERO_MID = false, typename V>
 __device__ __forceinline__ V* block_fft_c(V* a, V* b, int batch, int ld, const V* tw) {
   static_assert(fft_length_compiled(N), "no compiled plan for this length");
   // FP32: two passes over shared memory, whose load and store pipe bounds the
-  // transforms, with radices up to 24 in registers.  Against 8 4 4 3 (length
-  // 384; 3 or 4 passes each): z synthesis 221 -> 197 us, product 504 -> 467 us,
-  // z analysis 276 -> 256 us at N = 128, 255 x 128 modes; product of groups of 8 x
-  // (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 49.0 -> 44.6 us.  FP64 has no registers for it.
+  // transforms, with radices up to 24 in registers, where 3 or 4 passes (8 4 4 3
+  // at 384) took 221 against 197 us in the z synthesis and 504 against 467 us in
+  // the product at N = 128, 255 x 128 modes.  (Their kernels now take the same
+  // passes without the buffers; this form serves the fused launch.)  FP64 has
+  // no registers for it.
   if constexpr (sizeof(V) == sizeof(float2)) {
-    if constexpr (N == 48) return fft_stages_c<48, 1, SIGN, ZERO_MID, 8, 6>(a, b, ld, batch, tw);
-    else if constexpr (N == 72) return fft_stages_c<72, 1, SIGN, ZERO_MID, 8, 9>(a, b, ld, batch, tw);
-    else if constexpr (N == 96) return fft_stages_c<96, 1, SIGN, ZERO_MID, 8, 12>(a, b, ld, batch, tw);
-    else if constexpr (N == 192) return fft_stages_c<192, 1, SIGN, ZERO_MID, 16, 12>(a, b, ld, batch, tw);
-    else return fft_stages_c<384, 1, SIGN, ZERO_MID, 16, 24>(a, b, ld, batch, tw);
+    constexpr FftRadices r = fft_radices32(N);
+    if constexpr (SIGN > 0) return fft_stages_c<N, 1, SIGN, ZERO_MID, r.r1, r.r2>(a, b, ld, batch, tw);
+    else return fft_stages_c<N, 1, SIGN, ZERO_MID, r.r2, r.r1>(a, b, ld, batch, tw);
   } else if constexpr (N == 48) return fft_stages_c<48, 1, SIGN, ZERO_MID, 4, 4, 3>(a, b, ld, batch, tw);
   else if constexpr (N == 72) return fft_stages_c<72, 1, SIGN, ZERO_MID, 8, 3, 3>(a, b, ld, batch, tw);
   else if constexpr (N == 96) return fft_stages_c<96, 1, SIGN, ZERO_MID, 8, 4, 3>(a, b, ld, batch, tw);

@@ -296,14 +296,20 @@ static unsigned transform_threads(const dim3& g) {
 // ------------------------------------------------------------------ z synthesis (A2)
 
 // NZ > 0: the z length 3K is the compile-time constant NZ (compiled plan).
+// FP32 with a compiled plan: both passes work between registers, global memory
+// and one exchange through shared memory, whose pipe was 88 % busy with the
+// staging and every pass; half the footprint lets twice the blocks reside.
+// 197 -> 124 us at N = 128, 255 x 128 modes (500 MB, 75 us at the copy rate),
+// groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 28.7 -> 19.6 us.
 template <typename V, int NZ>
 __global__ void __launch_bounds__(256) k_zsynth(Dims d, FftPlan pz, const V* __restrict__ twz,
                                                 const V* __restrict__ W6, V* __restrict__ Z6) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nz = NZ > 0 ? NZ : d.nz, ld = nz + 1, MC = d.mcz;
+  constexpr bool kStream = NZ > 0 && sizeof(V) == sizeof(float2);
   V* A = (V*)smraw;
   V* B = A + MC * ld;
-  V* tw = B + MC * ld;
+  V* tw = kStream ? B : B + MC * ld;
   const int m0 = blockIdx.x * MC, n = blockIdx.y / 6, f = blockIdx.y % 6;
   const int K = d.K;
   twz = bofs(twz, d.ps);
@@ -313,6 +319,28 @@ __global__ void __launch_bounds__(256) k_zsynth(Dims d, FftPlan pz, const V* __r
   for (int e = threadIdx.x; e < nz; e += blockDim.x) tw[e] = twz[e];
   const long fs = d.F;
   grid_dep_wait();
+  if constexpr (kStream) {  // global to registers, one exchange through shared memory, and back
+    constexpr FftRadices r = fft_radices32(NZ > 0 ? NZ : 48);
+    const int mcn = min(MC, d.M - m0);
+    for (int w = threadIdx.x; w < mcn * (NZ / r.r1); w += blockDim.x) {
+      const int mc = w / (NZ / r.r1), j = w - mc * (NZ / r.r1);
+      const V* src = W6 + f * fs + ((long)(m0 + mc) * d.N + n) * d.nk + K - 1;
+      fft_first<r.r1, NZ, +1, true>(j, A + mc * ld, [&](int z) {
+        return z < K ? src[z] : z > NZ - K ? src[z - NZ] : V{0, 0};
+      });
+    }
+    __syncthreads();
+    grid_dep_trigger_at(d, 2);
+    V* out = Z6 + ((long)f * d.N + n) * NZ * d.M + m0;
+    for (int w = threadIdx.x; w < mcn * (NZ / r.r2); w += blockDim.x) {
+      const int j = w / mcn, mc = w - j * mcn;
+      V v[r.r2];
+      fft_last<r.r2, NZ, +1>(j, A + mc * ld, tw, v);
+#pragma unroll
+      for (int q = 0; q < r.r2; ++q) out[(long)(j + q * (NZ / r.r2)) * d.M + mc] = v[q];
+    }
+    return;
+  }
   block_copy_batched<8, V>(
       MC * nz,
       [&](int e) {
@@ -340,8 +368,9 @@ size_t zsynth_smem(const Dims& d, int mc, size_t vb) { return (2 * (size_t)mc * 
 void launch_zsynth32(const Dims& d, const DevSetup& s, const FftPlan& pz, const float2* W6,
                      float2* Z6, cudaStream_t st) {
   dim3 g((d.M + d.mcz - 1) / d.mcz, d.N * 6, d.B);
-  const size_t sm = zsynth_smem(d, d.mcz, sizeof(float2));
   with_fft_length(d.nz, [&](auto n) {
+    const size_t sm = decltype(n)::value ? (size_t)(d.mcz * (d.nz + 1) + d.nz) * sizeof(float2)
+                                         : zsynth_smem(d, d.mcz, sizeof(float2));
     launch_step_kernel(d, k_zsynth<float2, decltype(n)::value>, g, dim3(transform_threads(g)), sm, st, d, pz,
                        (const float2*)s.tw_z32, W6, Z6);
   });
@@ -364,6 +393,13 @@ __device__ __forceinline__ void sincos_pi(double x, double* s, double* c) { sinc
 __device__ __forceinline__ void sincos_pi(float x, float* s, float* c) { sincospif(x, s, c); }
 
 // NTH > 0: the theta length 3M is the compile-time constant NTH.
+// FP32 with a compiled plan (kStream): three exchanges through shared memory
+// instead of five passes with staging either side -- global memory to the first
+// pass of the syntheses; their last pass, the product and the first pass of the
+// analyses on the same points in registers; the last pass to global memory.
+// What bounds it: latency of the loads at 12 warps per SM (length 384).  N = 128,
+// 255 x 128 modes 467 -> 363 us; groups of 8 x (N = 32 .. 48) and 6 x (N = 64,
+// 63 x 32) 44.6 -> 36.3 us; N = 48, 63 x 24 modes 13.2 -> 12.6 us.
 template <typename V, int NTH>
 __global__ void __launch_bounds__(256) k_product(Dims d, FftPlan pth, const V* __restrict__ twth,
                                                  const V* __restrict__ Z6, V* __restrict__ ZN) {
@@ -375,9 +411,10 @@ __global__ void __launch_bounds__(256) k_product(Dims d, FftPlan pth, const V* _
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nth = NTH > 0 ? NTH : d.nth, ld = nth, M = d.M;
   const int ZC = d.zc;
+  constexpr bool kStream = NTH > 0 && sizeof(V) == sizeof(float2);
   V* A = (V*)smraw;            // 3 * ZC sequences
-  V* B = A + 3 * ZC * ld;      // 3 * ZC sequences
-  V* tw = B + 3 * ZC * ld;
+  V* B = A + 3 * ZC * ld;      // 3 * ZC sequences (kStream: none)
+  V* tw = kStream ? B : B + 3 * ZC * ld;
   const int z0 = blockIdx.x * ZC, n = blockIdx.y, nz = d.nz;
   const int zc = min(ZC, nz - z0);
   twth = bofs(twth, d.ps);
@@ -388,28 +425,34 @@ __global__ void __launch_bounds__(256) k_product(Dims d, FftPlan pth, const V* _
   const long fstride = (long)d.N * nz * M;
   grid_dep_wait();
   // spectra of the pairs (u_r,u_t), (u_z,w_r), (w_t,w_z):  Z = A + i B
-  block_copy_batched<8, V>(
-      zc * 3 * nth,
-      [&](int e) {
-        const int q = e % nth, pr = (e / nth) % 3, zr = e / (3 * nth);
-        const long rowa = ((long)(2 * pr) * d.N + n) * nz + z0 + zr;
-        V v = V{0, 0};
-        if (q < M) {
-          V a = Z6[rowa * M + q], b = Z6[(rowa + (long)d.N * nz) * M + q];
-          if (q == 0) { a.y = 0; b.y = 0; }
-          v = V{a.x - b.y, a.y + b.x};
-        } else if (q > nth - M) {
-          const int m = nth - q;
-          const V a = Z6[rowa * M + m], b = Z6[(rowa + (long)d.N * nz) * M + m];
-          v = V{a.x + b.y, -a.y + b.x};  // conj(a) + i conj(b)
-        }
-        return v;
-      },
-      [&](int e, V v) { A[(e / nth) * ld + e % nth] = v; });
-  __syncthreads();
-  V* res;
-  if constexpr (NTH > 0) res = block_fft_c<NTH, +1, true>(A, B, 3 * zc, ld, tw);
-  else res = block_fft(A, B, 3 * zc, ld, pth, tw, +1);
+  auto spectrum = [&](int zr, int pr, int q) {
+    const long rowa = ((long)(2 * pr) * d.N + n) * nz + z0 + zr;
+    const bool low = q < M;
+    const int m = low ? q : nth - q;
+    V a = V{0, 0}, b = V{0, 0};
+    if (low || q > nth - M) {
+      a = Z6[rowa * M + m];
+      b = Z6[(rowa + (long)d.N * nz) * M + m];
+    }
+    if (q == 0) a.y = b.y = 0;
+    return low ? V{a.x - b.y, a.y + b.x} : V{a.x + b.y, b.x - a.y};  // (mirrored: conj(a) + i conj(b))
+  };
+  V* res = nullptr;
+  constexpr FftRadices rx = fft_radices32(NTH > 0 ? NTH : 48);
+  if constexpr (kStream) {
+    for (int w = threadIdx.x; w < 3 * zc * (NTH / rx.r1); w += blockDim.x) {
+      const int bt = w / (NTH / rx.r1), j = w - bt * (NTH / rx.r1), zr = bt / 3, pr = bt - 3 * zr;
+      fft_first<rx.r1, NTH, +1, true>(j, A + bt * ld, [&](int q) { return spectrum(zr, pr, q); });
+    }
+    __syncthreads();
+  } else {
+    block_copy_batched<8, V>(
+        zc * 3 * nth, [&](int e) { return spectrum(e / (3 * nth), (e / nth) % 3, e % nth); },
+        [&](int e, V v) { A[(e / nth) * ld + e % nth] = v; });
+    __syncthreads();
+    if constexpr (NTH > 0) res = block_fft_c<NTH, +1, true>(A, B, 3 * zc, ld, tw);
+    else res = block_fft(A, B, 3 * zc, ld, pth, tw, +1);
+  }
   V* C = (res == A) ? B : A;
   // CFL number of this radial plane (optional): max over the grid of
   // |u_r|/dr, |u_t|/(r dtheta), |u_z|/dz for the TOTAL velocity (the FP32
@@ -429,31 +472,75 @@ __global__ void __launch_bounds__(256) k_product(Dims d, FftPlan pth, const V* _
     if constexpr (sizeof(T) == 4) Ubase = one - rn * rn;
   }
   T cmax = 0;
-  for (int e = threadIdx.x; e < zc * nth; e += blockDim.x) {
-    const int q = e % nth, zr = e / nth;
-    const V x0 = res[(zr * 3 + 0) * ld + q], x1 = res[(zr * 3 + 1) * ld + q], x2 = res[(zr * 3 + 2) * ld + q];
+  // u x w (with the Coriolis term) at point q from the three pairs
+  auto product = [&](int q, V x0, V x1, V x2, V* nrt, T* nzp) {
     const T ur = x0.x, ut = x0.y, uz = x1.x, wr = x1.y, wt = x2.x, wz = x2.y;
-    T nr = ut * wz - uz * wt, nt = uz * wr - ur * wz, nz = ur * wt - ut * wr;
+    T nr = madd(ut, wz, -(uz * wt)), nt = madd(uz, wr, -(ur * wz)), nz = madd(ur, wt, -(ut * wr));
     if (d.rotate) {  // Coriolis -2 Omega x u, Omega in cylindrical components at theta_q
       T sn, cs;
       sincos_pi((T)(2 * q) / (T)(d.m_p * nth), &sn, &cs);
       const T rx = (T)d.rot_x, ry = (T)d.rot_y;
-      const T o_r = rx * cs + ry * sn, o_t = -rx * sn + ry * cs;
+      const T o_r = madd(rx, cs, ry * sn), o_t = madd(ry, cs, -(rx * sn));
       const T o_z = (T)d.rot_z;
-      nr -= (T)2 * (o_t * uz - o_z * ut);
-      nt -= (T)2 * (o_z * ur - o_r * uz);
-      nz -= (T)2 * (o_r * ut - o_t * ur);
+      nr = madd((T)-2, madd(o_t, uz, -(o_z * ut)), nr);
+      nt = madd((T)-2, madd(o_z, ur, -(o_r * uz)), nt);
+      nz = madd((T)-2, madd(o_r, ut, -(o_t * ur)), nz);
     }
+    if (cfl) cmax = fmax(cmax, fmax(fabs(ur) * inv_dr, fmax(fabs(ut) * inv_rdt, fabs(uz + Ubase) * inv_dz)));
+    *nrt = V{nr, nt};
+    *nzp = nz;
+  };
+  if constexpr (kStream) {
+    // one item per thread (zc NTH / r2 <= 96): the last pass of the three
+    // syntheses, the product, and the first pass of the two analyses, which
+    // takes the same points; written back in place once all have read
+    constexpr int L = NTH / rx.r2;
+    const int zr = threadIdx.x / L, j = threadIdx.x - zr * L;
+    const bool have = zr < zc;
+    V x0[rx.r2], x1[rx.r2];
+    // (a zero the compiler cannot fold, which would let it round otherwise than
+    // the fused launch)
+    T zero = 0;
+    asm("" : "+f"(zero));
+    if (have) {
+      V x2[rx.r2];
+      fft_last<rx.r2, NTH, +1>(j, A + (zr * 3 + 0) * ld, tw, x0);
+      fft_last<rx.r2, NTH, +1>(j, A + (zr * 3 + 1) * ld, tw, x1);
+      fft_last<rx.r2, NTH, +1>(j, A + (zr * 3 + 2) * ld, tw, x2);
+#pragma unroll
+      for (int q = 0; q < rx.r2; ++q) {
+        V nrt;
+        T nzv;
+        product(j + q * L, x0[q], x1[q], x2[q], &nrt, &nzv);
+        x0[q] = nrt;
+        x1[q] = V{nzv, zero};
+      }
+      butterfly<rx.r2>(x0, -1);
+      butterfly<rx.r2>(x1, -1);
+    }
+    __syncthreads();
+    if (have) {
+#pragma unroll
+      for (int q = 0; q < rx.r2; ++q) {
+        A[zr * ld + fft_swz(j * rx.r2 + q)] = x0[q];
+        A[(zc + zr) * ld + fft_swz(j * rx.r2 + q)] = x1[q];
+      }
+    }
+  } else
+  for (int e = threadIdx.x; e < zc * nth; e += blockDim.x) {
+    const int q = e % nth, zr = e / nth;
+    V nrt;
+    T nz;
+    product(q, res[(zr * 3 + 0) * ld + q], res[(zr * 3 + 1) * ld + q], res[(zr * 3 + 2) * ld + q], &nrt, &nz);
     if constexpr (kPackNz) {  // rows zr, zr^1 share one sequence for N_z: re <- even row, im <- odd row
-      C[zr * ld + q] = V{nr, nt};
+      C[zr * ld + q] = nrt;
       T* pz = (T*)&C[(zc + (zr >> 1)) * ld + q];
       pz[zr & 1] = nz;
       if ((zc & 1) && zr == zc - 1) pz[1] = (T)0;  // the last row of an odd count has no partner
     } else {
-      C[(zr * 2 + 0) * ld + q] = V{nr, nt};
+      C[(zr * 2 + 0) * ld + q] = nrt;
       C[(zr * 2 + 1) * ld + q] = V{nz, (T)0};
     }
-    if (cfl) cmax = fmax(cmax, fmax(fabs(ur) * inv_dr, fmax(fabs(ut) * inv_rdt, fabs(uz + Ubase) * inv_dz)));
   }
   if (cfl) {  // warp max, then one atomic per warp (non-negative doubles order as integers)
     for (int o = 16; o > 0; o >>= 1) cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
@@ -462,6 +549,36 @@ __global__ void __launch_bounds__(256) k_product(Dims d, FftPlan pth, const V* _
       atomicMax((unsigned long long*)cfl, (unsigned long long)__double_as_longlong(cm));
   }
   __syncthreads();
+  if constexpr (kStream) {
+    // the last pass of the analyses: N_z goes out, N_r + i N_theta through the
+    // third of A that the products left free
+    constexpr int L = NTH / rx.r1;
+    V* Y = A + 2 * zc * ld;
+    for (int w = threadIdx.x; w < 2 * zc * L; w += blockDim.x) {
+      const int bt = w / L, j = w - bt * L;
+      V v[rx.r1];
+      fft_last<rx.r1, NTH, -1>(j, A + bt * ld, tw, v);
+      if (bt < zc) {
+#pragma unroll
+        for (int q = 0; q < rx.r1; ++q) Y[bt * ld + j + q * L] = v[q];
+      } else {
+        V* out = ZN + 2 * fstride + ((long)n * nz + z0 + bt - zc) * M;
+#pragma unroll
+        for (int q = 0; q < rx.r1; ++q)
+          if (j + q * L < M) out[j + q * L] = v[q];
+      }
+    }
+    __syncthreads();
+    grid_dep_trigger_at(d, 2);
+    for (int e = threadIdx.x; e < zc * M; e += blockDim.x) {
+      const int m = e % M, zr = e / M;
+      const V y = Y[zr * ld + m], yc = Y[zr * ld + (m == 0 ? 0 : nth - m)];
+      const long row = ((long)n * nz + z0 + zr) * M + m;
+      ZN[row] = V{(T)0.5 * (y.x + yc.x), (T)0.5 * (y.y - yc.y)};
+      ZN[fstride + row] = V{(T)0.5 * (y.y + yc.y), (T)-0.5 * (y.x - yc.x)};
+    }
+    return;
+  }
   V* D = (C == A) ? B : A;
   const V* out;
   const int nfwd = kPackNz ? zc + (zc + 1) / 2 : 2 * zc;
@@ -493,9 +610,13 @@ size_t product_smem(const Dims& d, int zc, size_t vb) { return (2 * 3 * (size_t)
 void launch_product32(const Dims& d, const DevSetup& s, const FftPlan& pth, const float2* Z6,
                       float2* ZN, cudaStream_t st) {
   dim3 g((d.nz + d.zc - 1) / d.zc, d.N, d.B);
-  const size_t sm = product_smem(d, d.zc, sizeof(float2));
   with_fft_length(d.nth, [&](auto n) {
-    launch_step_kernel(d, k_product<float2, decltype(n)::value>, g, dim3(transform_threads(g)), sm, st, d, pth,
+    const size_t sm = decltype(n)::value ? (size_t)(3 * d.zc + 1) * d.nth * sizeof(float2)
+                                         : product_smem(d, d.zc, sizeof(float2));
+    // (length 384: the 96 threads that its middle phase has work for -- 363 us at
+    // N = 128, 255 x 128 modes, with 128 435 us, with 192 587 us)
+    launch_step_kernel(d, k_product<float2, decltype(n)::value>, g,
+                       dim3(decltype(n)::value == 384 ? 96u : transform_threads(g)), sm, st, d, pth,
                        (const float2*)s.tw_th32, Z6, ZN);
   });
 }
@@ -515,6 +636,10 @@ void launch_product(const Dims& d, const DevSetup& s, const FftPlan& pth, const 
 __device__ __forceinline__ double wide(double x) { return x; }
 __device__ __forceinline__ double wide(float x) { return to_double(x); }
 
+// FP32 with a compiled plan: the first pass reads global memory itself.  N = 128,
+// 255 x 128 modes 256 -> 226 us (FP64 addends and output 41 % of the FP64 unit),
+// groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 40.3 -> 30.3 us, N = 48,
+// 63 x 24 modes 12.3 -> 11.0 us.
 template <typename V, int NZ>
 __global__ void __launch_bounds__(256) k_zanalysis(Dims d, FftPlan pz, const V* __restrict__ twz,
                                                    const V* __restrict__ ZN, const double2* __restrict__ Nlin,
@@ -561,22 +686,42 @@ __global__ void __launch_bounds__(256) k_zanalysis(Dims d, FftPlan pz, const V* 
   const bool have0 = threadIdx.x < mcn * nk;
   if (have0 && (Nlin || d.forcing)) addends(out_index(threadIdx.x), &pp, &pm, &pz0);
   const long fstride = (long)d.N * nz * M;
-  block_copy_batched<8, V>(
-      3 * MC * nz,
-      [&](int e) {
-        const int mc = e % MC, z = (e / MC) % nz, f = e / (MC * nz);
-        V v = V{0, 0};
-        if (mc < mcn) v = ZN[f * fstride + ((long)n * nz + z) * M + m0 + mc];
-        return v;
-      },
-      [&](int e, V v) {
-        const int mc = e % MC, z = (e / MC) % nz, f = e / (MC * nz);
-        A[(f * MC + mc) * ld + z] = v;
-      });
-  __syncthreads();
   const V* res;
-  if constexpr (NZ > 0) res = block_fft_c<NZ, -1>(A, B, 3 * MC, ld, tw);
-  else res = block_fft(A, B, 3 * MC, ld, pz, tw, -1);
+  if constexpr (NZ > 0 && sizeof(V) == sizeof(float2)) {  // the first pass from global memory
+    constexpr FftRadices r = fft_radices32(NZ > 0 ? NZ : 48);
+    for (int w = threadIdx.x; w < 3 * MC * (NZ / r.r2); w += blockDim.x) {
+      const int mc = w % MC, j = w / MC % (NZ / r.r2), f = w / (MC * (NZ / r.r2));
+      const V* src = ZN + f * fstride + (long)n * NZ * M + m0 + mc;
+      fft_first<r.r2, NZ, -1, false>(j, A + (f * MC + mc) * ld,
+                                     [&](int z) { return mc < mcn ? src[(long)z * M] : V{0, 0}; });
+    }
+    __syncthreads();
+    for (int w = threadIdx.x; w < 3 * MC * (NZ / r.r1); w += blockDim.x) {
+      const int bt = w / (NZ / r.r1), j = w - bt * (NZ / r.r1);
+      V v[r.r1];
+      fft_last<r.r1, NZ, -1>(j, A + bt * ld, tw, v);
+#pragma unroll
+      for (int q = 0; q < r.r1; ++q) B[bt * ld + j + q * (NZ / r.r1)] = v[q];
+    }
+    __syncthreads();
+    res = B;
+  } else {
+    block_copy_batched<8, V>(
+        3 * MC * nz,
+        [&](int e) {
+          const int mc = e % MC, z = (e / MC) % nz, f = e / (MC * nz);
+          V v = V{0, 0};
+          if (mc < mcn) v = ZN[f * fstride + ((long)n * nz + z) * M + m0 + mc];
+          return v;
+        },
+        [&](int e, V v) {
+          const int mc = e % MC, z = (e / MC) % nz, f = e / (MC * nz);
+          A[(f * MC + mc) * ld + z] = v;
+        });
+    __syncthreads();
+    if constexpr (NZ > 0) res = block_fft_c<NZ, -1>(A, B, 3 * MC, ld, tw);
+    else res = block_fft(A, B, 3 * MC, ld, pz, tw, -1);
+  }
   // scaling and the +- combination in the transform's precision, then FP64
   using T = typename Scalar<V>::T;
   const T sc = (T)d.inv_grid;
@@ -760,16 +905,16 @@ __global__ void __launch_bounds__(256) k_nl_fused32(Dims d, int C, const float2*
       const int q = e % NTH, zr = e / NTH;
       const V x0 = res[(zr * 3 + 0) * NTH + q], x1 = res[(zr * 3 + 1) * NTH + q], x2 = res[(zr * 3 + 2) * NTH + q];
       const T ur = x0.x, ut = x0.y, uz = x1.x, wr = x1.y, wt = x2.x, wz = x2.y;
-      T nr = ut * wz - uz * wt, nt = uz * wr - ur * wz, nz = ur * wt - ut * wr;
+      T nr = madd(ut, wz, -(uz * wt)), nt = madd(uz, wr, -(ur * wz)), nz = madd(ur, wt, -(ut * wr));
       if (d.rotate) {  // Coriolis -2 Omega x u, Omega in cylindrical components at theta_q
         T sn, cs;
         sincos_pi((T)(2 * q) / (T)(d.m_p * NTH), &sn, &cs);
         const T rx = (T)d.rot_x, ry = (T)d.rot_y;
-        const T o_r = rx * cs + ry * sn, o_t = -rx * sn + ry * cs;
+        const T o_r = madd(rx, cs, ry * sn), o_t = madd(ry, cs, -(rx * sn));
         const T o_z = (T)d.rot_z;
-        nr -= (T)2 * (o_t * uz - o_z * ut);
-        nt -= (T)2 * (o_z * ur - o_r * uz);
-        nz -= (T)2 * (o_r * ut - o_t * ur);
+        nr = madd((T)-2, madd(o_t, uz, -(o_z * ut)), nr);
+        nt = madd((T)-2, madd(o_z, ur, -(o_r * uz)), nt);
+        nz = madd((T)-2, madd(o_r, ut, -(o_t * ur)), nz);
       }
       Cb[(zr * 2 + 0) * NTH + q] = V{nr, nt};
       Cb[(zr * 2 + 1) * NTH + q] = V{nz, (T)0};
