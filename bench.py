@@ -64,9 +64,9 @@ def kernel_costs(w, precision=1):
     split between z (log2 3K) and theta (log2 3M) parts.  The solve counts,
     per mode and radial row: div N_eff (48), d_r p (36), right-hand sides (30),
     final update and influence correction (36), and 8 real banded
-    substitutions (2 nl + 2 nu + 1 each, nl/nu the row's band widths).  In FP64
-    steps the solve launches also take the curl of their output (A1) for the
-    next nonlinear evaluation, so their cost includes the curl's."""
+    substitutions (2 nl + 2 nu + 1 each, nl/nu the row's band widths).  The
+    stencils (48 + 36, and 72 per point of the curl) are digit products on the
+    tensor cores; they are counted as the operations they stand for."""
     N, K, M = w["N"], w["K"], w["M"]
     nz, nth, nk = 3 * K, 3 * M, 2 * K - 1
     n = nz * nth
@@ -82,15 +82,14 @@ def kernel_costs(w, precision=1):
         "zsynth": {"flops": 6 * N * 2.5 * n * lz, "bytes": 16 * (6 * F + 6 * P)},
         "product": {"flops": 9 * N * 2.5 * n * lt + 9 * N * n, "bytes": 16 * (6 * P + 3 * P)},
         "zanalysis": {"flops": 3 * N * 2.5 * n * lz, "bytes": 16 * (3 * P + 3 * F)},
-        "solve": {"flops": solve + (F * (2 * 9 * 4 + 30) if precision == 0 else 0),
-                  "bytes": 16 * (3 * F * 3 + 3 * F + (6 * F if precision == 0 else 0))},
+        "solve": {"flops": solve, "bytes": 16 * (3 * F * 3 + 3 * F)},
     }
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the current
 # kernels on the medium workload (one ncu capture each, summarised in the
 # named profile), keyed by (kernel, precision of the step)
-PROFILED_DRAM_BYTES = {("solve", 1): 20.78e6}  # kernels changed since a capture are left out
+PROFILED_DRAM_BYTES = {}  # kernels changed since a capture are left out
 PROFILE_FILES = {"solve": "profiles/k_solve_medium.md", "product": "profiles/transforms_medium.md"}
 
 
@@ -967,9 +966,8 @@ def run_gpu(args, w):
                "small_workload_100_steps": {"seconds": small["seconds"], "cores": 1,
                                             "timesteps_per_s": 100.0 / small["seconds"]},
                "large_workload": LARGE_ORACLE_NOTE}
-    # per pass: curl + 3 transform kernels + solve (mixed); FP64 steps take
-    # the curl inside the solve
-    launches_per_step = (5 if args.precision == 1 else 4) * 2
+    # per pass: curl + 3 transform kernels + solve
+    launches_per_step = 5 * 2
     line = {
         "metric": METRIC,
         "value": value,

@@ -397,7 +397,8 @@ __device__ __forceinline__ void sincos_pi(float x, float* s, float* c) { sincosp
 // instead of five passes with staging either side -- global memory to the first
 // pass of the syntheses; their last pass, the product and the first pass of the
 // analyses on the same points in registers; the last pass to global memory.
-// What bounds it: latency of the loads at 12 warps per SM (length 384).  N = 128,
+// What bounds it: barriers between the phases and instruction fetch, at 12 warps
+// per SM (length 384).  N = 128,
 // 255 x 128 modes 467 -> 363 us; groups of 8 x (N = 32 .. 48) and 6 x (N = 64,
 // 63 x 32) 44.6 -> 36.3 us; N = 48, 63 x 24 modes 13.2 -> 12.6 us.
 template <typename V, int NTH>
