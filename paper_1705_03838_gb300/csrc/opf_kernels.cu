@@ -299,7 +299,7 @@ static unsigned transform_threads(const dim3& g) {
 // FP32 with a compiled plan: both passes work between registers, global memory
 // and one exchange through shared memory, whose pipe was 88 % busy with the
 // staging and every pass; half the footprint lets twice the blocks reside.
-// 197 -> 124 us at N = 128, 255 x 128 modes (500 MB, 75 us at the copy rate),
+// 197 -> 113 us at N = 128, 255 x 128 modes (500 MB, 75 us at the copy rate),
 // groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 28.7 -> 19.6 us.
 template <typename V, int NZ>
 __global__ void __launch_bounds__(256) k_zsynth(Dims d, FftPlan pz, const V* __restrict__ twz,
@@ -371,7 +371,10 @@ void launch_zsynth32(const Dims& d, const DevSetup& s, const FftPlan& pz, const 
   with_fft_length(d.nz, [&](auto n) {
     const size_t sm = decltype(n)::value ? (size_t)(d.mcz * (d.nz + 1) + d.nz) * sizeof(float2)
                                          : zsynth_smem(d, d.mcz, sizeof(float2));
-    launch_step_kernel(d, k_zsynth<float2, decltype(n)::value>, g, dim3(transform_threads(g)), sm, st, d, pz,
+    // (length 384: its 128 and 192 butterflies in two rounds of 96 each, 124 -> 113 us
+    // at N = 128, 255 x 128 modes; for shorter lengths it changed no step)
+    launch_step_kernel(d, k_zsynth<float2, decltype(n)::value>, g,
+                       dim3(decltype(n)::value == 384 ? 96u : transform_threads(g)), sm, st, d, pz,
                        (const float2*)s.tw_z32, W6, Z6);
   });
 }
@@ -638,7 +641,7 @@ __device__ __forceinline__ double wide(double x) { return x; }
 __device__ __forceinline__ double wide(float x) { return to_double(x); }
 
 // FP32 with a compiled plan: the first pass reads global memory itself.  N = 128,
-// 255 x 128 modes 256 -> 226 us (FP64 addends and output 41 % of the FP64 unit),
+// 255 x 128 modes 256 -> 178 us (with the threads of its launch rule),
 // groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 40.3 -> 30.3 us, N = 48,
 // 63 x 24 modes 12.3 -> 11.0 us.
 template <typename V, int NZ>
@@ -780,7 +783,10 @@ void launch_zanalysis32(const Dims& d, const DevSetup& s, const FftPlan& pz, con
   dim3 g((d.M + d.mca - 1) / d.mca, d.N, d.B);
   const size_t sm = zanalysis_smem(d, d.mca, sizeof(float2));
   with_fft_length(d.nz, [&](auto n) {
-    launch_step_kernel(d, k_zanalysis<float2, decltype(n)::value>, g, dim3(transform_threads(g)), sm, st, d, pz,
+    // (length 384: its 576 and 384 butterflies in 3 and 2 rounds of 192, 226 -> 178 us
+    // at N = 128, 255 x 128 modes; 256 threads 192 us, 96 237 us)
+    launch_step_kernel(d, k_zanalysis<float2, decltype(n)::value>, g,
+                       dim3(decltype(n)::value == 384 ? 192u : transform_threads(g)), sm, st, d, pz,
                        (const float2*)s.tw_z32, ZN, Nlin, Nout);
   });
 }
