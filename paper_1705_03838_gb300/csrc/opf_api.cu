@@ -650,7 +650,7 @@ int tune_group(Runner* r, Group* g) {
   best = 1e30f;
   pick = d.zc;
   for (int c : cand) {
-    if (c > d.nz || opf::product_smem(d, c, vb) > (size_t)optin) continue;
+    if (c > d.nz || !opf::product_fits(d, c, vb, (size_t)optin)) continue;
     d.zc = c;
     const float t = time_launch(r, [&] {
       if (mixed) opf::launch_product32(d, g->ds, g->pth, g->Z6f, g->ZNf, st);
@@ -1193,6 +1193,26 @@ int opf_set_option(opf_t* h, const char* key, double v) {
     return OPF_OK;
   }
   return runner_option(&h->run, key, v);
+}
+
+// For tests (not part of opf.h): sets the transforms' launch shapes to one the
+// autotuner may choose, whose block fits in shared memory.
+int opf_test_launch_shape(opf_t* h, int mcz, int zc, int mca) {
+  if (check_handle(h)) return OPF_EINVAL;
+  opf::Dims& d = h->g.d;
+  const size_t vb = h->run.precision == 1 ? sizeof(float2) : sizeof(double2);
+  int dev = 0, optin = 0;
+  CU(cudaGetDevice(&dev));
+  CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  if (mcz < 1 || mcz > d.M || opf::zsynth_smem(d, mcz, vb) > (size_t)optin || zc < 1 || zc > d.nz ||
+      !opf::product_fits(d, zc, vb, (size_t)optin) || mca < 1 || mca > d.M ||
+      opf::zanalysis_smem(d, mca, vb) > (size_t)optin)
+    return fail(OPF_EINVAL, "launch shape does not fit");
+  d.mcz = mcz;
+  d.zc = zc;
+  d.mca = mca;
+  h->run.drop_graph();
+  return OPF_OK;
 }
 
 int opf_get_option(opf_t* h, const char* key, double* v) {

@@ -135,6 +135,7 @@ bool prepare_nonlinear_attrs(const Dims& d);  // FP64 nonlinear-term kernels onl
 size_t zsynth_smem(const Dims& d, int mc, size_t vb);
 size_t zanalysis_smem(const Dims& d, int mc, size_t vb);
 size_t product_smem(const Dims& d, int zc, size_t vb);
+bool product_fits(const Dims& d, int zc, size_t vb, size_t smem);
 size_t solve_smem_bytes(int N, int T);
 void set_last_error(const std::string& m);  // text returned by opf_last_error()
 

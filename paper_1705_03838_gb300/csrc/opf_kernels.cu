@@ -495,9 +495,11 @@ __global__ void __launch_bounds__(256) k_product(Dims d, FftPlan pth, const V* _
     *nzp = nz;
   };
   if constexpr (kStream) {
-    // one item per thread (zc NTH / r2 <= 96): the last pass of the three
-    // syntheses, the product, and the first pass of the two analyses, which
-    // takes the same points; written back in place once all have read
+    // one item per thread (product32_items, which the launch gives threads for
+    // at every zc; a loop over rounds of rows took 0.55 ms longer per step at
+    // N = 128, 255 x 128 modes): the last pass of the three syntheses, the
+    // product, and the first pass of the two analyses, which takes the same
+    // points; written back in place once all have read
     constexpr int L = NTH / rx.r2;
     const int zr = threadIdx.x / L, j = threadIdx.x - zr * L;
     const bool have = zr < zc;
@@ -611,16 +613,27 @@ __global__ void __launch_bounds__(256) k_product(Dims d, FftPlan pth, const V* _
 
 size_t product_smem(const Dims& d, int zc, size_t vb) { return (2 * 3 * (size_t)zc * d.nth + d.nth) * vb; }
 
+// The streamed FP32 product's middle phase has one item per thread, this many
+// of them with zc rows per block (0: the length has no compiled plan).
+static int product32_items(const Dims& d, int zc) {
+  return fft_length_compiled(d.nth) ? zc * (d.nth / fft_radices32(d.nth).r2) : 0;
+}
+// Whether a block may take zc rows: its shared memory, and a thread per item.
+bool product_fits(const Dims& d, int zc, size_t vb, size_t smem) {
+  return product_smem(d, zc, vb) <= smem && (vb != sizeof(float2) || product32_items(d, zc) <= 256);
+}
+
 void launch_product32(const Dims& d, const DevSetup& s, const FftPlan& pth, const float2* Z6,
                       float2* ZN, cudaStream_t st) {
   dim3 g((d.nz + d.zc - 1) / d.zc, d.N, d.B);
   with_fft_length(d.nth, [&](auto n) {
     const size_t sm = decltype(n)::value ? (size_t)(3 * d.zc + 1) * d.nth * sizeof(float2)
                                          : product_smem(d, d.zc, sizeof(float2));
-    // (length 384: the 96 threads that its middle phase has work for -- 363 us at
-    // N = 128, 255 x 128 modes, with 128 435 us, with 192 587 us)
+    // (length 384: the 96 threads that its middle phase has work for at 4 rows --
+    // 363 us at N = 128, 255 x 128 modes, with 128 435 us, with 192 587 us)
+    const unsigned items = ((unsigned)product32_items(d, d.zc) + 31) / 32 * 32;
     launch_step_kernel(d, k_product<float2, decltype(n)::value>, g,
-                       dim3(decltype(n)::value == 384 ? 96u : transform_threads(g)), sm, st, d, pth,
+                       dim3(std::max(items, decltype(n)::value == 384 ? 96u : transform_threads(g))), sm, st, d, pth,
                        (const float2*)s.tw_th32, Z6, ZN);
   });
 }
