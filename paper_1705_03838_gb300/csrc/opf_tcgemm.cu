@@ -77,26 +77,30 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
       : "memory");
 }
 
-// Wait for the phase of the given parity to complete; false after kWaitNs.
+// Wait for the phase of the given parity to complete; false after limit_ns.
+// Called by a whole warp, and one verdict for all its lanes: each lane has its
+// own last try and clock, and a warp that split over them would reach the
+// elected instructions, which take all lanes, in parts.
 // try_wait suspends the thread in hardware for a while; the clock is read on
 // one try in 64 only (reading it before every wait, and sleeping between
 // tests, was most of a K block's time).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns = kWaitNs) {
   unsigned long long t0 = 0;
+  uint32_t done = 0;
   for (unsigned tries = 1;; ++tries) {
-    uint32_t done;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
         : "=r"(done)
         : "r"(bar), "r"(parity)
         : "memory");
-    if (done) return true;
+    if (done) break;
     if ((tries & 63u) == 0) {
       const unsigned long long t = now_ns();
       if (t0 == 0) t0 = t;
-      else if (t - t0 > kWaitNs) return false;
+      else if (t - t0 > limit_ns) break;
     }
   }
+  return __all_sync(0xffffffffu, done);
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
@@ -345,6 +349,19 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
+// For tests: a warp waits with a limit of a millisecond, its first done_lanes
+// lanes for a phase that is complete, the others for one that nothing completes.
+__global__ void k_wait_verdict(int done_lanes, int* verdict) {
+  __shared__ uint64_t bars[2];
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&bars[0]), 1);
+    mbar_init(smem_u32(&bars[1]), 1);
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bars[0])) : "memory");
+  }
+  __syncwarp();
+  verdict[threadIdx.x] = mbar_wait(smem_u32(&bars[(int)threadIdx.x < done_lanes ? 0 : 1]), 0, 1000000ull);
+}
+
 // out[m][n] (row stride ldo) = sum over splits, in split order, of part[z][m][n]
 __global__ void k_split_sum(const float* __restrict__ part, int nsplit, int M, int N, float* __restrict__ out,
                             long ldo) {
@@ -487,3 +504,13 @@ int tc_gemm_columns(const void* A, long lda, const void* B, long ldb, int M, int
 }
 
 }  // namespace opf
+
+// For tests (not part of opf.h): the 32 lanes' verdicts of k_wait_verdict.
+extern "C" int opf_test_wait_verdict(int done_lanes, int* verdict) {
+  int* dev = nullptr;
+  if (cudaMalloc(&dev, 32 * sizeof(int)) != cudaSuccess) return OPF_ENOMEM;
+  opf::k_wait_verdict<<<1, 32>>>(done_lanes, dev);
+  const cudaError_t err = cudaMemcpy(verdict, dev, 32 * sizeof(int), cudaMemcpyDeviceToHost);
+  cudaFree(dev);
+  return err == cudaSuccess ? OPF_OK : OPF_ECUDA;
+}
