@@ -1884,9 +1884,8 @@ bool prepare_kernel_attrs(const Dims& d) {
 
 // Shared-memory limits of the FP64 nonlinear-term kernels only (z synthesis,
 // theta product, z analysis) for the allocation-free entry point: checks their
-// footprints against the opt-in limit and raises their dynamic shared-memory
-// limit to it.  The radial resolution it accepts is that of a block which
-// keeps four columns of the curl (N <= 968), although k_curl itself needs none.
+// footprints, which do not depend on N, against the opt-in limit and raises
+// their dynamic shared-memory limit to it.
 bool prepare_nonlinear_attrs(const Dims& d) {
   const size_t vb = sizeof(double2);
   int dev = 0, optin = 0;
@@ -1894,9 +1893,7 @@ bool prepare_nonlinear_attrs(const Dims& d) {
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
     return false;
   const size_t lim = (size_t)optin;
-  const size_t cols = (size_t)d.M * d.nk, blocks = (cols + 3) / 4, kc = (cols + blocks - 1) / blocks;
-  if (zsynth_smem(d, d.mcz, vb) > lim || zanalysis_smem(d, d.mca, vb) > lim ||
-      product_smem(d, d.zc, vb) > lim || (size_t)d.N * (56 * kc + 16) + 16 * kc > lim)
+  if (zsynth_smem(d, d.mcz, vb) > lim || zanalysis_smem(d, d.mca, vb) > lim || product_smem(d, d.zc, vb) > lim)
     return false;
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   bool ok = dft_prepare_attrs();
@@ -1910,6 +1907,18 @@ bool prepare_nonlinear_attrs(const Dims& d) {
     ok = ok && cudaFuncSetAttribute(k_product<double2, L>, a, optin) == cudaSuccess;
   });
   return ok;
+}
+
+// The radial resolution that entry point accepts: that of a block which keeps
+// up to four columns of the curl (N <= 968 with four), although k_curl itself
+// needs no shared memory.
+bool nonlinear_radial_fits(const Dims& d) {
+  int dev = 0, optin = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+    return false;
+  const size_t cols = (size_t)d.M * d.nk, blocks = (cols + 3) / 4, kc = (cols + blocks - 1) / blocks;
+  return (size_t)d.N * (56 * kc + 16) + 16 * kc <= (size_t)optin;
 }
 
 void launch_solve(const Dims& d, const DevSetup& s, const SolveArgs& a, int nJ, cudaStream_t st) {

@@ -209,6 +209,9 @@ extern "C" int opf_nonlinear_noalloc(int N, int K, int M, int m_p, double alpha,
                               "cannot be read); this call synchronises its stream and cannot run inside a capture");
     }
   }
+  // (on every call: what the transforms need is checked once per pair of lengths)
+  if (!opf::nonlinear_radial_fits(d))
+    return fail(OPF_EINVAL, "opf_nonlinear_noalloc: resolution needs more shared memory than a block has");
   if (!g_scratch_addr[dev]) {  // once per device, with that device current
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
