@@ -139,9 +139,12 @@ __global__ void __launch_bounds__(kPoolThreads) k_pool_head(const bf16* __restri
 // Gradient tiles: a block takes 32 rows x 64 columns, thread (tx, ty) columns
 // 2 tx, 2 tx + 1 of rows ty, ty + 8, ..; column sums (bias gradients) of the
 // block go to csum[block row][C], added up by k_bias_sum in a fixed order.
-constexpr int kGradRows = 32;
+// Blocks along one grid axis, a row's tiles next to one another (the other
+// axes end at 65,535).
+constexpr int kGradRows = 32, kGradCols = 64;
+int grad_tiles(int C) { return (C + kGradCols - 1) / kGradCols; }
 
-__device__ __forceinline__ void grad_column_sums(float s0, float s1, int c, int C, float* csum) {
+__device__ __forceinline__ void grad_column_sums(float s0, float s1, long row, int c, int C, float* csum) {
   __shared__ float2 part[8][32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   part[ty][tx] = make_float2(s0, s1);
@@ -151,8 +154,8 @@ __device__ __forceinline__ void grad_column_sums(float s0, float s1, int c, int 
       s0 += part[q][tx].x;
       s1 += part[q][tx].y;
     }
-    if (c < C) csum[(long)blockIdx.y * C + c] = s0;
-    if (c + 1 < C) csum[(long)blockIdx.y * C + c + 1] = s1;
+    if (c < C) csum[row * C + c] = s0;
+    if (c + 1 < C) csum[row * C + c + 1] = s1;
   }
 }
 
@@ -182,12 +185,13 @@ __global__ void __launch_bounds__(256) k_out_grad(const float* __restrict__ y, c
                                                   int L, int C, float scale, bf16* __restrict__ dz, long ldz,
                                                   bf16* __restrict__ dzcol, long ldc, float* __restrict__ csum,
                                                   double* __restrict__ sum) {
-  const int c = blockIdx.x * 64 + 2 * (threadIdx.x & 31);
+  const int tiles = (C + kGradCols - 1) / kGradCols, row = blockIdx.x / tiles;
+  const int c = (blockIdx.x - row * tiles) * kGradCols + 2 * (threadIdx.x & 31);
   double acc = 0.0;
   float s0 = 0.f, s1 = 0.f;
 #pragma unroll
   for (int q = 0; q < kGradRows / 8; ++q) {
-    const long m = (long)blockIdx.y * kGradRows + q * 8 + (threadIdx.x >> 5);
+    const long m = (long)row * kGradRows + q * 8 + (threadIdx.x >> 5);
     if (m >= BL || c >= C) continue;
     const long i = m * C + c;
     const float r0 = y[i] - t[i], r1 = c + 1 < C ? y[i + 1] - t[i + 1] : 0.f;
@@ -198,7 +202,7 @@ __global__ void __launch_bounds__(256) k_out_grad(const float* __restrict__ y, c
     s1 += g1;
     put_grad(g0, g1, m, c, C, L, dz, ldz, dzcol, ldc);
   }
-  grad_column_sums(s0, s1, c, C, csum);
+  grad_column_sums(s0, s1, row, c, C, csum);
   __shared__ double sh[8];
   for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
@@ -215,12 +219,13 @@ __global__ void __launch_bounds__(256) k_hidden_grad(const float* __restrict__ d
                                                      const float* __restrict__ pre, int BL, int L, int C,
                                                      const float* __restrict__ dpool, bf16* __restrict__ dz, long ldz,
                                                      bf16* __restrict__ dzcol, long ldc, float* __restrict__ csum) {
-  const int c = blockIdx.x * 64 + 2 * (threadIdx.x & 31);
+  const int tiles = (C + kGradCols - 1) / kGradCols, row = blockIdx.x / tiles;
+  const int c = (blockIdx.x - row * tiles) * kGradCols + 2 * (threadIdx.x & 31);
   const long total = (long)BL * C;
   float s0 = 0.f, s1 = 0.f;
 #pragma unroll
   for (int q = 0; q < kGradRows / 8; ++q) {
-    const long m = (long)blockIdx.y * kGradRows + q * 8 + (threadIdx.x >> 5);
+    const long m = (long)row * kGradRows + q * 8 + (threadIdx.x >> 5);
     if (m >= BL || c >= C) continue;
     const long i = m * C + c;
     float v[2] = {0.f, 0.f};
@@ -236,18 +241,19 @@ __global__ void __launch_bounds__(256) k_hidden_grad(const float* __restrict__ d
     s1 += v[1];
     put_grad(v[0], v[1], m, c, C, L, dz, ldz, dzcol, ldc);
   }
-  grad_column_sums(s0, s1, c, C, csum);
+  grad_column_sums(s0, s1, row, c, C, csum);
 }
 
-// head, dz = 2 zscale (z - tz).  Grid y < O: dWh[o][c] = sum_b dz[b][o]
-// pooled[b][c], dbh[o] and sum (z - tz)^2; then one grid row per sample:
-// dpool[b][c] = sum_o dz[b][o] Wh[o][c] / L.
+// head, dz = 2 zscale (z - tz).  A row of 128-channel blocks for each output o:
+// dWh[o][c] = sum_b dz[b][o] pooled[b][c], dbh[o] and sum (z - tz)^2; then one
+// for each sample: dpool[b][c] = sum_o dz[b][o] Wh[o][c] / L.
 __global__ void __launch_bounds__(128) k_head_grad(const float* __restrict__ z, const float* __restrict__ tz,
                                                    float zscale, const float* __restrict__ pooled,
                                                    const float* __restrict__ Wh, int B, int L, int C, int O,
                                                    float* __restrict__ dWh, float* __restrict__ dbh,
                                                    float* __restrict__ dpool, double* __restrict__ sum) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x, o = blockIdx.y;
+  const int per = (C + 127) / 128, o = blockIdx.x / per, cb = blockIdx.x - o * per;
+  const int c = cb * 128 + threadIdx.x;
   if (o >= O) {
     const long b = o - O;
     if (c >= C) return;
@@ -270,7 +276,7 @@ __global__ void __launch_bounds__(128) k_head_grad(const float* __restrict__ z, 
     }
   }
   if (c < C) dWh[(long)o * C + c] = s;
-  if (blockIdx.x == 0 && threadIdx.x < 32) {  // one warp per output
+  if (cb == 0 && threadIdx.x < 32) {  // one warp per output
     double acc = 0.0;
     float t = 0.f;
     for (int b = threadIdx.x; b < B; b += 32) {
@@ -497,13 +503,13 @@ int net_gradients(opf_net* n, const float* x, const float* ty, const float* tz, 
     return r;
   };
   auto hidden = [&](const float* pre, bool head, bf16* dzcol, float* csum) {
-    k_hidden_grad<<<dim3((unsigned)((H + 63) / 64), (unsigned)rows), 256, 0, n->st>>>(
+    k_hidden_grad<<<(unsigned)grad_tiles(H) * rows, 256, 0, n->st>>>(
         dh, nsplit, pre, (int)BL, L, H, head ? n->dpool : nullptr, n->dz, ldz, dzcol, K2, csum);
   };
   // layer 3 (linear): dZ = dL/dy = 2 (y - ty) / (BL Ci); head: dL/dz = 2 lambda (z - tz) / (B O)
-  k_out_grad<<<dim3((unsigned)((Ci + 63) / 64), (unsigned)rows), 256, 0, n->st>>>(
+  k_out_grad<<<(unsigned)grad_tiles(Ci) * rows, 256, 0, n->st>>>(
       n->y, ty, (int)BL, L, Ci, 1.f / (float)(BL * Ci), n->dz, ldz, n->dzcol[1], K1, cs3, n->sums);
-  k_head_grad<<<dim3((unsigned)((H + 127) / 128), (unsigned)(O + B)), 128, 0, n->st>>>(
+  k_head_grad<<<(unsigned)((H + 127) / 128) * (unsigned)(O + B), 128, 0, n->st>>>(
       n->z, tz, zscale, n->pooled, Pf(n, 6), B, L, H, O, Gf(n, 6), Gf(n, 7), n->dpool, n->sums + 1);
   if ((rc = weights(n->col[2], K2, H, Ci, Gf(n, 4)))) return rc;
   if ((rc = inputs(n->dzcol[1], n->ws[1], H, (int)K1))) return rc;
