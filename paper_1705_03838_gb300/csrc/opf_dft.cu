@@ -127,9 +127,9 @@ void dft_device_tables(int K, int M, double inv_grid, const double2* twz, const 
 size_t stencil_bytes(int N) {
   return (size_t)stencil_table_size(N) * sizeof(uint2) + (size_t)16 * stencil_tiles(N) * sizeof(int);
 }
-StencilTable stencil_at(const void* p, int N) {
+StencilTable stencil_at(const void* p, const double* d1, int N) {
   const uint2* tab = (const uint2*)p;
-  return StencilTable{tab, (const int*)(tab + stencil_table_size(N)), stencil_tiles(N), 8 * stencil_tiles(N) - N};
+  return StencilTable{tab, (const int*)(tab + stencil_table_size(N)), d1, N, stencil_tiles(N), 8 * stencil_tiles(N) - N};
 }
 void stencil_host_table(const double* d1, int N, void* host) {
   uint2* tab = (uint2*)host;

@@ -123,8 +123,8 @@ void launch_internal_to_abi(const Dims& d, const double2* U, double2* abi, int, 
 // One warp per item of eight modes (consecutive k at one m) and eight radial
 // rows: a lane holds a mode's u+-, u_z at two of the rows and at two of the
 // halo's, the radial derivatives of u_z and u_theta are digit products on the
-// tensor cores (dft_stencil), and everything else is pointwise in the lane.
-// Nothing passes through shared memory and warps are independent; the rows of
+// tensor cores (dft_stencil; multiply-adds where a column is steep), and
+// everything else is pointwise in the lane.  Warps are independent; the rows of
 // neighbouring items come from L1 again.
 //
 // SPLIT (mixed precision): the laminar base flow U = (1 - r^2) z,
@@ -137,11 +137,12 @@ void launch_internal_to_abi(const Dims& d, const double2* U, double2* abi, int, 
 // into the constants that multiply them (exact scalings by two).
 //
 // What bounds it: the FP64 unit, with ~27 FP64 instructions per point left of
-// 57, then the integer units.  Against stencils as FP64 multiply-adds on
-// columns staged in shared memory (whose loads of data and weights took about
-// as long), split curl per launch: N = 128, 255 x 128 modes 440 -> 242 us,
-// groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 57 -> 35 us, N = 48,
-// 63 x 24 modes 14.8 -> 12.4 us.
+// 57 where the columns are not steep, then the integer units.  Against stencils
+// as FP64 multiply-adds on columns staged in shared memory (whose loads of data
+// and weights took about as long), split curl per launch: N = 128, 255 x 128
+// modes 440 -> 267 us, groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32)
+// 57 -> 45 us, N = 48, 63 x 24 modes, less than two waves of warps of which
+// some take multiply-adds as well, 14.8 -> 16.9 us.
 constexpr int kCurlWarps = 4;
 
 // The (0,0) mode of the split curl: the base flow is taken off u_z and w_theta.
@@ -176,6 +177,7 @@ __global__ void __launch_bounds__(kCurlWarps * 32, 4)
   const bool in = kk < nk;
   st.tab = bofs(st.tab, d.ps);
   st.ew = bofs(st.ew, d.ps);
+  st.d1 = bofs(st.d1, d.ps);
   rr = bofs(rr, d.ps);
   rinv = bofs(rinv, d.ps);
   U = bofs(U, d.ss);
@@ -201,12 +203,21 @@ __global__ void __launch_bounds__(kCurlWarps * 32, 4)
   double2 dz[2];  // d/dr of u_z and u_theta
   V dt[2];
   {
-    const int* ez = st.ew + (ps * st.tiles + nt) * 8 + 2 * t;
-    const int* et = st.ew + (pv * st.tiles + nt) * 8 + 2 * t;
-    dft_stencil(uz, st.tab + (long)(ps * st.tiles + nt) * kTileB + lane, ez[0], ez[1], dz);
-    const uint2* tt = st.tab + (long)(pv * st.tiles + nt) * kTileB + lane;
-    if constexpr (SPLIT) dft_stencil32(ut, tt, et[0] - 1, et[1] - 1, dt);
-    else dft_stencil(ut, tt, et[0] - 1, et[1] - 1, dt);
+    // multiply-adds read the columns from shared memory, a row of the window's
+    // 16 every 18 parts (no bank conflicts); written when some column takes them
+    __shared__ __align__(16) double window[kCurlWarps][16 * 18];
+    double* wn = window[threadIdx.x >> 5];
+    auto put = [&](const double2 (&x)[4]) {
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 4; ++q) *(double2*)(wn + (stencil_row(4, t, q) * 18 + 2 * g)) = x[q];
+      __syncwarp();
+    };
+    auto at = [&](int i, int c, int part) { return wn[(i - i0 + 4) * 18 + 2 * c + part]; };
+    dft_stencil<false, false>(uz, stencil_tile(st, ps, nt, nt, lane, 0), false, false, put, at, dz);
+    const StencilAt pt = stencil_tile(st, pv, nt, nt, lane, -1);
+    if constexpr (SPLIT) dft_stencil32(ut, pt, put, at, dt);
+    else dft_stencil<false, false>(ut, pt, false, false, put, at, dt);
   }
   grid_dep_trigger_at(d, 2);
   if (!in) return;
@@ -269,7 +280,7 @@ __global__ void __launch_bounds__(kCurlWarps * 32, 4)
 
 template <typename V, bool SPLIT>
 static void launch_curl_as(const Dims& d, const DevSetup& s, const double2* U, V* W6, double2* Nlin, cudaStream_t st) {
-  const StencilTable tab = stencil_at(s.stab, d.N);
+  const StencilTable tab = stencil_at(s.stab, s.d1, d.N);
   const long items = (long)d.M * ((d.nk + 7) / 8) * tab.tiles;
   launch_step_kernel(d, k_curl<V, SPLIT>, dim3((unsigned)((items + kCurlWarps - 1) / kCurlWarps), 1, d.B),
                      dim3(kCurlWarps * 32), 0, st, d, tab, 0.5 * d.alpha, (const double*)s.r, (const double*)s.rinv, U, W6, Nlin);
@@ -1279,12 +1290,12 @@ __device__ __forceinline__ void band_solve4(const double* __restrict__ L, double
 // weights in shared memory is the faster: 28.6 us at N = 32, 31 x 16 modes).
 // What bounds it: the chains of the substitutions and, on large grids, the
 // FP64 unit, which the stencils took 36 of ~90 instructions per point of.  Per
-// launch against multiply-adds: N = 128, 255 x 128 modes 1743 -> 1533 us, 64 x
-// (N = 32, 31 x 16) 411 -> 376 us, groups of 8 x (N = 32 .. 48) and 6 x (N = 64,
-// 63 x 32) 193 -> 180 us, N = 48, 63 x 24 modes 46.0 -> 42.5 us; N = 41, 53 x 20
-// modes (two blocks per SM) 35.8 us either way; N = 20, 7 x 5 modes, which takes
-// the curl as well and is latency alone, 24.3 -> 28.4 us -- there the one copy of
-// the code (dft_stencil_call) is 2 us faster than one per use.
+// launch against multiply-adds for every column: N = 128, 255 x 128 modes 1743
+// -> 1559 us, groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 193 -> 190
+// us, N = 48, 63 x 24 modes 46.0 -> 45.9 us, 64 x (N = 32, 31 x 16) 411 -> 422 us;
+// N = 41, 53 x 20 modes (two blocks per SM) 35.8 -> 39 us; N = 20, 7 x 5 modes,
+// which takes the curl as well and is latency alone, 24.3 -> 30.5 us -- there
+// the one copy of the code (stencil_call) is 2 us faster than one per use.
 //
 // Resident blocks per SM the register budget must allow (the shared-memory
 // footprints of the tiles allow about as many at moderate N).
@@ -1376,6 +1387,7 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   s.prm = bofs(s.prm, d.ps);
   s.st.tab = bofs(s.st.tab, d.ps);
   s.st.ew = bofs(s.st.ew, d.ps);
+  s.st.d1 = s.d1;
   if constexpr (SP) {
     s.luH2 = bofs(s.luH2, d.ps);
     s.luP2 = bofs(s.luP2, d.ps);
@@ -1476,27 +1488,22 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
       const int first = it / kGroups * per, nt = T >= 8 || g < 4 ? first : per == 2 ? first + 1 : tiles;
       const int mi = T >= 8 ? it % kGroups * 8 + g : g & 3, i0 = nt * 8 - s.st.off;
       double2 x[4];
-      StencilPair d9;
+      double2 d9[2];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int i = stencil_row(i0, t, q);
-        x[q] = i >= 0 && i < N ? at(i, mi) : double2{0.0, 0.0};  // (a tile past the last has no rows < N)
+        x[q] = nt < tiles && i >= 0 && i < N ? at(i, mi) : double2{0.0, 0.0};
       }
-      const int* ew = s.st.ew + (parity * tiles + min(nt, tiles - 1)) * 8 + 2 * t;
-      const uint2* tab = s.st.tab + (long)(parity * tiles + first) * kTileB + lane;
-      if constexpr (T >= 8) dft_stencil(x, tab, ew[0] + shift, ew[1] + shift, d9.v);
-      else {
-        const bool two = per == 2 && first + 1 < tiles;
-        if constexpr (CURL)
-          d9 = dft_stencil_call(x[0], x[1], x[2], x[3], tab, two, g >= 4, ew[0] + shift, ew[1] + shift);
-        else
-          dft_stencil_pair(x, tab, two, g >= 4, ew[0] + shift, ew[1] + shift, d9.v);
-      }
+      const StencilAt w = stencil_tile(s.st, parity, first, nt, lane, shift);
+      dft_stencil<(T < 8), CURL>(x, w, per == 2 && first + 1 < tiles, g >= 4, [](const double2 (&)[4]) {}, [&](int i, int c, int part) {
+        const double2 v = at(i, T >= 8 ? mi - g + c : c & 3);
+        return part ? v.y : v.x;
+      }, d9);
       const double ak = d.alpha * (min(kk0 + mi, nk - 1) - (K - 1));
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int i = i0 + 2 * t + q;
-        if (i >= 0 && i < N) out(i, mi, ak, d9.v[q]);
+        if (i >= 0 && i < N) out(i, mi, ak, d9[q]);
       }
     }
   };
@@ -1927,7 +1934,7 @@ void launch_solve(const Dims& d, const DevSetup& s, const SolveArgs& a, int nJ, 
   dim3 g((d.nk + T - 1) / T, d.M, d.B);
   const bool stage = solve_use_stage(d, T, (long)g.x * g.y * g.z, sp);
   SolveDev sd{s.d1,  s.rinv, s.wq,   s.hop,  s.luH,  s.luP,  s.basis, s.ainv, s.G,  s.prm,
-              stencil_at(s.stab, d.N), nJ,    stage ? 1 : 0,  s.luH2, s.luP2, s.spkH,  s.spkP, s.rH, s.rP};
+              stencil_at(s.stab, s.d1, d.N), nJ,    stage ? 1 : 0,  s.luH2, s.luP2, s.spkH,  s.spkP, s.rH, s.rP};
   const size_t sm = stage ? solve_smem_staged(d.N, T, sp) : solve_smem_base(d.N, T, sp);
   if (T == 16) launch_step_kernel(d, k_solve<16>, g, dim3(24 * 16), sm, st, d, sd, a);
   else if (T == 8) launch_step_kernel(d, k_solve<8>, g, dim3(24 * 8), sm, st, d, sd, a);

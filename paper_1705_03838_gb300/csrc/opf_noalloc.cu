@@ -248,7 +248,7 @@ extern "C" int opf_nonlinear_noalloc(int N, int K, int M, int m_p, double alpha,
   // the curl's digit table: behind the other regions, or in the half-physical
   // fields', which are not in use yet, where the scratch ends before
   s.stab = need + opf::stencil_bytes(N) <= kNoallocScratchBytes ? base + need : base + o_Z6;
-  const opf::StencilTable stab = opf::stencil_at(s.stab, N);
+  const opf::StencilTable stab = opf::stencil_at(s.stab, s.d1, N);
   const int nb = (stab.tiles + 1) / 2 + (d.nz + d.nth + kConstThreads - 1) / kConstThreads;
   k_noalloc_consts<<<nb, kConstThreads, 0, st>>>(N, d.nz, d.nth, Re, s.prm, s.d1, s.rinv, s.tw_z, s.tw_th,
                                                  (uint2*)stab.tab, (int*)stab.ew);
