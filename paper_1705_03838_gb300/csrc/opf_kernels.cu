@@ -1137,10 +1137,11 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // The host stages only where that costs no resident blocks (see
 // launch_solve); the launch gives the staged size then, the base size else.
 // sp: the split solve's interface values (6T chains x 8 doubles) after misc.
-// The stencils are digit products (dft_stencil; results do not depend on the
-// tile) and only the wall divergence's weights are kept here, except in the
-// split solve, whose grids of few blocks are better off with multiply-adds.
-__host__ __device__ constexpr int solve_weights(int N, bool sp) { return sp ? 2 * N * 9 : 10; }
+// Where the stencils are digit products only the wall divergence's weights are
+// kept here.
+constexpr int kSolveDigitRows = 64;
+__host__ __device__ constexpr bool solve_by_digits(int N, bool sp) { return !sp && N >= kSolveDigitRows; }
+__host__ __device__ constexpr int solve_weights(int N, bool sp) { return solve_by_digits(N, sp) ? 10 : 2 * N * 9; }
 __host__ __device__ constexpr size_t solve_smem_base(int N, int T, bool sp = false) {
   return (size_t)(2 * N * T + T) * 16 + (size_t)6 * N * T * 8 +
          (size_t)(solve_weights(N, sp) + 3 * N + 2) * 8 + 16 + (sp ? (size_t)48 * T * 8 : 0);
@@ -1285,17 +1286,18 @@ __device__ __forceinline__ void band_solve4(const double* __restrict__ L, double
 // then takes the curl of its new state for the next nonlinear evaluation.
 //
 // The radial derivatives (of N+ + N- and of p) are digit products on the tensor
-// cores (dft_stencil), a warp per eight modes and rows, except in the split
-// solve (on a block per SM its wider block with FP64 multiply-adds and the
-// weights in shared memory is the faster: 28.6 us at N = 32, 31 x 16 modes).
+// cores (dft_stencil), a warp per eight modes and rows, from N = 64 on; on
+// coarser meshes, whose windows reach from the axis or the wall and of whose columns
+// many are steep, and in the split solve (a block per SM), FP64 multiply-adds with
+// the weights in shared memory are the faster.
 // What bounds it: the chains of the substitutions and, on large grids, the
 // FP64 unit, which the stencils took 36 of ~90 instructions per point of.  Per
-// launch against multiply-adds for every column: N = 128, 255 x 128 modes 1743
-// -> 1559 us, groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 193 -> 190
-// us, N = 48, 63 x 24 modes 46.0 -> 45.9 us, 64 x (N = 32, 31 x 16) 411 -> 422 us;
-// N = 41, 53 x 20 modes (two blocks per SM) 35.8 -> 39 us; N = 20, 7 x 5 modes,
-// which takes the curl as well and is latency alone, 24.3 -> 30.5 us -- there
-// the one copy of the code (stencil_call) is 2 us faster than one per use.
+// launch, multiply-adds against digits: N = 128, 255 x 128 modes 1734, 1558 us;
+// 8 x (63 x 32 modes) at N = 96 660, 521 us, 80 486, 452, 64 385, 372, 48 300,
+// 298 us; 63 x 24 modes at N = 96 82.8, 78.4 us, 64 55.2, 58.3, 56 50.1, 54.2; 64
+// x (N = 32, 31 x 16) 410, 422 us; N = 41, 53 x 20 modes 35.7, 39 us; N = 20, 7 x
+// 5 modes, which takes the curl as well (by digits either way, in one copy of
+// the code, stencil_call, 2 us faster than one per use), 28.4, 30.5 us.
 //
 // Resident blocks per SM the register budget must allow (the shared-memory
 // footprints of the tiles allow about as many at moderate N).
@@ -1341,7 +1343,8 @@ __device__ __forceinline__ void spike_fix(int tid, int N, int nch, int st, doubl
 // chain's substitution runs on 8 lanes, the two halves of its rows at once
 // (twice the threads; the other phases use them too).
 // CURL: may take the curl of its new state (a.W6).
-template <int T, bool SP = false, bool CURL = SP>
+// DIG: the stencils by digit products (solve_by_digits).
+template <int T, bool DIG, bool SP = false, bool CURL = SP>
 __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     k_solve(Dims d, SolveDev s, SolveArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1404,10 +1407,9 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   const double ci = s.prm[kPrmCi], cu = s.prm[kPrmCu];  // 1 / (c dt), (1 - c) / c
   const long fs = d.F;
   const long base = (long)m * N * nk;
-  constexpr bool kDigits = !SP;
   const double* wv = W1 + pv * N * 9;  // stencils of u_r, u_theta parity
   const double* ws = W1 + ps * N * 9;  // stencils of u_z, p parity
-  const double* wall = kDigits ? W1 : wv + (N - 1) * 9;  // wall row of wv
+  const double* wall = DIG ? W1 : wv + (N - 1) * 9;  // wall row of wv
   // chain c -> (field f, mode mi, part); element (f, row i, mode mi) of a field
   auto uj = [&](int f, int i, int mi) {
     return a.Uj[f * fs + base + (long)i * nk + min(kk0 + mi, nk - 1)];
@@ -1431,14 +1433,14 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   }
 
   // The stencils by asynchronous copies, waited for at the first barrier.
-  if constexpr (kDigits) {
+  if constexpr (DIG) {
     if (tid < 9) cp_async8(W1 + tid, s.d1 + ((long)pv * N + N - 1) * 9 + tid);
-    if (CURL && a.W6)  // a block per SM: the digit tables to the SM's cache while it waits for its input
-      for (int e = tid; e < 2 * s.st.tiles * (kTileB / 16); e += NB)
-        asm volatile("{\n.reg .b32 t;\nld.global.ca.b32 t, [%0];\n}" ::"l"(s.st.tab + 16 * e));
   } else {
     for (int e = tid; e < 2 * N * 9; e += NB) cp_async8(W1 + e, s.d1 + e);
   }
+  if (CURL && !SP && a.W6)  // a block per SM: the digit tables to the SM's cache while it waits for its input
+    for (int e = tid; e < 2 * s.st.tiles * (kTileB / 16); e += NB)
+      asm volatile("{\n.reg .b32 t;\nld.global.ca.b32 t, [%0];\n}" ::"l"(s.st.tab + 16 * e));
   cp_async_commit();
 
   // ---- N_eff = N_a (predictor) or (N_a + N_b) / 2 (corrector, c = 1/2), and
@@ -1509,7 +1511,7 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
   };
 
   // ---- pressure right-hand side: div N_eff (rows < N-1), 0 at the wall
-  if constexpr (kDigits) {
+  if constexpr (DIG) {
     for_stencil_items([&](int i, int mi) { return S[i * T + mi]; }, pv, -1, [&](int i, int mi, double ak, double2 dr) {  // dr: half the derivative
       const double2 np = ne_at(0, i, mi), nm = ne_at(1, i, mi), nz = ne_at(2, i, mi);
       const double bx = dr.x + fma(RIp[i], np.x, fma(RIm[i], nm.x, -ak * nz.y));
@@ -1603,7 +1605,7 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
     xr[c2] = fma(ak, pp.y, xr[c2]);
     xr[c2 + 1] = fma(-ak, pp.x, xr[c2 + 1]);
   };
-  if constexpr (kDigits) {
+  if constexpr (DIG) {
     for_stencil_items([&](int i, int mi) { return P[i * T + mi]; }, ps, 0, [&](int i, int mi, double ak, double2 dp) {
       if (i < N - 1) subtract_gradient(i, mi, ak, dp);
     });
@@ -1746,7 +1748,7 @@ __global__ void __launch_bounds__((SP ? 48 : 24) * T, solve_min_blocks<T, SP>())
       W[4 * fs] = double2{fma(-ak, ur.y, -dz.x), fma(ak, ur.x, -dz.y)};
       W[5 * fs] = double2{fma(mri, ur.y, fma(ri, ut.x, dt.x)), fma(-mri, ur.x, fma(ri, ut.y, dt.y))};
     };
-    if constexpr (kDigits) {  // (a row and mode belong to the same lane in both passes)
+    if constexpr (!SP) {  // (a row and mode belong to the same lane in both passes)
       for_stencil_items([&](int i, int mi) { return P[i * T + mi]; }, pv, 0,
                         [&](int i, int mi, double, double2 dt) { S[i * T + mi] = dt; });
       for_stencil_items([&](int i, int mi) { return *(const double2*)(X + i * NT + ((2 * T + mi) << 1)); }, ps, 0,
@@ -1876,11 +1878,16 @@ bool prepare_kernel_attrs(const Dims& d) {
     constexpr int L = decltype(n)::value;
     ok = ok && cudaFuncSetAttribute(k_product<float2, L>, a, optin) == cudaSuccess;
   });
-  ok = ok && cudaFuncSetAttribute(k_solve<16>, a, optin) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(k_solve<8>, a, optin) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(k_solve<4>, a, optin) == cudaSuccess;
+  auto solves = [&](auto dig) {
+    constexpr bool D = decltype(dig)::value;
+    ok = ok && cudaFuncSetAttribute(k_solve<16, D>, a, optin) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(k_solve<8, D>, a, optin) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(k_solve<4, D>, a, optin) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(k_solve<4, D, false, true>, a, optin) == cudaSuccess;
+  };
+  if (solve_by_digits(d.N, false)) solves(std::true_type{});
+  else solves(std::false_type{});
   ok = ok && cudaFuncSetAttribute(k_solve<4, false, true>, a, optin) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(k_solve<4, true>, a, optin) == cudaSuccess;
   auto fusable = [](int n) { return n == 48 || n == 72 || n == 96; };
   if (fusable(d.nz) && fusable(d.nth))  // (the option or the autotuner may switch the fused launch on later)
     with_fused_lengths(d.nz, d.nth, [&](auto z, auto t) {
@@ -1936,11 +1943,16 @@ void launch_solve(const Dims& d, const DevSetup& s, const SolveArgs& a, int nJ, 
   SolveDev sd{s.d1,  s.rinv, s.wq,   s.hop,  s.luH,  s.luP,  s.basis, s.ainv, s.G,  s.prm,
               stencil_at(s.stab, s.d1, d.N), nJ,    stage ? 1 : 0,  s.luH2, s.luP2, s.spkH,  s.spkP, s.rH, s.rP};
   const size_t sm = stage ? solve_smem_staged(d.N, T, sp) : solve_smem_base(d.N, T, sp);
-  if (T == 16) launch_step_kernel(d, k_solve<16>, g, dim3(24 * 16), sm, st, d, sd, a);
-  else if (T == 8) launch_step_kernel(d, k_solve<8>, g, dim3(24 * 8), sm, st, d, sd, a);
-  else if (sp) launch_step_kernel(d, k_solve<4, true>, g, dim3(48 * 4), sm, st, d, sd, a);
-  else if (a.W6) launch_step_kernel(d, k_solve<4, false, true>, g, dim3(24 * 4), sm, st, d, sd, a);
-  else launch_step_kernel(d, k_solve<4>, g, dim3(24 * 4), sm, st, d, sd, a);
+  if (sp) return launch_step_kernel(d, k_solve<4, false, true>, g, dim3(48 * 4), sm, st, d, sd, a);
+  auto go = [&](auto dig) {
+    constexpr bool D = decltype(dig)::value;
+    if (T == 16) launch_step_kernel(d, k_solve<16, D>, g, dim3(24 * 16), sm, st, d, sd, a);
+    else if (T == 8) launch_step_kernel(d, k_solve<8, D>, g, dim3(24 * 8), sm, st, d, sd, a);
+    else if (a.W6) launch_step_kernel(d, k_solve<4, D, false, true>, g, dim3(24 * 4), sm, st, d, sd, a);
+    else launch_step_kernel(d, k_solve<4, D>, g, dim3(24 * 4), sm, st, d, sd, a);
+  };
+  if (solve_by_digits(d.N, false)) go(std::true_type{});
+  else go(std::false_type{});
 }
 
 // ------------------------------------------------------------------ diagnostics
