@@ -312,7 +312,7 @@ __device__ __forceinline__ void dft_put(uint4* tile, int lane, const long long (
 // 16) of the columns' windows take multiply-adds, in a quarter to three fifths
 // of the warps; the other rows' derivatives cost no FP64 instruction.  Per
 // launch, digits alone -> with the choice: split curl, N = 128: 242 -> 267 us,
-// N = 48, 63 x 24 modes 12.6 -> 16.9 us; solve 1545 -> 1559 and 42.8 -> 45.9 us.
+// N = 48, 63 x 24 modes 12.6 -> 15.9 us; solve 1545 -> 1559 and 42.8 -> 45.9 us.
 struct StencilAt {      // one lane's share of a tile
   const uint2* tab;      // the tile's table plus lane
   const double* d1;      // the parity's weights, [N][9]
@@ -382,17 +382,15 @@ __device__ __forceinline__ unsigned stencil_steep(const double2 (&x)[4], const S
   return cols;
 }
 
-// The derivative of these columns by multiply-adds in the type of V, from the
-// lowest row up, into out of the lanes whose column it is.  Two columns at a
-// time, a lane per row and part: a warp's FP64 instruction takes its time
-// whatever the lanes in use, and often few of the eight columns are steep (a
-// lane doing its own two rows, for all columns of the warp: solve at N = 128
+// The derivative of these columns by multiply-adds, from the lowest row up, into
+// out of the lanes whose column it is.  Two columns at a time, a lane per row
+// and part: a warp's FP64 instruction takes its time whatever the lanes in use,
+// and often few of the eight columns are steep (a lane doing its own two rows, for all columns of the warp: solve at N = 128
 // 1682 us instead of 1564, curl 314 instead of 277; taking the steep rows alone,
 // the digits for the rest: the same on the whole).
 // at(row, g, part): column g's value.
-template <typename V, typename At>
-__device__ __forceinline__ void stencil_fma(unsigned cols, const StencilAt& s, At at, V (&out)[2]) {
-  using T = decltype(V{}.x);
+template <typename At>
+__device__ __forceinline__ void stencil_fma(unsigned cols, const StencilAt& s, At at, double2 (&out)[2]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, part = (lane >> 3) & 1;
 #pragma unroll 1
   while (cols) {
@@ -401,23 +399,23 @@ __device__ __forceinline__ void stencil_fma(unsigned cols, const StencilAt& s, A
     const int c1 = cols ? (__ffs(cols) - 1) >> 2 : c0;
     cols &= cols - 1;
     const int c = lane < 16 ? c0 : c1, i = __shfl_sync(0xffffffffu, s.i0, 4 * c) + (lane & 7);
-    T sum = 0;
+    double sum = 0.0;
     if (i >= 0 && i < s.N) {
       const int lo = min(max(i - 4, 0), s.N - 9);
-      T v[9], w[9];
+      double v[9], w[9];
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
         const bool in = lo + k <= i + 4;  // (the axis rows' weights beyond are zero, and past the window)
-        w[k] = in ? (T)__ldg(s.d1 + i * 9 + k) : (T)0;
-        v[k] = in ? (T)at(lo + k, c, part) : (T)0;
+        w[k] = in ? __ldg(s.d1 + i * 9 + k) : 0.0;
+        v[k] = in ? at(lo + k, c, part) : 0.0;
       }
 #pragma unroll
       for (int k = 0; k < 9; ++k) sum = fma(w[k], v[k], sum);
       if (s.shift) sum = halved(sum);
     }
     const int src = (g == c0 ? 0 : 16) + 2 * t;
-    const V a = V{__shfl_sync(0xffffffffu, sum, src), __shfl_sync(0xffffffffu, sum, src + 8)};
-    const V b = V{__shfl_sync(0xffffffffu, sum, src + 1), __shfl_sync(0xffffffffu, sum, src + 9)};
+    const double2 a = double2{__shfl_sync(0xffffffffu, sum, src), __shfl_sync(0xffffffffu, sum, src + 8)};
+    const double2 b = double2{__shfl_sync(0xffffffffu, sum, src + 1), __shfl_sync(0xffffffffu, sum, src + 9)};
     if (g == c0 || g == c1) {
       out[0] = a;
       out[1] = b;
@@ -579,11 +577,18 @@ __device__ __forceinline__ void dft_stencil32(const double2 (&x)[4], const Stenc
   bool all, row[2];
   const unsigned cols = stencil_steep<kNearBits32, false>(x, w, s.i0, s.N, &all, row);
   if (cols) {
-    float2 y[2];
+    double2 y[2] = {double2{0.0, 0.0}, double2{0.0, 0.0}};
     put(x);
-    stencil_fma(cols, s, at, y);
-    if (row[0]) out[0] = y[0];
-    if (row[1]) out[1] = y[1];
+    stencil_fma(cols, s, at, y);  // (in FP64: converting the data takes its unit longer)
+    bool rare = false;
+    float2 f[2] = {float2{to_float(y[0].x, &rare), to_float(y[0].y, &rare)},
+                   float2{to_float(y[1].x, &rare), to_float(y[1].y, &rare)}};
+    if (rare) {
+      f[0] = float2{(float)y[0].x, (float)y[0].y};
+      f[1] = float2{(float)y[1].x, (float)y[1].y};
+    }
+    if (row[0]) out[0] = f[0];
+    if (row[1]) out[1] = f[1];
   }
 }
 #endif  // __CUDACC__

@@ -141,8 +141,8 @@ void launch_internal_to_abi(const Dims& d, const double2* U, double2* abi, int, 
 // as FP64 multiply-adds on columns staged in shared memory (whose loads of data
 // and weights took about as long), split curl per launch: N = 128, 255 x 128
 // modes 440 -> 267 us, groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32)
-// 57 -> 45 us, N = 48, 63 x 24 modes, less than two waves of warps of which
-// some take multiply-adds as well, 14.8 -> 16.9 us.
+// 57 -> 44 us, N = 48, 63 x 24 modes, less than two waves of warps of which
+// some take multiply-adds as well, 14.8 -> 15.9 us.
 constexpr int kCurlWarps = 4;
 
 // The (0,0) mode of the split curl: the base flow is taken off u_z and w_theta.

@@ -75,7 +75,6 @@ __device__ __forceinline__ double halved(double x) {
   const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
   return e - 2u < 0x7fdu ? __hiloint2double(hi - 0x100000, __double2loint(x)) : 0.5 * x;
 }
-__device__ __forceinline__ float halved(float x) { return 0.5f * x; }
 
 // Batched launches: trajectory b = blockIdx.z; its buffers sit `stride` bytes
 // after trajectory b-1's (stride 0: shared).  Null stays null.
