@@ -304,6 +304,24 @@ static unsigned transform_threads(const dim3& g) {
   return (long)g.x * g.y * g.z <= 4L * device_sms() ? 256u : 128u;
 }
 
+// The FP32 kernels that stream (a compiled plan) do with fewer, at every
+// length: their composite butterflies take up to 164 registers a thread, and
+// what counts is how many small blocks reside.  z synthesis and product: 96
+// threads, us per launch against 64, 128 and 192 (z synthesis | product): N =
+// 128, 384 x 384 points 113, 121, 123, 172 | 354, 360, 415, 536; 4 x (N = 64, 192 x
+// 192) 58, 62, 60, 70 | 153, 143, 157, 228; 16 x (N = 48, 96 x 96) 47, 45, 50, 64 |
+// 96, 100, 105, 127; 16 x (N = 48, 72 x 72) 32, 31, 35, 44 | 62, 66, 70, 86; 64 x
+// (N = 32, 48 x 48) 36, 32, 41, 49 | 72, 81, 80, 106; a single N = 48, 96 x 72
+// 8.2 | 12.1, the others up to 0.1 and 1.1 more.
+constexpr unsigned kStreamThreads = 96;
+// z analysis, whose block takes three components and reads the addends: a
+// thread for nine of its points, at least 128, at most 192.  Those grids at 128
+// and 192: 226, 178; 101, 90; 80, 70; 47, 45; 49, 57 (8 columns of 48 points,
+// 1152); 11.2, 11.2 us.
+static unsigned zanalysis_threads(int nz, int mca) {
+  return (unsigned)std::min(192, std::max(128, mca * nz / 3 / 32 * 32));
+}
+
 // ------------------------------------------------------------------ z synthesis (A2)
 
 // NZ > 0: the z length 3K is the compile-time constant NZ (compiled plan).
@@ -382,10 +400,8 @@ void launch_zsynth32(const Dims& d, const DevSetup& s, const FftPlan& pz, const 
   with_fft_length(d.nz, [&](auto n) {
     const size_t sm = decltype(n)::value ? (size_t)(d.mcz * (d.nz + 1) + d.nz) * sizeof(float2)
                                          : zsynth_smem(d, d.mcz, sizeof(float2));
-    // (length 384: its 128 and 192 butterflies in two rounds of 96 each, 124 -> 113 us
-    // at N = 128, 255 x 128 modes; for shorter lengths it changed no step)
     launch_step_kernel(d, k_zsynth<float2, decltype(n)::value>, g,
-                       dim3(decltype(n)::value == 384 ? 96u : transform_threads(g)), sm, st, d, pz,
+                       dim3(decltype(n)::value ? kStreamThreads : transform_threads(g)), sm, st, d, pz,
                        (const float2*)s.tw_z32, W6, Z6);
   });
 }
@@ -640,11 +656,9 @@ void launch_product32(const Dims& d, const DevSetup& s, const FftPlan& pth, cons
   with_fft_length(d.nth, [&](auto n) {
     const size_t sm = decltype(n)::value ? (size_t)(3 * d.zc + 1) * d.nth * sizeof(float2)
                                          : product_smem(d, d.zc, sizeof(float2));
-    // (length 384: the 96 threads that its middle phase has work for at 4 rows --
-    // 363 us at N = 128, 255 x 128 modes, with 128 435 us, with 192 587 us)
     const unsigned items = ((unsigned)product32_items(d, d.zc) + 31) / 32 * 32;
     launch_step_kernel(d, k_product<float2, decltype(n)::value>, g,
-                       dim3(std::max(items, decltype(n)::value == 384 ? 96u : transform_threads(g))), sm, st, d, pth,
+                       dim3(decltype(n)::value ? std::max(items, kStreamThreads) : transform_threads(g)), sm, st, d, pth,
                        (const float2*)s.tw_th32, Z6, ZN);
   });
 }
@@ -807,10 +821,8 @@ void launch_zanalysis32(const Dims& d, const DevSetup& s, const FftPlan& pz, con
   dim3 g((d.M + d.mca - 1) / d.mca, d.N, d.B);
   const size_t sm = zanalysis_smem(d, d.mca, sizeof(float2));
   with_fft_length(d.nz, [&](auto n) {
-    // (length 384: its 576 and 384 butterflies in 3 and 2 rounds of 192, 226 -> 178 us
-    // at N = 128, 255 x 128 modes; 256 threads 192 us, 96 237 us)
     launch_step_kernel(d, k_zanalysis<float2, decltype(n)::value>, g,
-                       dim3(decltype(n)::value == 384 ? 192u : transform_threads(g)), sm, st, d, pz,
+                       dim3(decltype(n)::value ? zanalysis_threads(d.nz, d.mca) : transform_threads(g)), sm, st, d, pz,
                        (const float2*)s.tw_z32, ZN, Nlin, Nout);
   });
 }
