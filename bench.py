@@ -57,33 +57,51 @@ def config_dict(w, precision):
 
 
 # ------------------------------------------------------------------ algorithmic costs
-def kernel_costs(w, precision=1):
-    """Algorithmic flops and bytes per launch, per kernel.
+SOLVE_DIGIT_ROWS = 64  # from this N on the solve's stencils are digit products
+DIGIT_LENGTH = 96      # as are the FP64 transforms up to this length
+
+
+def kernel_costs(w, precision=1, curl_in_solve=False, split=False):
+    """Flops on the unit that kernel_peak names, and algorithmic bytes, per
+    launch, per kernel.  What is done by digit products on the tensor cores is
+    not counted: the curl's stencils (72 of 102 per point; the multiply-adds of
+    steep columns, which depend on the state, neither), the solve's (72 of 150
+    per row) from N = 64 on except in the split solve, and the FP64 transforms
+    up to length 96, of which the pointwise product is left.
 
     FFT flops use 2.5 n log2 n per real 2-D transform of n = 9KM points,
     split between z (log2 3K) and theta (log2 3M) parts.  The solve counts,
-    per mode and radial row: div N_eff (48), d_r p (36), right-hand sides (30),
-    final update and influence correction (36), and 8 real banded
-    substitutions (2 nl + 2 nu + 1 each, nl/nu the row's band widths).  The
-    stencils (48 + 36, and 72 per point of the curl) are digit products on the
-    tensor cores; they are counted as the operations they stand for."""
+    per mode and radial row: div N_eff (48, of which stencils 36), d_r p (36),
+    right-hand sides (30), final update and influence correction (36), and 8
+    real banded substitutions (2 nl + 2 nu + 1 each, nl/nu the row's band
+    widths).  curl_in_solve: no curl is launched, the solve takes it as well
+    (with its stencils as multiply-adds in the split solve)."""
     N, K, M = w["N"], w["K"], w["M"]
     nz, nth, nk = 3 * K, 3 * M, 2 * K - 1
     n = nz * nth
     F = N * nk * M  # complex per spectral field
     P = N * nz * M  # complex per half-physical field
-    lz, lt = math.log2(nz), math.log2(nth)
+    lz, lt = (0.0 if precision == 0 and length <= DIGIT_LENGTH else math.log2(length) for length in (nz, nth))
     lo = [min(max(i - 4, 0), N - 9) for i in range(N)]
     band = sum(2 * (i - lo[i]) + 2 * (min(i + 4, N - 1) - i) + 1 for i in range(N))
     modes = nk * M
-    solve = modes * (N * (48 + 36 + 30 + 36) + 8 * band)
+    stencils = 0 if N >= SOLVE_DIGIT_ROWS and not split else 72
+    solve = modes * (N * (12 + stencils + 30 + 36) + 8 * band)
+    if curl_in_solve:
+        solve += F * (30 + (72 if split else 0))
     return {
-        "curl": {"flops": F * (2 * 9 * 4 + 30), "bytes": 16 * (3 * F + 6 * F)},
+        "curl": {"flops": F * 30, "bytes": 16 * (3 * F + 6 * F)},
         "zsynth": {"flops": 6 * N * 2.5 * n * lz, "bytes": 16 * (6 * F + 6 * P)},
         "product": {"flops": 9 * N * 2.5 * n * lt + 9 * N * n, "bytes": 16 * (6 * P + 3 * P)},
         "zanalysis": {"flops": 3 * N * 2.5 * n * lz, "bytes": 16 * (3 * P + 3 * F)},
-        "solve": {"flops": solve, "bytes": 16 * (3 * F * 3 + 3 * F)},
+        "solve": {"flops": solve, "bytes": 16 * (3 * F * 3 + 3 * F + (6 * F if curl_in_solve else 0))},
     }
+
+
+def launches_per_step(kernel_times, steps):
+    """Kernel launches of one step, from the per-kernel counts of `steps` timed
+    ones: {name: (total ms, launches)} as opf_kernel_times gives them."""
+    return sum(n for _, n in kernel_times.values()) // steps
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the current
@@ -414,7 +432,7 @@ def run_ensemble(args):
     algo_bytes = (528 if args.precision == 0 else 432) * Fsum
     flops = {}
     for (N, K, M), cnt in ((sh, shapes.count(sh)) for sh in dict.fromkeys(shapes)):
-        c = kernel_costs({"N": N, "K": K, "M": M})
+        c = kernel_costs({"N": N, "K": K, "M": M}, args.precision)
         for k, v in c.items():
             flops[k] = flops.get(k, 0.0) + cnt * v["flops"]
     dom = max(kt, key=lambda k: kt[k][0])
@@ -834,6 +852,8 @@ def run_gpu(args, w):
 
     names = ["curl", "zsynth", "product", "zanalysis", "solve"]
 
+    launches, curl_in_solve = {}, {}
+
     def timed(precision):
         """K steps at one precision from U0; per-step CUDA events, L2 flushed
         between, the step graph free of any inner event record.  A few
@@ -849,10 +869,13 @@ def run_gpu(args, w):
         opf.opf_set_state(h, U0)
         opf.opf_set_option(h, "timing", 1)
         opf.opf_kernel_times(h, reset=True)
-        for _ in range(max(3, args.warmup)):
+        timed_steps = max(3, args.warmup)
+        for _ in range(timed_steps):
             flush_l2()
             opf.opf_step(h, 1)
         kt_all = opf.opf_kernel_times(h, reset=True)
+        launches[precision] = launches_per_step(kt_all, timed_steps)
+        curl_in_solve[precision] = not kt_all.get("curl", (0.0, 0))[1]
         dom = max(kt_all, key=lambda k: kt_all[k][0])
         opf.opf_set_option(h, "timing", 0)
         opf.opf_step(h, 1)  # capture the plain step graph outside the timed region
@@ -934,7 +957,7 @@ def run_gpu(args, w):
     value = job_rate(args.steps, world, total_ms / 1000.0)
     peaks, peak_kind = load_peaks()
     def roofline(kt, precision):
-        costs = kernel_costs(w, precision)
+        costs = kernel_costs(w, precision, curl_in_solve[precision], opf.opf_get_option(h, "spike") != 0)
         dom = max(kt, key=lambda k: kt[k][0])
         dom_ms = kt[dom][0] / max(1, kt[dom][1])
         pk, src = kernel_peak(dom, precision)
@@ -966,8 +989,6 @@ def run_gpu(args, w):
                "small_workload_100_steps": {"seconds": small["seconds"], "cores": 1,
                                             "timesteps_per_s": 100.0 / small["seconds"]},
                "large_workload": LARGE_ORACLE_NOTE}
-    # per pass: curl + 3 transform kernels + solve
-    launches_per_step = 5 * 2
     line = {
         "metric": METRIC,
         "value": value,
@@ -1000,7 +1021,7 @@ def run_gpu(args, w):
                 "h2d_bytes_per_step": int(U0.nbytes), "d2h_bytes_per_step": int(U0.nbytes),
                 "per_step": "set_state from pinned host memory, one step, get_state (the new state) to "
                             "pinned host memory", "state_finite": e2e_state_ok},
-        "gpu_launches": launches_per_step * args.steps,
+        "gpu_launches": launches[args.precision] * args.steps,
         "clocks": clk,
         "wall_s_timed_region": wall,
         "energy_EID": [float(x) for x in E],

@@ -189,7 +189,11 @@ int opf_set_stream(opf_t* h, void* stream);
 
 /* Per-kernel device time of the steps run since the last call with reset=1:
  * names[i] (library-owned) and total_ms[i], launches[i] for i < *count
- * (capacity cap).  Collected only while option "timing" = 1. */
+ * (capacity cap).  Collected only while option "timing" = 1.  Where the solve
+ * launches take the curl of their output (FP64 steps with 4-mode tiles and no
+ * more of their blocks than SMs) the curl's own kernel runs only when a step
+ * starts after the state, the work buffers or an option changed, and is not
+ * timed then: "curl" reports no launches there. */
 int opf_kernel_times(opf_t* h, int cap, int* count, const char** names,
                      double* total_ms, int* launches, int reset);
 
