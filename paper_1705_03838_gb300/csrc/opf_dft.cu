@@ -171,11 +171,31 @@ size_t dft_zsynth_smem(const Dims& d) {
   return (size_t)synth_shape(d).R * 2 * dft_tiles(d.K, 16) * kTileA * sizeof(uint4);
 }
 
+// A block's results as plain sums (dft_outside), here and for the kernels
+// below: functions of their own, which leave the code around them as it is.
+static __device__ __noinline__ void zsynth_sums(int t0, int RT, int K, int M, int N, const double2* __restrict__ tw,
+                                                const double2* __restrict__ W6, double2* Z6) {
+  const int nz = 3 * K, nk = 2 * K - 1, MT = (M + 7) / 8;
+  for (int e = threadIdx.x; e < RT * 8 * nz; e += blockDim.x) {
+    const int p = e / 8 % nz, r = t0 + e / (8 * nz), fn = r / MT, f = fn / N, m = (r - fn * MT) * 8 + e % 8;
+    if (m >= M) continue;
+    const double2* x = W6 + ((long)(f * M + m) * N + fn - f * N) * nk + K - 1;
+    double2 sum = double2{0.0, 0.0};
+#pragma unroll 1
+    for (int k = 1 - K; k < K; ++k) {
+      const double2 w = tw[(k + nz) * p % nz];
+      sum.x = fma(x[k].x, w.x, fma(-x[k].y, w.y, sum.x));
+      sum.y = fma(x[k].x, w.y, fma(x[k].y, w.x, sum.y));
+    }
+    Z6[((long)fn * nz + p) * M + m] = sum;
+  }
+}
+
 __global__ void __launch_bounds__(kThreads, 2)
     k_dft_zsynth(Dims d, int R, const uint2* __restrict__ Tc, const uint2* __restrict__ Ts,
-                 const double2* __restrict__ W6, double2* __restrict__ Z6) {
+                 const double2* __restrict__ tw, const double2* __restrict__ W6, double2* __restrict__ Z6) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ int emx[kWarps][8];
+  __shared__ int emx[kWarps][8], outside;
   const int K = d.K, M = d.M, N = d.N, nk = d.nk, nz = d.nz;
   const int MT = (M + 7) / 8, t0 = blockIdx.x * R, RT = min(R, 6 * N * MT - t0);
   const int KT = dft_tiles(K, 16), P = dft_points(nz), NT = dft_tiles(P, 8);
@@ -185,6 +205,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   Z6 = bofs(Z6, d.ss);
   grid_dep_trigger_at(d, 1);
   if (threadIdx.x < kWarps * 8) emx[threadIdx.x >> 3][threadIdx.x & 7] = 0;
+  if (threadIdx.x == 0) outside = 0;
   double2 xp[4], xm[4];  // X_k, X_-k
   const int rt = warp / KT, kt = warp - rt * KT;  // KT <= 2: one item per warp
   const bool have = rt < RT;
@@ -211,6 +232,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __syncthreads();
   if (have) {
     const int e = emx[rt][g];
+    if (dft_outside(e)) outside = 1;
     long long sr[4], si[4], dr[4], di[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -247,6 +269,10 @@ __global__ void __launch_bounds__(kThreads, 2)
         dst[(long)(nz - p) * M] = double2{dft_plus(c[q], s[2 + q], sc), dft_minus(c[2 + q], s[q], sc)};
     }
   }
+  if (outside) {
+    __syncthreads();
+    zsynth_sums(t0, RT, K, M, N, bofs(tw, d.ps), W6, Z6);
+  }
 }
 
 // ------------------------------------------------------------------ theta transforms and product
@@ -279,6 +305,35 @@ __host__ __device__ inline ProductShape product_shape(int M, int nth, int fields
 }
 }  // namespace
 
+static __device__ __noinline__ void theta_sums(int z0, int nz, int n, int N, int M, int nth, int ldq,
+                                               const double2* __restrict__ tw, const double2* __restrict__ Z6,
+                                               double* ph) {
+  for (int e = threadIdx.x; e < 6 * 16 * nth; e += blockDim.x) {
+    const int q = e % nth, r = e / nth, z = z0 + (r & 15);
+    if (z >= nz) continue;
+    const double2* x = Z6 + (((long)(r >> 4) * N + n) * nz + z) * M;
+    double sum = 0.0;
+#pragma unroll 1
+    for (int m = 1; m < M; ++m) sum = fma(x[m].x, tw[m * q % nth].x, fma(-x[m].y, tw[m * q % nth].y, sum));
+    ph[r * ldq + q] = fma(2.0, sum, x[0].x);
+  }
+}
+static __device__ __noinline__ void theta_back_sums(int z0, int nz, int n, int N, int M, int nth, int ldq,
+                                                    const double2* __restrict__ tw, const double* ph, double2* ZN) {
+  for (int e = threadIdx.x; e < 3 * 16 * M; e += blockDim.x) {
+    const int m = e % M, r = e / M, z = z0 + (r & 15);
+    if (z >= nz) continue;
+    double2 sum = double2{0.0, 0.0};
+#pragma unroll 1
+    for (int q = 0; q < nth; ++q) {
+      const double f = ph[r * ldq + q];
+      sum.x = fma(f, tw[m * q % nth].x, sum.x);
+      sum.y = fma(-f, tw[m * q % nth].y, sum.y);
+    }
+    ZN[(((long)(r >> 4) * N + n) * nz + z) * M + m] = sum;
+  }
+}
+
 // FIELDS per round.  16 warps and all six where there are no more blocks than
 // SMs.  Else 8 warps, two blocks per SM: with one k tile per row (M <= 16) and
 // its small footprint all six fields at once, 6 digit tiles and 24 products for
@@ -291,7 +346,7 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
                   double2* __restrict__ ZN) {
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int kFields = FIELDS;
-  __shared__ int emx[kFields][16], emn[3][16];
+  __shared__ int emx[kFields][16], emn[3][16], outside[2];  // (of the six fields; of the products)
   const int M = d.M, N = d.N, nz = d.nz, nth = d.nth;
   const ProductShape ps = product_shape(M, nth, FIELDS);
   const int ldq = ps.ldq, KT = ps.KT, KT2 = ps.KT2, P = dft_points(nth);
@@ -305,6 +360,7 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
   ZN = bofs(ZN, d.ss);
   const long fstride = (long)N * nz * M;
   grid_dep_trigger_at(d, 1);
+  if (threadIdx.x < 2) outside[threadIdx.x] = 0;
   grid_dep_wait();
   for (int round = 0; round < 6 / kFields; ++round) {
     if (threadIdx.x < kFields * 16) emx[threadIdx.x >> 4][threadIdx.x & 15] = 0;
@@ -338,6 +394,7 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
     __syncthreads();
     if (have) {
       const int ex = emx[fi][g], ey = emx[fi][g + 8];
+      if (dft_outside(ex) || dft_outside(ey)) outside[0] = 1;
       long long xr[4], xi[4], yr[4], yi[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -372,6 +429,10 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
         }
       }
     }
+    __syncthreads();
+  }
+  if (outside[0]) {
+    theta_sums(z0, nz, n, N, M, nth, ldq, tw, Z6, ph);
     __syncthreads();
   }
   // ---- u x omega (with the Coriolis force and the CFL number), one warp per row
@@ -436,6 +497,7 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = g + 8 * h, e = emn[c][r];
+      if (dft_outside(e)) outside[1] = 1;
       const double* row = ph + (c * 16 + r) * ldq;
       const bool in = z0 + r < nz;
 #pragma unroll
@@ -477,6 +539,10 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
       }
     }
   }
+  if (outside[1]) {  // (the products' rows lie below their digits)
+    __syncthreads();
+    theta_back_sums(z0, nz, n, N, M, nth, ldq, tw, ph, ZN);
+  }
 }
 
 // ------------------------------------------------------------------ z analysis
@@ -488,6 +554,25 @@ size_t dft_zanalysis_smem(const Dims& d) {
   return std::max(a, (size_t)24 * d.nk * sizeof(double2));
 }
 
+static __device__ __noinline__ void zanalysis_sums(int m0, int n, int K, int M, int N, double scale,
+                                                   const double2* __restrict__ tw, const double2* __restrict__ ZN,
+                                                   double2* R) {
+  const int nz = 3 * K, nk = 2 * K - 1;
+  for (int e = threadIdx.x; e < 24 * nk; e += blockDim.x) {
+    const int r = e / nk, m = m0 + (r & 7), h = e - r * nk - (K - 1) + nz;  // harmonic k + nz
+    if (m >= M) continue;
+    const double2* x = ZN + ((long)(r >> 3) * N + n) * nz * M + m;
+    double2 sum = double2{0.0, 0.0};
+#pragma unroll 1
+    for (int p = 0; p < nz; ++p) {
+      const double2 v = x[(long)p * M], w = tw[h * p % nz];
+      sum.x = fma(v.x, w.x, fma(v.y, w.y, sum.x));
+      sum.y = fma(v.y, w.x, fma(-v.x, w.y, sum.y));
+    }
+    R[e] = double2{sum.x * scale, sum.y * scale};
+  }
+}
+
 // WARPS: its 3, 6, 9 or 12 digit tiles and as many products or fewer take
 // multiples of three; six, with a third block per SM where the digits fit, were
 // 106 -> 86 us against eight on 64 x (N = 32, 31 x 16 modes), and twelve where
@@ -496,9 +581,9 @@ size_t dft_zanalysis_smem(const Dims& d) {
 template <int WARPS, int BLOCKS>
 __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
     k_dft_zanalysis(Dims d, int zshift, const uint2* __restrict__ Tc, const uint2* __restrict__ Ts,
-                    const double2* __restrict__ ZN, double2* __restrict__ Nout) {
+                    const double2* __restrict__ tw, const double2* __restrict__ ZN, double2* __restrict__ Nout) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ int emx[3][8];
+  __shared__ int emx[3][8], outside;
   const int K = d.K, M = d.M, N = d.N, nk = d.nk, nz = d.nz;
   const int KT = dft_tiles(dft_points(nz), 16), NT = dft_tiles(K, 8), P = dft_points(nz);
   const int m0 = blockIdx.x * 8, n = blockIdx.y;
@@ -511,6 +596,7 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
   const long fs = d.F, fstride = (long)N * nz * M;
   grid_dep_trigger_at(d, 1);
   if (threadIdx.x < 24) emx[threadIdx.x >> 3][threadIdx.x & 7] = 0;
+  if (threadIdx.x == 0) outside = 0;
   __syncthreads();
   grid_dep_wait();
   constexpr int kItems = (12 + WARPS - 1) / WARPS;  // 3 KT <= 12 items
@@ -544,6 +630,7 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
     const int it = warp + u * WARPS;
     if (it < 3 * KT) {
       const int f = it / KT, kt = it - f * KT, e = emx[f][g];
+      if (dft_outside(e)) outside = 1;
       long long sr[4], si[4], dr[4], di[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -599,6 +686,10 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
     }
   }
   __syncthreads();
+  if (outside) {
+    zanalysis_sums(m0, n, K, M, N, d.inv_grid, bofs(tw, d.ps), ZN, R);
+    __syncthreads();
+  }
   grid_dep_trigger_at(d, 2);
   const int mcn = min(8, M - m0);
   for (int e = threadIdx.x; e < mcn * nk; e += WARPS * 32) {
@@ -644,7 +735,7 @@ bool dft_prepare_attrs() {
 void launch_dft_zsynth(const Dims& d, const DevSetup& s, const double2* W6, double2* Z6, cudaStream_t st) {
   const SynthShape sh = synth_shape(d);
   launch_step_kernel(d, k_dft_zsynth, dim3(sh.blocks, 1, d.B), dim3(kThreads), dft_zsynth_smem(d), st, d, sh.R,
-                     s.dft.m[0], s.dft.m[1], W6, Z6);
+                     s.dft.m[0], s.dft.m[1], (const double2*)s.tw_z, W6, Z6);
 }
 void launch_dft_product(const Dims& d, const DevSetup& s, const double2* Z6, double2* ZN, cudaStream_t st) {
   const dim3 g((d.nz + 15) / 16, d.N, d.B);
@@ -660,7 +751,7 @@ void launch_dft_zanalysis(const Dims& d, const DevSetup& s, const double2* ZN, d
   const dim3 g((d.M + 7) / 8, d.N, d.B);
   auto go = [&](auto kern, int warps) {
     launch_step_kernel(d, kern, g, dim3(warps * 32), dft_zanalysis_smem(d), st, d, s.dft.zshift, s.dft.m[6],
-                       s.dft.m[7], ZN, Nout);
+                       s.dft.m[7], (const double2*)s.tw_z, ZN, Nout);
   };
   if ((long)g.x * g.y * g.z > device_sms()) go(k_dft_zanalysis<6, 3>, 6);
   else if (3 * dft_tiles(dft_points(d.nz), 16) > 8) go(k_dft_zanalysis<12, 1>, 12);
