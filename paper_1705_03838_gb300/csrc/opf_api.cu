@@ -244,7 +244,6 @@ int group_fill_setups(Group* g, bool first) {
     double prm[opf::kPrmCount] = {0};
     prm[opf::kPrmRe] = s.Re;
     prm[opf::kPrmDt] = s.dt;
-    prm[opf::kPrmC] = s.c;
     prm[opf::kPrmSumWG] = s.flux_G;
     prm[opf::kPrmCi] = 1.0 / (s.c * s.dt);  // the solve's scalings, divided here once
     prm[opf::kPrmCu] = (1.0 - s.c) / s.c;
@@ -311,7 +310,6 @@ int group_build(Group* g, int N, int K, int M, int m_p, double alpha, int B, con
   d.alpha = alpha;
   d.Re = Re[0];
   d.dt = dt[0];
-  d.c = 0.5;
   d.F = (long)M * N * d.nk;
   d.B = B;
   opf::choose_chunks(&d);

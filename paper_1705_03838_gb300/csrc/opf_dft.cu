@@ -338,7 +338,8 @@ static __device__ __noinline__ void theta_back_sums(int z0, int nz, int n, int N
 // SMs.  Else 8 warps, two blocks per SM: with one k tile per row (M <= 16) and
 // its small footprint all six fields at once, 6 digit tiles and 24 products for
 // the 8 warps where two rounds of 3 and 12 left warps waiting (64 x (N = 32,
-// 31 x 16 modes) 409 -> 352 us; six warps in three blocks 379 us); else three.
+// 31 x 16 modes) 409 -> 352 us; six warps in three blocks 379 us); else three
+// (M = 30 and 32: 120 and 123 KB of shared memory, so that one block resides).
 template <int WARPS, int FIELDS, int BLOCKS>
 __global__ void __launch_bounds__(WARPS * 32, BLOCKS)
     k_dft_product(Dims d, const uint2* __restrict__ Sc, const uint2* __restrict__ Ss, const uint2* __restrict__ Ac,

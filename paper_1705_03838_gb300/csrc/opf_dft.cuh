@@ -16,12 +16,15 @@
 // spectra of every slope, and within its error where one term outweighs the
 // rest; whole steps are as far from 64-bit references as with it.  FP64
 // kernels against these, per launch (z synthesis, theta product, z analysis):
-// N = 48, 96 x 72: 33, 82, 26 -> 20, 40, 18 us; 64 x (N = 32, 48 x 48): 321,
-// 956, 199 -> 184, 412, 106 us; N = 32, 48 x 48: 13, 25, 13 -> 10, 21, 11 us.
+// N = 48, 96 x 72: 33, 82, 26 -> 20, 39, 17 us; 64 x (N = 32, 48 x 48): 321,
+// 956, 199 -> 142, 357, 86 us; N = 32, 48 x 48: 13, 25, 13 -> 10, 21, 11 us.
 // What bounds them now is the latency of their phases at 16 warps per SM: the
 // tensor pipe is a third to two thirds busy in the products, the integer
-// units in the splitting and joining.  The work grows with the square of the
-// length, the FFT's does not: lengths above 96 stay with it.
+// units in the splitting and joining.  Lengths above 96 stay with the FFT: the
+// kernels give each warp one digit tile of a row's at most 32 harmonics, and
+// the bound on a level's sums has been worked out up to there.  (The work grows
+// with the square of the length, the FFT's does not; at 96 these are 1.6 times
+// as fast in z, and where the two cross has not been measured.)
 // Symmetry halves the work: with c, s the cosine and sine sums over
 // harmonics h (or points p), a result at p and its mirror n - p are c + s and
 // c - s (up to factors i).

@@ -36,8 +36,6 @@ __device__ __forceinline__ V cmadd(T f, V a, V b) { return V{madd(f, a.x, b.x), 
 // multiply by s*i (s = +-1)
 template <typename V>
 __device__ __forceinline__ V cmul_si(V a, int s) { return s > 0 ? V{-a.y, a.x} : V{a.y, -a.x}; }
-template <typename V, typename T>
-__device__ __forceinline__ V cscale(V a, T f) { return V{a.x * f, a.y * f}; }
 
 // In-place DFT of size R on v[0..R-1] with kernel e^{sign 2 pi i tq/R}.
 // Radix 8 with v[3] = v[4] = 0 (the first stage of a synthesis whose middle
@@ -398,11 +396,11 @@ __device__ __forceinline__ V* block_fft_c(V* a, V* b, int batch, int ld, const V
     constexpr FftRadices r = fft_radices32(N);
     if constexpr (SIGN > 0) return fft_stages_c<N, 1, SIGN, ZERO_MID, r.r1, r.r2>(a, b, ld, batch, tw);
     else return fft_stages_c<N, 1, SIGN, ZERO_MID, r.r2, r.r1>(a, b, ld, batch, tw);
-  } else if constexpr (N == 48) return fft_stages_c<48, 1, SIGN, ZERO_MID, 4, 4, 3>(a, b, ld, batch, tw);
-  else if constexpr (N == 72) return fft_stages_c<72, 1, SIGN, ZERO_MID, 8, 3, 3>(a, b, ld, batch, tw);
-  else if constexpr (N == 96) return fft_stages_c<96, 1, SIGN, ZERO_MID, 8, 4, 3>(a, b, ld, batch, tw);
-  else if constexpr (N == 192) return fft_stages_c<192, 1, SIGN, ZERO_MID, 8, 8, 3>(a, b, ld, batch, tw);
-  else return fft_stages_c<384, 1, SIGN, ZERO_MID, 8, 4, 4, 3>(a, b, ld, batch, tw);
+  } else {  // (FP64 lengths up to 96 are digit products)
+    static_assert(N == 192 || N == 384, "no compiled FP64 plan for this length");
+    if constexpr (N == 192) return fft_stages_c<192, 1, SIGN, ZERO_MID, 8, 8, 3>(a, b, ld, batch, tw);
+    else return fft_stages_c<384, 1, SIGN, ZERO_MID, 8, 4, 4, 3>(a, b, ld, batch, tw);
+  }
 }
 
 // Calls f(std::integral_constant<int, n>) for a compiled length n, else

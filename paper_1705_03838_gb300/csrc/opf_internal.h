@@ -55,7 +55,7 @@ bool build_setup(Setup* s, std::string* err);
 
 // --------------------------------------------------------------- device side
 // Per-trajectory scalars at the head of each trajectory's setup arrays.
-constexpr int kPrmRe = 0, kPrmDt = 1, kPrmC = 2, kPrmSumWG = 3, kPrmCi = 4, kPrmCu = 5, kPrmCount = 8;
+constexpr int kPrmRe = 0, kPrmDt = 1, kPrmSumWG = 3, kPrmCi = 4, kPrmCu = 5, kPrmCount = 8;
 
 // Digit tables of the FP64 transforms on the tensor cores (opf_dft.cuh): z
 // synthesis, theta synthesis, theta analysis, z analysis, each cosine then
@@ -71,7 +71,7 @@ __host__ __device__ constexpr int basis_ld(int N) { return (3 * N + 1) & ~1; }
 
 struct DevSetup {
   DftTables dft;
-  double* prm = nullptr;  // [kPrmCount] Re, dt, c, sum(wq G)
+  double* prm = nullptr;  // [kPrmCount] Re, dt, sum(wq G), 1 / (c dt), (1 - c) / c
   double* rinv = nullptr;
   double* d1 = nullptr;
   double* wq = nullptr;
@@ -98,7 +98,7 @@ struct DevSetup {
 struct Dims {
   int N, K, M, m_p, nk, nz, nth;
   double inv_grid;  // 1 / (nz nth): scaling of the forward transforms
-  double alpha, Re, dt, c;  // host copies (trajectory 0); kernels read DevSetup::prm
+  double alpha, Re, dt;  // host copies (trajectory 0); kernels read DevSetup::prm
   long F;         // complex values per spectral field = M * N * nk
   int mcz, mca;   // m columns per block: z synthesis, z analysis
   int zc;         // z rows per block in the theta/product kernel

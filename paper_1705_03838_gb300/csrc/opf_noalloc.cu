@@ -170,7 +170,6 @@ extern "C" int opf_nonlinear_noalloc(int N, int K, int M, int m_p, double alpha,
   d.alpha = alpha;
   d.Re = Re;
   d.dt = 1.0;
-  d.c = 0.5;
   d.F = (long)M * N * d.nk;
   opf::choose_chunks(&d);
   opf::FftPlan pz{}, pth{};
