@@ -328,8 +328,8 @@ static unsigned zanalysis_threads(int nz, int mca) {
 // FP32 with a compiled plan: both passes work between registers, global memory
 // and one exchange through shared memory, whose pipe was 88 % busy with the
 // staging and every pass; half the footprint lets twice the blocks reside.
-// 197 -> 113 us at N = 128, 255 x 128 modes (500 MB, 75 us at the copy rate),
-// groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 28.7 -> 19.6 us.
+// 197 -> 114 us at N = 128, 255 x 128 modes (500 MB, 75 us at the copy rate),
+// groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 28.7 -> 18.1 us.
 template <typename V, int NZ>
 __global__ void __launch_bounds__(256) k_zsynth(Dims d, FftPlan pz, const V* __restrict__ twz,
                                                 const V* __restrict__ W6, V* __restrict__ Z6) {
@@ -429,8 +429,8 @@ __device__ __forceinline__ void sincos_pi(float x, float* s, float* c) { sincosp
 // analyses on the same points in registers; the last pass to global memory.
 // What bounds it: barriers between the phases and instruction fetch, at 12 warps
 // per SM (length 384).  N = 128,
-// 255 x 128 modes 467 -> 363 us; groups of 8 x (N = 32 .. 48) and 6 x (N = 64,
-// 63 x 32) 44.6 -> 36.3 us; N = 48, 63 x 24 modes 13.2 -> 12.6 us.
+// 255 x 128 modes 467 -> 362 us; groups of 8 x (N = 32 .. 48) and 6 x (N = 64,
+// 63 x 32) 44.6 -> 34.3 us; N = 48, 63 x 24 modes 13.2 -> 12.1 us.
 template <typename V, int NTH>
 __global__ void __launch_bounds__(256) k_product(Dims d, FftPlan pth, const V* __restrict__ twth,
                                                  const V* __restrict__ Z6, V* __restrict__ ZN) {
@@ -679,9 +679,9 @@ __device__ __forceinline__ double wide(double x) { return x; }
 __device__ __forceinline__ double wide(float x) { return to_double(x); }
 
 // FP32 with a compiled plan: the first pass reads global memory itself.  N = 128,
-// 255 x 128 modes 256 -> 178 us (with the threads of its launch rule),
-// groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 40.3 -> 30.3 us, N = 48,
-// 63 x 24 modes 12.3 -> 11.0 us.
+// 255 x 128 modes 256 -> 179 us (with the threads of its launch rule),
+// groups of 8 x (N = 32 .. 48) and 6 x (N = 64, 63 x 32) 40.3 -> 29.2 us, N = 48,
+// 63 x 24 modes 12.3 -> 11.3 us.
 template <typename V, int NZ>
 __global__ void __launch_bounds__(256) k_zanalysis(Dims d, FftPlan pz, const V* __restrict__ twz,
                                                    const V* __restrict__ ZN, const double2* __restrict__ Nlin,
@@ -1294,7 +1294,7 @@ __device__ __forceinline__ void band_solve4(const double* __restrict__ L, double
 // 0 solves the pressure system the other warps assemble the p-independent part
 // of the velocity right-hand sides (and stage u_j and the influence
 // responses); the last pass applies u_j, the influence correction and the
-// flux correction on the way out to global memory, and with a.curl the block
+// flux correction on the way out to global memory, and with a.W6 the block
 // then takes the curl of its new state for the next nonlinear evaluation.
 //
 // The radial derivatives (of N+ + N- and of p) are digit products on the tensor
